@@ -358,19 +358,6 @@ __global__ void __launch_bounds__(256) k_spmm_out(int32_t n_items, const Item *_
     }
 }
 
-// scalar transpose aggregation: ds[u] += sum over out-edges of q da[w]; a thread per node
-__global__ void k_spmm_out_scalar(int32_t n, const int32_t *__restrict__ row_ptr, const uint2 *__restrict__ ic_edge,
-                                  const float *__restrict__ da, float *__restrict__ ds) {
-    for (int32_t u = blockIdx.x * blockDim.x + threadIdx.x; u < n; u += gridDim.x * blockDim.x) {
-        float s = 0.0f;
-        for (int32_t e = row_ptr[u]; e < row_ptr[u + 1]; ++e) {
-            const uint2 ed = ic_edge[e];
-            s += edge_q(ed.y) * da[ed.x];
-        }
-        ds[u] += s;
-    }
-}
-
 // --------------------------------------------------------------------------- dense layers
 // Per warp a 16-row tile; lane = 4 g + t (g = lane / 4 row group, t = lane % 4).
 template <int DIN>
@@ -766,24 +753,69 @@ __global__ void k_sum_parts(int32_t nblocks, const double *__restrict__ part, do
     *out = sum;
 }
 
-__global__ void k_scores(int32_t n, const float *__restrict__ o, const __nv_bfloat16 *__restrict__ x,
-                         const float *__restrict__ ds0, float *__restrict__ score) {
-    for (int32_t v = blockIdx.x * blockDim.x + threadIdx.x; v < n; v += gridDim.x * blockDim.x) {
-        const float s = __bfloat162float(x[(size_t)v * D0]);
-        score[v] = (1.0f - s) * (1.0f - sigmoidf_(o[v])) + ds0[v];
+// Scores of candidate c from the scalar sum over its out-edges (c -> w), T_c:
+//   MODE 0 (screening):  T = sum of q da0[w],       (1 - s)(1 - sigmoid(o)) + ds0[c] + T
+//   MODE 1 (one-hop):    T = sum of q (1 - yhat[w]), (1 - yhat_c) (1 + T)
+template <int MODE>
+__device__ __forceinline__ float out_score(int32_t c, float T, const float *__restrict__ o,
+                                           const __nv_bfloat16 *__restrict__ x, const float *__restrict__ ds0,
+                                           const float *__restrict__ yhat) {
+    if (MODE == 1) return (1.0f - yhat[c]) * (1.0f + T);
+    const float s = __bfloat162float(x[(size_t)c * D0]);
+    return (1.0f - s) * (1.0f - sigmoidf_(o[c])) + (ds0[c] + T);
+}
+
+// Scores of all nodes: 8 lanes per work item of <= 256 out-edges.  The sum is one float per edge at a
+// random node, so it is bound by how many such loads are in flight; a thread per node (the form
+// before) left the whole sum of a hub's out-row to one thread's chain of loads.  8 lanes rather than a
+// warp because most rows are shorter than 32 edges.  R-MAT-17 (1.94 M edges, GB300): 862 -> 23 us.
+// Items of a split row write their partial sum to scratch[slot]; k_out_scores_split adds them.
+template <int MODE>
+__global__ void __launch_bounds__(256) k_out_scores(int32_t n_items, const Item *__restrict__ items,
+                                                    const uint2 *__restrict__ ic_edge, const float *__restrict__ val,
+                                                    const float *__restrict__ o, const __nv_bfloat16 *__restrict__ x,
+                                                    const float *__restrict__ ds0, float *__restrict__ scratch,
+                                                    float *__restrict__ score) {
+    const int sub = threadIdx.x & 7;
+    const int group = (blockIdx.x * blockDim.x + threadIdx.x) >> 3;
+    const int ngroups = (gridDim.x * blockDim.x) >> 3;
+    const int rounds = (n_items + ngroups - 1) / ngroups;  // the same for every lane of a warp
+    for (int r = 0; r < rounds; ++r) {
+        const int it = r * ngroups + group;
+        Item item{0, 0, 0, -1};
+        if (it < n_items) item = items[it];
+        float s = 0.0f;
+#pragma unroll 4
+        for (int32_t e = item.begin + sub; e < item.end; e += 8) {
+            const uint2 ed = ic_edge[e];
+            s += edge_q(ed.y) * (MODE == 0 ? val[ed.x] : 1.0f - val[ed.x]);
+        }
+        __syncwarp();
+#pragma unroll
+        for (int d = 4; d; d >>= 1) s += __shfl_xor_sync(0xffffffffu, s, d);
+        if (sub == 0 && it < n_items) {
+            if (item.slot < 0) score[item.node] = out_score<MODE>(item.node, s, o, x, ds0, val);
+            else scratch[item.slot] = s;
+        }
     }
 }
 
-// (1 - yhat_c) (1 + sum over out-edges of q (1 - yhat_w)); a thread per node
-__global__ void k_onehop(int32_t n, const int32_t *__restrict__ row_ptr, const uint2 *__restrict__ ic_edge,
-                         const float *__restrict__ yhat, float *__restrict__ score) {
-    for (int32_t c = blockIdx.x * blockDim.x + threadIdx.x; c < n; c += gridDim.x * blockDim.x) {
-        float s = 1.0f;
-        for (int32_t e = row_ptr[c]; e < row_ptr[c + 1]; ++e) {
-            const uint2 ed = ic_edge[e];
-            s += edge_q(ed.y) * (1.0f - yhat[ed.x]);
-        }
-        score[c] = (1.0f - yhat[c]) * s;
+// scores of the nodes whose out-row is split over several items: a warp per node, the partial sums
+// added in a fixed order
+template <int MODE>
+__global__ void k_out_scores_split(int32_t n_split, const int32_t *__restrict__ split_node,
+                                   const int32_t *__restrict__ first, const float *__restrict__ scratch,
+                                   const float *__restrict__ val, const float *__restrict__ o,
+                                   const __nv_bfloat16 *__restrict__ x, const float *__restrict__ ds0,
+                                   float *__restrict__ score) {
+    const int lane = threadIdx.x & 31;
+    const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int nwarps = (gridDim.x * blockDim.x) >> 5;
+    for (int i = warp; i < n_split; i += nwarps) {
+        float s = 0.0f;
+        for (int32_t j = first[i] + lane; j < first[i + 1]; j += 32) s += scratch[j];
+        for (int d = 16; d; d >>= 1) s += __shfl_xor_sync(0xffffffffu, s, d);
+        if (lane == 0) score[split_node[i]] = out_score<MODE>(split_node[i], s, o, x, ds0, val);
     }
 }
 
@@ -967,6 +999,16 @@ void aggregate_out(cnd_sur *s, const float *da, float *dh, cudaStream_t st) {
     if (s->n_split_out)
         k_split_out_finish<<<grid_for((int64_t)s->n_split_out * 32, 256, s->num_sms), 256, 0, st>>>(
             s->n_split_out, s->split_out_node, s->split_out_first, s->scratch_out, dh);
+}
+
+// scores of all nodes from the sums over their out-edges (k_out_scores)
+template <int MODE>
+void out_scores(cnd_sur *s, const float *val, float *score, cudaStream_t st) {
+    k_out_scores<MODE><<<grid_for((int64_t)s->n_items_out * 8, 256, s->num_sms), 256, 0, st>>>(
+        s->n_items_out, s->items_out, s->g->d.ic_edge, val, s->o, s->x, s->ds0, s->scratch_out, score);
+    if (s->n_split_out)
+        k_out_scores_split<MODE><<<grid_for((int64_t)s->n_split_out * 32, 256, s->num_sms), 256, 0, st>>>(
+            s->n_split_out, s->split_out_node, s->split_out_first, s->scratch_out, val, s->o, s->x, s->ds0, score);
 }
 
 // the predicted spread (sum of yhat) into *spread, summed in a fixed order
@@ -1293,9 +1335,7 @@ cnd_status cnd_sur_scores(cnd_sur *s, const int32_t *seeds, int32_t n_seeds, flo
     aggregate_out(s, s->da, s->dhB, cs);
     k_dense_bwd<D0, 0, 2, false><<<tb, 128, 0, cs>>>(n, s->h[0], s->dhB, none, s->wt, 0, s->p, nullptr, s->ds0,
                                                      s->da0, nullptr);
-    const cnd_graph_dev &G = s->g->d;
-    k_spmm_out_scalar<<<grid_for(n, 256, s->num_sms), 256, 0, cs>>>(n, G.row_ptr, G.ic_edge, s->da0, s->ds0);
-    k_scores<<<grid_for(n, 256, s->num_sms), 256, 0, cs>>>(n, s->o, s->x, s->ds0, s->yv);
+    out_scores<0>(s, s->da0, s->yv, cs);
     seed_clear(s, s->seeds, ns, cs);
     CND_CUDA_TRY(cudaGetLastError());
     CND_CUDA_TRY(cudaMemcpyAsync(score_out, s->yv, sizeof(float) * n, cudaMemcpyDeviceToHost, cs));
@@ -1320,8 +1360,7 @@ cnd_status cnd_sur_onehop(cnd_sur *s, const int32_t *seeds, int32_t n_seeds, flo
     seed_set(s, s->seeds, ns, cs);
     forward(s, cs);
     spread_sum(s, s->dsum, cs);
-    const cnd_graph_dev &G = s->g->d;
-    k_onehop<<<grid_for(n, 256, s->num_sms), 256, 0, cs>>>(n, G.row_ptr, G.ic_edge, s->yv, s->ds0);
+    out_scores<1>(s, s->yv, s->ds0, cs);
     seed_clear(s, s->seeds, ns, cs);
     CND_CUDA_TRY(cudaGetLastError());
     CND_CUDA_TRY(cudaMemcpyAsync(score_out, s->ds0, sizeof(float) * n, cudaMemcpyDeviceToHost, cs));
