@@ -1,0 +1,589 @@
+// Column engine: IC, and LT in the counting form, on graphs whose state of up to 32 trials fits the
+// shared memory of one SM.
+//
+// Trials never interact, so a block takes a column of up to 32 consecutive trials of one item through
+// all of its steps by itself: the state of every node in those trials is one 32-bit word per array, in
+// shared memory, a step ends with one block barrier, and the whole call is one launch.  The pass engine
+// (cnd_sim.cu) pays launches, counter copies and a host round trip for every step, about 40 us on a
+// 1,000-node graph whose steps hold a few hundred edges each, and its batches run as many steps as
+// their deepest item.
+//
+//   vis[v]      trials in which v is active
+//   nx[v]       trials activated in the current step
+//   lists       the frontier's nodes and bits and the nodes of the next one; the first `cap` entries in
+//               shared memory, the others in global memory (so that 8 bytes per node, not 16, decide how
+//               many columns an SM holds: steps are latency-bound and want several)
+//   planes      LT: 32-lane bit-sliced in-neighbour counters, L_v words per node (see k_lt_init in
+//               cnd_sim.cu for why the carry out of the top plane is the activation)
+//
+// A warp takes up to 32 frontier nodes, spreads their out-edges over its lanes (a warp-wide or of the
+// rows' first positions gives each lane the node of its edge), and IC draws the coins of the (edge,
+// 4-trial block) pairs that need one: in place where no lane needs more than one, else from a per-warp
+// queue.  Rows of kHub edges and more are left to the whole block after the others.
+//
+// Columns are handed out by an atomic counter, since their depths differ.  What bounds a step is the
+// latency of its chain (row offsets, edges, target, coins, three shared-memory atomics, two barriers)
+// where its frontier is small, and issue slots where it is large (62 % issue active, ncu, on a dense
+// Watts-Strogatz 10k).  Against the pass engine's host step loop (GB300): G(1000, 10000), p = 0.1, 1,000
+// trials 1,710 -> 165 us per call, Watts-Strogatz 10k U[0, 1] 2,300 -> 650 us, CELF k = 10 on the
+// 7-regular graph (n = 5,000) 149 -> 21.8 ms.
+#include <cuda_runtime.h>
+
+#include <algorithm>
+#include <cmath>
+
+#include "cnd_cols.cuh"
+
+namespace cnd {
+namespace {
+
+constexpr int kHub = 256;       // out-edges from which the whole block expands a node
+constexpr int kHubCap = 64;     // hubs set aside per step (more are expanded by the warp that finds them)
+constexpr int kColMaxN = 65535; // node ids are kept in 16 bits
+
+struct ColItem {
+    int64_t out0;     // position of the item's first trial in the spread output
+    uint64_t key;
+    int32_t s_begin, s_end;
+    int32_t trials;
+    int32_t col0;     // its first column
+};
+
+struct ColParams {
+    int32_t n, n_items;
+    int32_t bits;             // trials per column (a multiple of 4, at most 32)
+    int32_t n_cols;
+    int32_t cap;              // list entries kept in shared memory
+    uint16_t *over_node;      // [blocks][2][n] list entries beyond cap
+    uint32_t *over_bits;      // [blocks][n]
+    const int32_t *row_ptr;
+    const uint2 *edge;        // {col, IC threshold} or {col, counter tag}
+    const ColItem *items;
+    const int32_t *seeds;
+    const int32_t *cnt_off;   // LT: first plane of each node
+    const uint32_t *unit_w;
+    int64_t first_trial;
+    int32_t *spread, *count;
+    unsigned long long *checks, *level_counts;
+    int32_t lc_len, max_levels;
+    unsigned long long timeout_ns;
+    int32_t *next;            // column counter
+    CallFlags *flags;
+};
+
+struct __align__(16) WarpQueue {
+    uint4 task[32];    // {edge, threshold, target, wanted trials} of each lane
+    uint8_t q[256];    // (lane << 3) | 4-trial block
+};
+
+// The warp's frontier nodes that have edges to expand, in order: {edge id of the warp's t-th edge
+// less t, frontier bits}.
+struct __align__(8) WarpNodes {
+    uint2 node[32];
+};
+
+struct BlockState {
+    int32_t n_list[3];   // frontier sizes, by step mod 3
+    int32_t n_hub[3];
+    int32_t col, item;
+    int32_t stop;        // first step not to run (set by the time limit)
+    uint32_t spread[32];
+    uint2 hub[kHubCap];  // {node, frontier bits}
+    __align__(16) uint32_t rk[20];
+};
+
+__device__ __forceinline__ unsigned long long timer_ns() {
+    unsigned long long t;
+    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+    return t;
+}
+
+// 32 x 32 bit transpose over a warp: bit i of lane b's result is bit b of lane i's x.
+__device__ __forceinline__ uint32_t transpose32(uint32_t x) {
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int s = 16; s; s >>= 1) {
+        const uint32_t m = s == 16 ? 0x0000FFFFu : s == 8 ? 0x00FF00FFu : s == 4 ? 0x0F0F0F0Fu : s == 2 ? 0x33333333u : 0x55555555u;
+        const uint32_t y = __shfl_xor_sync(kFull, x, s);
+        x = (lane & s) ? ((x & ~m) | ((y & ~m) >> s)) : ((x & m) | ((y & m) << s));
+    }
+    return x;
+}
+
+// The parts of a step that its edges need.
+struct StepCtx {
+    uint32_t *vis, *nx;
+    uint16_t *lnext, *gnext;  // the next frontier's nodes: entries below cap, and beyond
+    int32_t *n_next;
+    int32_t cap;
+    uint32_t *planes;
+    const uint2 *edge;
+    const uint32_t *rk;
+    uint64_t g0;
+    uint32_t gained;  // activations of this thread in the step
+
+    // v becomes active in the trials of `bits` where it is not yet
+    __device__ __forceinline__ void activate(uint32_t v, uint32_t bits) {
+        const uint32_t nw = bits & ~atomicOr(&vis[v], bits);
+        if (nw) {
+            gained += __popc(nw);
+            if (atomicOr(&nx[v], nw) == 0u) {
+                const int i = atomicAdd(n_next, 1);
+                (i < cap ? lnext : gnext)[i] = (uint16_t)v;
+            }
+        }
+    }
+};
+
+// One IC draw: the coins of edge e in the 4-trial block g, as 4 bits.
+__device__ __forceinline__ uint32_t coins(const StepCtx &s, uint32_t e, uint32_t thr, uint32_t j) {
+    const uint64_t g = s.g0 + j;
+    uint32_t c0 = e, c1 = (uint32_t)g, c2 = 0u, c3 = (uint32_t)(g >> 32);
+#pragma unroll
+    for (int h = 0; h < 5; ++h) {
+        const uint4 k = reinterpret_cast<const uint4 *>(s.rk)[h];
+        const uint32_t kk[4] = {k.x, k.y, k.z, k.w};
+#pragma unroll
+        for (int r = 0; r < 4; r += 2) {
+            const uint64_t a = (uint64_t)0xD2511F53u * c0;
+            const uint64_t b = (uint64_t)0xCD9E8D57u * c2;
+            c0 = (uint32_t)(b >> 32) ^ c1 ^ kk[r];
+            c2 = (uint32_t)(a >> 32) ^ c3 ^ kk[r + 1];
+            c1 = (uint32_t)b;
+            c3 = (uint32_t)a;
+        }
+    }
+    return (uint32_t)(c0 < thr) | ((uint32_t)(c1 < thr) << 1) | ((uint32_t)(c2 < thr) << 2) | ((uint32_t)(c3 < thr) << 3);
+}
+
+// Expand one edge per lane, {v, thr} = ed, by the frontier bits f (0: nothing to do in this lane).
+template <int MODEL>
+__device__ __forceinline__ void expand(StepCtx &s, WarpQueue &wq, uint32_t e, uint2 ed, uint32_t f) {
+    const int lane = threadIdx.x & 31;
+    const uint32_t v = ed.x, thr = ed.y;
+    uint32_t c = 0;
+    if (f && thr != 0u) c = f & ~*(volatile uint32_t *)&s.vis[v];
+    if (MODEL == 1) {
+        if (c) {  // one bit-sliced increment of v's counter by the trials of c
+            const uint32_t L = thr & 31u;
+            uint32_t *pl = s.planes + (thr >> 5);
+            for (uint32_t i = 0; i < L && c; ++i) c &= atomicXor(pl + i, c);
+            if (c) s.activate(v, c);
+        }
+        return;
+    }
+    if (c && thr == kAlways) {
+        s.activate(v, c);
+        c = 0;
+    }
+    uint32_t nm = c | (c >> 1);
+    nm = (nm | (nm >> 2)) & 0x11111111u;  // the 4-trial blocks to draw
+    const uint32_t d = __popc(nm);
+    if (!__any_sync(kFull, d > 1u)) {
+        // at most one block per lane: each lane draws its own
+        if (d) {
+            const uint32_t j = (uint32_t)(__ffs(nm) - 1) >> 2;
+            const uint32_t live = (coins(s, e, thr, j) << (4 * j)) & c;
+            if (live) s.activate(v, live);
+        }
+        return;
+    }
+    // queue the blocks: positions from the ballots of the bits of d (0 .. 8)
+    const uint32_t lt = (1u << lane) - 1u;
+    uint32_t D = 0, r = 0;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const uint32_t b = __ballot_sync(kFull, (d >> k) & 1u);
+        D += (uint32_t)__popc(b) << k;
+        r += (uint32_t)__popc(b & lt) << k;
+    }
+    wq.task[lane] = make_uint4(e, thr, v, c);
+    while (nm) {
+        const int b = __ffs(nm) - 1;
+        nm &= nm - 1;
+        wq.q[r++] = (uint8_t)((lane << 3) | (b >> 2));
+    }
+    __syncwarp();
+    for (uint32_t i = lane; i < D; i += 32) {
+        const uint32_t ent = wq.q[i];
+        const uint4 t = wq.task[ent >> 3];
+        const uint32_t j = ent & 7u;
+        const uint32_t live = (coins(s, t.x, t.y, j) << (4 * j)) & t.w;
+        if (live) s.activate(t.z, live);
+    }
+    __syncwarp();
+}
+
+template <int MODEL>
+__global__ void __launch_bounds__(1024, 1) k_columns(ColParams p) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ BlockState S;
+    const int n = p.n, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const int n_warps = blockDim.x >> 5;
+    WarpQueue *queues = reinterpret_cast<WarpQueue *>(smem);
+    const int n4 = (n + 3) & ~3;
+    WarpNodes *wnodes = reinterpret_cast<WarpNodes *>(smem + (MODEL == 0 ? sizeof(WarpQueue) * n_warps : 0));
+    uint32_t *vis = reinterpret_cast<uint32_t *>(wnodes + n_warps);
+    uint32_t *nx = vis + n4, *lbits = nx + n4;
+    const int cap = p.cap;  // a multiple of 8
+    uint16_t *la = reinterpret_cast<uint16_t *>(lbits + cap), *lb = la + cap;
+    uint32_t *planes = reinterpret_cast<uint32_t *>(lb + cap);
+    uint16_t *const ga = p.over_node + (size_t)blockIdx.x * 2 * n, *const gb = ga + n;
+    uint32_t *const gbits = p.over_bits + (size_t)blockIdx.x * n;
+    WarpQueue &wq = queues[MODEL == 0 ? wid : 0];
+    uint2 *wn = wnodes[wid].node;
+    const uint32_t lt = (1u << lane) - 1u, le = lt | (1u << lane);
+    unsigned long long ck = 0;
+    for (;;) {
+        if (tid == 0) S.col = atomicAdd(p.next, 1);
+        __syncthreads();
+        const int col = S.col;
+        if (col >= p.n_cols) break;
+        // ---- clear the state; warp 0 finds the column's item (the last one with col0 <= col)
+        for (int i = tid; i < 2 * (n4 >> 2); i += blockDim.x)
+            reinterpret_cast<uint4 *>(vis)[i] = make_uint4(0u, 0u, 0u, 0u);
+        if (tid < 32) {
+            int lo = 0, hi = p.n_items;  // item in [lo, hi)
+            while (hi - lo > 1) {
+                const int step = (hi - lo + 31) / 32;
+                const int probe = lo + lane * step;
+                const unsigned ok = __ballot_sync(kFull, probe < hi && p.items[probe].col0 <= col);
+                lo += (31 - __clz(ok)) * step;
+                hi = min(hi, lo + step);
+            }
+            if (lane == 0) {
+                S.item = lo;
+                S.stop = 0x7FFFFFFF;
+                S.n_list[0] = S.n_list[1] = S.n_list[2] = 0;
+                S.n_hub[0] = S.n_hub[1] = S.n_hub[2] = 0;
+                uint32_t k0 = (uint32_t)p.items[lo].key, k1 = (uint32_t)(p.items[lo].key >> 32);
+                for (int r = 0; r < 10; ++r) {
+                    S.rk[2 * r] = k0;
+                    S.rk[2 * r + 1] = k1;
+                    k0 += 0x9E3779B9u;
+                    k1 += 0xBB67AE85u;
+                }
+            }
+            S.spread[lane] = 0u;
+        }
+        __syncthreads();
+        const ColItem it = p.items[S.item];
+        const int t0 = (col - it.col0) * p.bits;  // first trial of the column within the item
+        const int nt = min(p.bits, it.trials - t0);
+        const uint32_t valid = nt >= 32 ? 0xFFFFFFFFu : ((1u << nt) - 1u);
+        const uint64_t g0 = (uint64_t)(p.first_trial + t0) >> 2;
+        if (MODEL == 1) {
+            // counter starts c0 = 2^L - 1 - floor(theta / w) (0 when negative), a thread per node
+            for (int v = tid; v < n; v += blockDim.x) {
+                const int o0 = p.cnt_off[v];
+                const int L = p.cnt_off[v + 1] - o0;
+                if (L == 0) continue;
+                const uint32_t wv = p.unit_w[v];
+                const uint32_t top = L >= 32 ? 0xFFFFFFFFu : ((1u << L) - 1u);
+                for (int i = 0; i < L; ++i) planes[o0 + i] = 0u;
+                for (int j = 0; 4 * j < nt; ++j) {
+                    const uint64_t g = g0 + (uint64_t)j;
+                    const U4 th = philox4x32_10((uint32_t)v, (uint32_t)g, 1u, (uint32_t)(g >> 32), (uint32_t)it.key,
+                                                (uint32_t)(it.key >> 32));
+                    const uint32_t tv[4] = {th.x, th.y, th.z, th.w};
+                    uint32_t c0[4];
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        const uint32_t q = tv[k] / wv;
+                        c0[k] = q < top ? top - q : 0u;
+                    }
+                    for (int i = 0; i < L; ++i) {
+                        const uint32_t nib = ((c0[0] >> i) & 1u) | (((c0[1] >> i) & 1u) << 1) |
+                                             (((c0[2] >> i) & 1u) << 2) | (((c0[3] >> i) & 1u) << 3);
+                        planes[o0 + i] |= nib << (4 * j);
+                    }
+                }
+            }
+        }
+        // ---- step 0: the seeds (duplicates count once)
+        for (int i = it.s_begin + tid; i < it.s_end; i += blockDim.x) {
+            const int u = p.seeds[i];
+            if (u < 0 || u >= n) {
+                p.flags->bad_seed = 1;
+                continue;
+            }
+            if (atomicOr(&vis[u], valid) == 0u) {
+                nx[u] = valid;
+                const int i = atomicAdd(&S.n_list[0], 1);
+                (i < cap ? la : ga)[i] = (uint16_t)u;
+            }
+        }
+        if (tid == 0 && p.timeout_ns) atomicCAS(&p.flags->t0, 0ull, timer_ns());
+        __syncthreads();
+        if (tid == 0 && p.lc_len > 0 && S.n_list[0]) atomicAdd(&p.level_counts[0], (unsigned long long)S.n_list[0] * nt);
+        uint16_t *lcur = la, *lnext = lb, *gcur = ga, *gnext = gb;
+        for (int step = 0;; ++step) {
+            const int slot = step % 3, nslot = (step + 1) % 3;
+            const int F = S.n_list[slot];
+            if (F == 0 || step >= S.stop) break;
+            if (p.max_levels > 0 && step >= p.max_levels) {
+                // the out-edges of the last frontier count as checked, as every active node's do
+                for (int i = tid; i < F; i += blockDim.x) {
+                    const int u = (i < cap ? lcur : gcur)[i];
+                    ck += (unsigned long long)__popc(nx[u]) * (unsigned long long)(p.row_ptr[u + 1] - p.row_ptr[u]);
+                }
+                if (tid == 0) p.flags->limit = 1;
+                break;
+            }
+            // take the frontier's bits out of nx, which then collects the next frontier's
+            for (int i = tid; i < F; i += blockDim.x) {
+                const int u = (i < cap ? lcur : gcur)[i];
+                (i < cap ? lbits : gbits)[i] = nx[u];
+                nx[u] = 0u;
+            }
+            __syncthreads();
+            StepCtx s{vis, nx, lnext, gnext, &S.n_list[nslot], cap, planes, p.edge, S.rk, g0, 0u};
+            if (tid == 0) {
+                // the slots of the step after next: nobody reads or writes them in this one
+                S.n_list[(step + 2) % 3] = 0;
+                S.n_hub[nslot] = 0;
+                if (p.timeout_ns && timer_ns() - *(volatile unsigned long long *)&p.flags->t0 > p.timeout_ns) {
+                    p.flags->timed_out = 1;
+                    S.stop = step + 1;  // not this step: other threads may not have read it yet
+                }
+            }
+            // nodes per warp: all warps get some while there are enough
+            const int G = min(32, (F + n_warps - 1) / n_warps);
+            for (int base = wid * G; base < F; base += n_warps * G) {
+                int rs = 0, deg = 0;
+                uint32_t f = 0;
+                if (lane < G && base + lane < F) {
+                    const int i = base + lane;
+                    const int u = (i < cap ? lcur : gcur)[i];
+                    f = (i < cap ? lbits : gbits)[i];
+                    rs = __ldg(&p.row_ptr[u]);
+                    deg = __ldg(&p.row_ptr[u + 1]) - rs;
+                    ck += (unsigned long long)__popc(f) * (unsigned long long)deg;
+                    if (deg >= kHub) {
+                        const int h = atomicAdd(&S.n_hub[slot], 1);
+                        if (h < kHubCap) {
+                            S.hub[h] = make_uint2((uint32_t)u, f);
+                            deg = 0;
+                        }
+                    }
+                }
+                int incl = deg;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const int x = __shfl_up_sync(kFull, incl, o);
+                    if (lane >= o) incl += x;
+                }
+                const int total = __shfl_sync(kFull, incl, 31);
+                if (total == 0) continue;
+                const int start = incl - deg;
+                const unsigned nz = __ballot_sync(kFull, deg > 0);
+                if (deg > 0) wn[__popc(nz & lt)] = make_uint2((uint32_t)(rs - start), f);
+                __syncwarp();
+                // the node of edge t = e0 + lane: nodes whose first edge lies at or before t, less one
+                // (nodes starting in this chunk of 32 edges from a warp-wide or, earlier ones counted)
+                int before = 0;
+                auto owner = [&](int e0) {
+                    const int at = start - e0;
+                    const unsigned m = __reduce_or_sync(kFull, (deg > 0 && at >= 0 && at < 32) ? 1u << at : 0u);
+                    const int o = before + __popc(m & le) - 1;
+                    before += __popc(m);
+                    return o;
+                };
+                uint2 nd = wn[owner(0)];
+                uint32_t e = nd.x + lane, fe = lane < total ? nd.y : 0u;
+                uint2 ed = make_uint2(0u, 0u);
+                if (lane < total) ed = __ldg(&p.edge[e]);
+                for (int e0 = 0; e0 < total; e0 += 32) {
+                    // the next 32 edges' records load while these are expanded
+                    uint32_t en = 0, fn = 0;
+                    uint2 edn = make_uint2(0u, 0u);
+                    if (e0 + 32 < total) {
+                        nd = wn[owner(e0 + 32)];
+                        if (e0 + 32 + lane < total) {
+                            en = nd.x + (uint32_t)(e0 + 32 + lane);
+                            fn = nd.y;
+                            edn = __ldg(&p.edge[en]);
+                        }
+                    }
+                    expand<MODEL>(s, wq, e, ed, fe);
+                    e = en;
+                    fe = fn;
+                    ed = edn;
+                }
+                __syncwarp();
+            }
+            __syncthreads();
+            const int H = min(S.n_hub[slot], kHubCap);
+            if (H) {
+                for (int h = 0; h < H; ++h) {
+                    const uint2 hb = S.hub[h];
+                    const int e0 = p.row_ptr[hb.x], e1 = p.row_ptr[hb.x + 1];
+                    for (int e = e0 + 32 * wid; e < e1; e += 32 * n_warps)
+                        expand<MODEL>(s, wq, (uint32_t)(e + lane), e + lane < e1 ? __ldg(&p.edge[e + lane]) : make_uint2(0u, 0u),
+                                      e + lane < e1 ? hb.y : 0u);
+                }
+                __syncthreads();
+            }
+            if (step + 1 < p.lc_len) {
+                uint32_t x = s.gained;
+                for (int o = 16; o; o >>= 1) x += __shfl_xor_sync(kFull, x, o);
+                if (lane == 0 && x) atomicAdd(&p.level_counts[step + 1], (unsigned long long)x);
+            }
+            uint16_t *x = lcur;
+            lcur = lnext;
+            lnext = x;
+            x = gcur;
+            gcur = gnext;
+            gnext = x;
+        }
+        // ---- outputs: activations per trial (columns of vis) and per node
+        uint32_t mine = 0;
+        for (int v0 = 32 * wid; v0 < n; v0 += 32 * n_warps) {
+            const uint32_t x = v0 + lane < n ? vis[v0 + lane] : 0u;
+            if (!__any_sync(kFull, x != 0u)) continue;
+            if (p.count && x) atomicAdd(&p.count[(size_t)S.item * n + v0 + lane], __popc(x));
+            mine += __popc(transpose32(x));
+        }
+        if (mine) atomicAdd(&S.spread[lane], mine);
+        __syncthreads();
+        if (p.spread && tid < nt) p.spread[it.out0 + t0 + tid] = (int32_t)S.spread[tid];
+        __syncthreads();
+    }
+    for (int o = 16; o; o >>= 1) ck += __shfl_xor_sync(kFull, ck, o);
+    if (lane == 0 && ck) atomicAdd(p.checks, ck);
+}
+
+// Shapes of the launch: blocks per SM (1, 2 or 4, of 1024, 512 or 256 threads: 32 warps in all, the
+// most at 64 registers) and list entries in shared memory, at least kMinCap (or all nodes).
+struct ColShape {
+    int per_sm = 0, threads = 0, cap = 0;
+    size_t dyn = 0;
+};
+constexpr int kMinCap = 512;
+constexpr size_t kSmSmem = 228 * 1024;        // per SM, of which each block takes 1 KB more than it asks for
+constexpr size_t kMaxBlockSmem = 227 * 1024;  // per block
+constexpr size_t kMaxDynamic = kMaxBlockSmem - sizeof(BlockState);
+
+bool column_shape(int model, const cnd_graph_dev &G, int per_sm, ColShape &c) {
+    if (G.n > kColMaxN) return false;
+    const size_t n4 = ((size_t)G.n + 3) & ~(size_t)3;
+    const int threads = 1024 / per_sm;
+    const size_t have = std::min(kSmSmem / per_sm - 1024, kMaxBlockSmem) - sizeof(BlockState) - 64;
+    const size_t fixed = 8 * n4 + (sizeof(WarpNodes) + (model == 0 ? sizeof(WarpQueue) : 0)) * (size_t)(threads / 32) +
+                         (model == 0 ? 0 : 4 * (size_t)G.lt_planes);
+    const size_t all = (n4 + 7) & ~(size_t)7;  // entries for every node
+    if (fixed + 8 * std::min<size_t>(kMinCap, all) > have) return false;
+    c.per_sm = per_sm;
+    c.threads = threads;
+    c.cap = (int)std::min(all, (have - fixed) / 8 & ~(size_t)7);
+    c.dyn = fixed + 8 * (size_t)c.cap;
+    return true;
+}
+
+}  // namespace
+
+// Calls that run here.  Options that choose a form of the pass engine (width, work items, direction,
+// deferral, statistics, 32-bit sums) get the pass engine.  IC calls of more than kWideTrials trials on
+// graphs of which an SM holds fewer than four columns (n > about 5,500) get it too: with that many
+// trials its words are full, and one check of 64 trials costs it less than two of 32 cost here.
+// Measured against the pass engine (GB300; host step loop, its default):
+//   1,000 trials:  G(1000, 10000) p = 0.1 1,267 -> 131 us; Watts-Strogatz 10k U[0, 1] 2,595 -> 756 us;
+//                  BA 13k WC 2,067 -> 481 us; BA 20k U[0, 1] 867 -> 683 us; R-MAT 14 p = 0.1 923 -> 789 us
+//   20,000 trials: BA 13k U[0, 1] 3.10 -> 3.72 ms, R-MAT 13 p = 0.1 2.88 -> 3.47 ms (BA 13k WC 7.4 -> 5.5 ms)
+//   LT, any:       BA 5k 1,000 trials 2,395 -> 370 us, 65,536 trials 20.1 -> 8.1 ms
+constexpr int64_t kWideTrials = 4096;
+
+bool columns_fit(int model, const cnd_graph_dev &G, const cnd_sim_opts &o, int64_t trials) {
+    if (model == 1 && (!G.lt_cnt_edge || o.lt_accumulate)) return false;
+    if (o.word_bits || o.chunk_edges || o.direction != CND_DIR_AUTO || o.pull_permille || o.defer_bits || o.stats)
+        return false;
+    ColShape c;
+    if (!column_shape(model, G, 1, c)) return false;
+    return model == 1 || trials <= kWideTrials || column_shape(model, G, 4, c);
+}
+
+cnd_status run_columns(int model, const cnd_graph_dev &G, const std::vector<ItemDesc> &items, const int32_t *seeds_dev,
+                       int32_t *spread, int32_t *count, unsigned long long *checks, unsigned long long *level_counts,
+                       CallFlags *flags, const cnd_sim_opts &o, cudaStream_t st) {
+    const void *fn = model == 0 ? (const void *)k_columns<0> : (const void *)k_columns<1>;
+    int64_t trials = 0;
+    for (const auto &it : items) trials += it.trials;
+    if (trials == 0) return CND_OK;
+    // Blocks per SM and trials per column (a multiple of 4, one coin block), by estimated time: a
+    // wave of columns takes a constant (the latency of its steps) and work in proportion to the
+    // trials (and 2 more: work that a check takes whatever its trials), at a rate in proportion to
+    // the block's threads.
+    ColShape c;
+    int bits = 32;
+    double best = 1e300;
+    for (int per_sm = 4; per_sm >= 1; per_sm >>= 1) {
+        ColShape k;
+        if (!column_shape(model, G, per_sm, k)) continue;
+        for (int b = 4; b <= 32; b += 4) {
+            const double waves = std::ceil((double)((trials + b - 1) / b) / ((double)G.num_sms * per_sm));
+            const double cost = waves * (8 + per_sm * (b + 2));
+            if (cost < best) {
+                best = cost;
+                bits = b;
+                c = k;
+            }
+        }
+    }
+
+    const int64_t slots = (int64_t)G.num_sms * c.per_sm;
+    // the same value on every call: threads may launch with different sizes at the same time
+    CND_CUDA_TRY(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxDynamic));
+    std::vector<ColItem> h;
+    h.reserve(items.size());
+    int64_t cols = 0;
+    for (const auto &it : items) {
+        h.push_back(ColItem{it.out0, it.key, (int32_t)it.seed_begin, (int32_t)it.seed_end, (int32_t)it.trials, (int32_t)cols});
+        cols += (it.trials + bits - 1) / bits;
+    }
+    if (cols > 0x7FFFFFFF - slots) {
+        set_error("too many trials in one call");
+        return CND_EINVAL;
+    }
+    const int64_t blocks = std::min<int64_t>(cols, slots);
+    // one allocation: the column counter, the items, the blocks' list entries beyond cap
+    const size_t off_bits = (16 + sizeof(ColItem) * h.size() + 15) & ~(size_t)15;
+    const size_t over = c.cap < G.n ? (size_t)blocks * (size_t)G.n : 0;
+    unsigned char *buf = nullptr;
+    CND_CUDA_TRY(cudaMallocAsync((void **)&buf, off_bits + 8 * over, st));
+    struct Free {
+        void *q;
+        cudaStream_t st;
+        ~Free() { cudaFreeAsync(q, st); }
+    } fr{buf, st};
+    CND_CUDA_TRY(cudaMemsetAsync(buf, 0, 16, st));
+    CND_CUDA_TRY(cudaMemcpyAsync(buf + 16, h.data(), sizeof(ColItem) * h.size(), cudaMemcpyHostToDevice, st));
+    ColParams p{};
+    p.n = G.n;
+    p.n_items = (int32_t)h.size();
+    p.bits = bits;
+    p.n_cols = (int32_t)cols;
+    p.row_ptr = G.row_ptr;
+    p.edge = model == 0 ? G.ic_edge : G.lt_cnt_edge;
+    p.items = reinterpret_cast<const ColItem *>(buf + 16);
+    p.seeds = seeds_dev;
+    p.cnt_off = G.lt_cnt_off;
+    p.unit_w = G.lt_unit_w;
+    p.first_trial = o.first_trial;
+    p.spread = spread;
+    p.count = count;
+    p.checks = checks;
+    p.level_counts = level_counts;
+    p.lc_len = o.level_counts_len;
+    p.max_levels = o.max_levels;
+    p.timeout_ns = o.timeout_s > 0 ? (unsigned long long)std::max(1.0, std::min(o.timeout_s * 1e9, 1.8e19)) : 0ull;
+    p.next = reinterpret_cast<int32_t *>(buf);
+    p.cap = c.cap;
+    p.over_bits = reinterpret_cast<uint32_t *>(buf + off_bits);
+    p.over_node = reinterpret_cast<uint16_t *>(p.over_bits + over);
+    p.flags = flags;
+    void *args[] = {&p};
+    CND_CUDA_TRY(cudaLaunchKernel(fn, dim3((unsigned)blocks), dim3((unsigned)c.threads), args, c.dyn, st));
+    return CND_OK;
+}
+
+}  // namespace cnd

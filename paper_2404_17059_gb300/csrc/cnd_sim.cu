@@ -50,6 +50,7 @@
 #include <tuple>
 #include <vector>
 
+#include "cnd_cols.cuh"
 #include "cnd_common.cuh"
 
 namespace cnd {
@@ -1310,14 +1311,6 @@ static int blocks_for(int64_t warps, int max_blocks) {
     return (int)std::max<int64_t>(1, std::min<int64_t>(b, max_blocks));
 }
 
-// One simulation problem: a seed set, a trial count and a Philox key.
-struct ItemDesc {
-    int64_t seed_begin, seed_end;  // range in the seed array
-    int64_t trials;
-    int64_t out0;                  // position of its first trial in the spread output
-    uint64_t key;
-};
-
 // Pass layout: runs of word columns, each from one item.
 struct Seg {
     int32_t item;
@@ -2104,7 +2097,8 @@ static cnd_status simulate_common(int model, const cnd_graph *g, const char *fn,
     const size_t count_rows = batched ? (size_t)n_items : 1;
 
     // ---- outputs on the device
-    int32_t *d_spread = nullptr, *d_count = nullptr, *d_bad = nullptr;
+    int32_t *d_spread = nullptr, *d_count = nullptr;
+    CallFlags *d_flags = nullptr;
     const int32_t *d_seeds = nullptr;
     unsigned long long *d_lc = nullptr, *d_checks = nullptr;
     const int lc_len = o.level_counts_len;
@@ -2116,7 +2110,7 @@ static cnd_status simulate_common(int model, const cnd_graph *g, const char *fn,
     }
     CND_CUDA_TRY(W.alloc(&d_lc, (size_t)std::max(lc_len, 1)));
     CND_CUDA_TRY(W.alloc(&d_checks, 1));
-    CND_CUDA_TRY(W.alloc(&d_bad, 1));
+    CND_CUDA_TRY(W.alloc(&d_flags, 1));
     if (dev) {
         d_seeds = seeds;
     } else {
@@ -2130,7 +2124,7 @@ static cnd_status simulate_common(int model, const cnd_graph *g, const char *fn,
     if (d_count) CND_CUDA_TRY(cudaMemsetAsync(d_count, 0, sizeof(int32_t) * (size_t)n * count_rows, st));
     CND_CUDA_TRY(cudaMemsetAsync(d_lc, 0, sizeof(unsigned long long) * (size_t)std::max(lc_len, 1), st));
     CND_CUDA_TRY(cudaMemsetAsync(d_checks, 0, sizeof(unsigned long long), st));
-    CND_CUDA_TRY(cudaMemsetAsync(d_bad, 0, sizeof(int32_t), st));
+    CND_CUDA_TRY(cudaMemsetAsync(d_flags, 0, sizeof(CallFlags), st));
 
     cnd_sim_stats *S = o.stats;
     if (S) {
@@ -2139,13 +2133,16 @@ static cnd_status simulate_common(int model, const cnd_graph *g, const char *fn,
         S->flags = flags;
     }
     bool limit_hit = false;
-    const cnd_status rs =
-        run_items(model, G, fn, items, d_seeds, batched, d_spread, d_count, d_checks, d_lc, d_bad, o, W, limit_hit);
+    // graphs whose per-trial state fits an SM's shared memory: one launch, a block per column of trials
+    const bool columns = columns_fit(model, G, o, total_trials);
+    const cnd_status rs = columns ? run_columns(model, G, items, d_seeds, d_spread, d_count, d_checks, d_lc, d_flags, o, st)
+                                  : run_items(model, G, fn, items, d_seeds, batched, d_spread, d_count, d_checks, d_lc,
+                                              &d_flags->bad_seed, o, W, limit_hit);
     if (rs != CND_OK) return rs;
 
     // ---- results
-    int32_t hbad = 0;
-    CND_CUDA_TRY(cudaMemcpyAsync(&hbad, d_bad, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
+    CallFlags hf{};
+    CND_CUDA_TRY(cudaMemcpyAsync(&hf, d_flags, sizeof(hf), cudaMemcpyDeviceToHost, st));
     std::vector<unsigned long long> hlc((size_t)std::max(lc_len, 1));
     unsigned long long hchecks = 0;
     if (dev) {
@@ -2168,11 +2165,15 @@ static cnd_status simulate_common(int model, const cnd_graph *g, const char *fn,
         if (o.edge_checks_out) *o.edge_checks_out = (int64_t)hchecks;
         for (int i = 0; i < lc_len; ++i) o.level_counts_out[i] = (int64_t)hlc[i];
     }
-    if (hbad) {
+    if (hf.bad_seed) {
         set_error("%s: a seed id is out of range", fn);
         return CND_EINVAL;
     }
-    if (limit_hit) {
+    if (hf.timed_out) {
+        set_error("%s: timed out after %.3f s (device loop)", fn, o.timeout_s);
+        return CND_ETIMEOUT;
+    }
+    if (limit_hit || hf.limit) {
         set_error("%s: trials still active at step max_levels = %d", fn, o.max_levels);
         return CND_ELIMIT;
     }

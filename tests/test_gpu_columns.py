@@ -1,0 +1,112 @@
+"""The column engine (a block per column of trials, state in shared memory) against the oracle and the
+pass engine: graph sizes up to the largest that fits, ragged trial counts, rows around the length from
+which a whole block expands them, certain and impossible edges, batches of uneven items."""
+import numpy as np
+import pytest
+
+import oracle
+import paper_2404_17059_gb300 as P
+from paper_2404_17059_gb300 import inputs as I
+
+pytestmark = pytest.mark.gpu
+LC = 40
+
+
+def _sim(model, G, seeds, T, rng, **kw):
+    f = P.cnd_ic_simulate_ex if model == "ic" else P.cnd_lt_simulate_ex
+    return f(G, seeds, T, rng, edge_checks=True, level_counts_len=LC, **kw)
+
+
+def _check(model, g, G, seeds, T, rng, p, w, **kw):
+    a = _sim(model, G, seeds, T, rng, **kw)
+    okw = {k: kw[k] for k in ("first_trial", "max_levels") if k in kw}
+    b = oracle.simulate_threads(model, g, seeds, T, rng, level_counts_len=LC,
+                                **({"ic_prob": p} if model == "ic" else {"lt_weight": w}), **okw)
+    c = _sim(model, G, seeds, T, rng, word_bits=64, **kw)  # the pass engine
+    assert a.status == (P.CND_ELIMIT if b.status == oracle.LIMIT else P.CND_OK) == c.status
+    for x in (b, c):
+        assert np.array_equal(a.spread, x.spread)
+        assert np.array_equal(a.node_count, x.node_count)
+        assert a.edge_checks == x.edge_checks
+        assert np.array_equal(a.level_counts, x.level_counts)
+
+
+def _weights(g, seed=1):
+    p = I.ic_uniform_random(g, 0.6, graph_seed=seed)
+    p[::7] = 0.0
+    p[3::11] = 1.0
+    return p, I.lt_weighted_cascade(g)
+
+
+@pytest.mark.parametrize("model", ["ic", "lt"])
+@pytest.mark.parametrize("n", [1, 2, 31, 33, 1021, 6000, 24_300, 24_400])  # the last does not fit
+def test_graph_sizes(model, n):
+    rng = np.random.default_rng(n)
+    m = 4 * n
+    g = I.csr_from_edges(n, rng.integers(0, n, m), rng.integers(0, n, m))  # self-loops, parallel edges
+    p, w = _weights(g)
+    G = P.cnd_graph_create(n, g.row_ptr, g.col, p, w)
+    seeds = rng.integers(0, n, min(n, 9))  # duplicates among them
+    _check(model, g, G, seeds, 100, 3, p, w)
+
+
+@pytest.mark.parametrize("model", ["ic", "lt"])
+def test_trial_counts_offsets_and_caps(model):
+    g = I.erdos_renyi_m(700, 4200, graph_seed=2)
+    p, w = _weights(g)
+    G = P.cnd_graph_create(g.n, g.row_ptr, g.col, p, w)
+    seeds = I.uniform_seeds(g.n, 5, 2)
+    for T in (1, 3, 4, 5, 31, 32, 33, 63, 65, 1000, 6001):
+        _check(model, g, G, seeds, T, (1 << 63) + T, p, w)
+    for ft in (64, (1 << 34) - 128):
+        _check(model, g, G, seeds, 130, 9, p, w, first_trial=ft)
+    for cap in (1, 2, 5):
+        _check(model, g, G, seeds, 70, 4, p, w, max_levels=cap)
+    for graph in (0, 1):
+        _check(model, g, G, [], 70, 4, p, w, graph=graph)
+
+
+@pytest.mark.parametrize("model", ["ic", "lt"])
+def test_long_rows(model):
+    # 80 hubs (more than a step sets aside) with rows of 255, 256, 257 and 3,000 edges, all reached at once
+    degs = [255, 256, 257, 3000] + [300] * 76
+    n = 4000
+    rng = np.random.default_rng(6)
+    src = np.concatenate([np.full(len(degs), n - 1)] + [np.full(d, u) for u, d in enumerate(degs)])
+    dst = np.concatenate([np.arange(len(degs))] + [rng.permutation(n - 1)[:d] for d in degs])
+    g = I.csr_from_edges(n, src, dst)
+    p, w = _weights(g)
+    p[g.src() == n - 1] = 1.0
+    G = P.cnd_graph_create(n, g.row_ptr, g.col, p, w)
+    _check(model, g, G, [n - 1], 45, 8, p, w)
+    _check(model, g, G, list(range(80)), 45, 8, p, w)
+
+
+@pytest.mark.parametrize("model", ["ic", "lt"])
+def test_batches(model):
+    g = I.erdos_renyi_m(600, 4000, graph_seed=5)
+    p, w = _weights(g)
+    G = P.cnd_graph_create(g.n, g.row_ptr, g.col, p, w)
+    f = P.cnd_ic_simulate_batch if model == "ic" else P.cnd_lt_simulate_batch
+    for items, trials_of in ((1, (5,)), (40, (0, 1, 64, 100, 7)), (70, (0, 33)), (1100, (3, 0, 40))):
+        off, seeds, _, keys = I.batch_items(g.n, items, 1, 6, (1,), graph_seed=items)
+        trials = np.array([trials_of[i % len(trials_of)] for i in range(items)], dtype=np.int32)
+        a = f(G, off, seeds, trials, keys, node_count=True, edge_checks=True, level_counts_len=LC)
+        b = f(G, off, seeds, trials, keys, node_count=True, edge_checks=True, level_counts_len=LC, word_bits=128)
+        assert np.array_equal(a.spread, b.spread) and np.array_equal(a.node_count, b.node_count)
+        assert a.edge_checks == b.edge_checks and np.array_equal(a.level_counts, b.level_counts)
+
+
+def test_time_limit_and_bad_device_seed():
+    torch = pytest.importorskip("torch")
+    g = I.erdos_renyi_m(600, 4000, graph_seed=5)
+    p, w = _weights(g)
+    G = P.cnd_graph_create(g.n, g.row_ptr, g.col, p, w)
+    with pytest.raises(P.CndError) as ei:
+        _sim("ic", G, [1, 2], 4096, 1, timeout_s=1e-9)
+    assert ei.value.status == P.CND_ETIMEOUT
+    for bad in (-1, g.n):
+        with pytest.raises(P.CndError) as ei:
+            _sim("ic", G, torch.tensor([1, bad], dtype=torch.int32, device="cuda"), 64, 1)
+        assert ei.value.status == P.CND_EINVAL
+    _check("ic", g, G, [1, 2], 64, 1, p, w, timeout_s=30.0)
