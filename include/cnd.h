@@ -75,7 +75,7 @@ typedef int32_t cnd_status;
 #define CND_ETIMEOUT (-5)  /* time limit (timeout_s) reached; outputs are not valid */
 #define CND_EOVERFLOW (-6) /* LT in-weights of a node sum above 2^32 - 1 */
 
-#define CND_DIR_AUTO 0 /* push or pull per step, by frontier size (see pull_permille) */
+#define CND_DIR_AUTO 0 /* push or pull per step, by the frontier (see pull_permille) */
 #define CND_DIR_PUSH 1
 #define CND_DIR_PULL 2
 
@@ -122,7 +122,7 @@ typedef struct cnd_sim_opts {
                                   (outputs are still written) */
     int32_t direction;         /* CND_DIR_* */
     int32_t word_bits;         /* trials held per node per pass: 0 = automatic, else a multiple
-                                  of 64 up to 131072 (pulling passes hold at most 16384) */
+                                  of 64 up to 131072 (IC passes that may pull hold at most 16384) */
     int32_t device_ptrs;       /* 1: seeds and all outputs are device pointers; the work runs
                                   on `stream`, and the call returns once it is complete */
     void *stream;              /* cudaStream_t to run on; NULL = legacy default stream */
@@ -131,8 +131,9 @@ typedef struct cnd_sim_opts {
                                   (trial, node) pairs activated at step L */
     int32_t level_counts_len;
     int32_t pull_permille;     /* IC, AUTO: pull when the frontier's out-edges exceed this many
-                                  thousandths of m; 0 = push only (the measured default).  LT
-                                  always pushes */
+                                  thousandths of m; 0 = push only (the measured default).  LT in
+                                  the counting form (see lt_accumulate) chooses per step by the
+                                  work of its frontier; its 32-bit sums always push */
     int32_t chunk_edges;       /* edges per push work item (0 = automatic) */
     int32_t defer_bits;        /* > 0: a node's word with fewer newly active trials than this may
                                   wait for more before its out-edges are examined; the spreads,

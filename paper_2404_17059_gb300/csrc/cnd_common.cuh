@@ -13,6 +13,9 @@ namespace cnd {
 
 constexpr uint32_t kAlways = 0xFFFFFFFFu;  // IC threshold of an edge with p == 1
 constexpr uint32_t kFull = 0xFFFFFFFFu;    // full warp mask
+constexpr uint32_t kNoSource = 0xFFFFFFFFu;
+constexpr int kPullShort = 64;
+constexpr int kPullItem = 255;  // an 8-bit bit-sliced count holds it
 
 // ---------------------------------------------------------------- Philox4x32-10
 // Counter-based generator of Salmon et al. (SC'11).  One call yields four
@@ -96,6 +99,13 @@ struct cnd_graph_dev {
     int32_t *lt_cnt_off = nullptr;  // [n+1] prefix sums of L_v
     uint32_t *lt_unit_w = nullptr;  // [n] the common in-weight of v (0: no in-edge of non-zero weight)
     int64_t lt_planes = 0;          // sum of L_v (planes per word column)
+    // ... and its pull step: the source of every in-edge (kNoSource: zero weight), and the in-rows as
+    // items {node, first edge, edges | 256 if the row is split over several items, counter tag of the
+    // node}, longest first; the first n_lt_long items have more than kPullShort edges, none more than
+    // kPullItem
+    uint32_t *lt_in_src = nullptr;  // [m]
+    int4 *lt_pull_items = nullptr;
+    int32_t n_lt_pull_items = 0, n_lt_long = 0;
 };
 
 // ---------------------------------------------------------------- errors

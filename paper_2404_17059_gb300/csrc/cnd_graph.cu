@@ -62,6 +62,14 @@ __global__ void k_build_in_edges(int32_t m, const int32_t *__restrict__ in_src, 
     }
 }
 
+// sources of the in-edges for the LT pull step
+__global__ void k_build_lt_in_src(int32_t m, const uint4 *__restrict__ in_edge, uint32_t *__restrict__ out) {
+    for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < m; k += (int64_t)gridDim.x * blockDim.x) {
+        const uint4 e = in_edge[k];
+        out[k] = e.w ? e.x : kNoSource;
+    }
+}
+
 __global__ void k_philox(uint32_t k0, uint32_t k1, const uint4 *__restrict__ ctr, int64_t count, uint4 *__restrict__ out) {
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < count; i += (int64_t)gridDim.x * blockDim.x) {
         const uint4 c = ctr[i];
@@ -114,6 +122,8 @@ static void free_dev(cnd_graph_dev &d) {
     cudaFree(d.lt_cnt_edge);
     cudaFree(d.lt_cnt_off);
     cudaFree(d.lt_unit_w);
+    cudaFree(d.lt_in_src);
+    cudaFree(d.lt_pull_items);
     d = cnd_graph_dev{};
 }
 
@@ -308,6 +318,29 @@ cnd_status cnd_graph_create(int32_t n, int32_t m, const int32_t *row_ptr, const 
             if ((e = cudaMemcpy(d_tmp_a, in_src.data(), sizeof(int32_t) * (size_t)m, cudaMemcpyHostToDevice)) != cudaSuccess) { fail(e, "copy in_src"); break; }
             if ((e = cudaMemcpy(d_tmp_b, in_eid.data(), sizeof(int32_t) * (size_t)m, cudaMemcpyHostToDevice)) != cudaSuccess) { fail(e, "copy in_eid"); break; }
             k_build_in_edges<<<blocks, threads>>>(m, d_tmp_a, d_tmp_b, d.ic_edge, d.lt_edge, d.in_edge);
+        }
+        if (d.lt_cnt_edge) {
+            // counting sort of the items by descending length
+            std::vector<int32_t> at(kPullItem + 2, 0);
+            auto each = [&](auto &&f) {
+                for (int32_t v = 0; v < n; ++v)
+                    for (int64_t k = in_row_ptr[v]; k < in_row_ptr[v + 1]; k += kPullItem)
+                        f(v, (int32_t)k, (int32_t)std::min<int64_t>(kPullItem, in_row_ptr[v + 1] - k));
+            };
+            each([&](int32_t, int32_t, int32_t len) { at[(size_t)(kPullItem - len) + 1]++; });
+            for (size_t i = 1; i < at.size(); ++i) at[i] += at[i - 1];
+            std::vector<int4> items((size_t)at.back());
+            d.n_lt_long = at[(size_t)(kPullItem - kPullShort)];
+            each([&](int32_t v, int32_t k, int32_t len) {
+                items[(size_t)at[(size_t)(kPullItem - len)]++] =
+                    make_int4(v, k, len | (in_row_ptr[v + 1] - in_row_ptr[v] > kPullItem ? 256 : 0),
+                              (int32_t)(((uint32_t)cnt_off[v] << 5) | (uint32_t)(cnt_off[v + 1] - cnt_off[v])));
+            });
+            if ((e = cudaMalloc(&d.lt_in_src, sizeof(uint32_t) * mb)) != cudaSuccess) { fail(e, "alloc lt_in_src"); break; }
+            if ((e = cudaMalloc(&d.lt_pull_items, sizeof(int4) * std::max<size_t>(items.size(), 1))) != cudaSuccess) { fail(e, "alloc lt_pull_items"); break; }
+            if (m > 0) k_build_lt_in_src<<<blocks, threads>>>(m, d.in_edge, d.lt_in_src);
+            if (!items.empty() && (e = cudaMemcpy(d.lt_pull_items, items.data(), sizeof(int4) * items.size(), cudaMemcpyHostToDevice)) != cudaSuccess) { fail(e, "copy lt_pull_items"); break; }
+            d.n_lt_pull_items = (int32_t)items.size();
         }
         if ((e = cudaGetLastError()) != cudaSuccess) { fail(e, "launch"); break; }
         if ((e = cudaDeviceSynchronize()) != cudaSuccess) { fail(e, "sync"); break; }

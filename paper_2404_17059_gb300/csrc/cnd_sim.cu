@@ -78,8 +78,11 @@ struct Frontier {
     uint16_t *pw = nullptr;    // [n*B] pool: word index
     uint64_t *pb = nullptr;    // [n*B] pool: frontier bits
     int2 *work = nullptr;      // [work_cap] (slot, first edge of the item within the row)
-    int32_t *cnt = nullptr;    // device [4]: pool pairs, slots (one 64-bit word), work items, out-edges of the slots
+    // device [kCnt]: pool pairs, slots (one 64-bit word), work items, out-edges of the slots, and their
+    // (edge, word) checks (64 bits)
+    int32_t *cnt = nullptr;
 };
+constexpr int kCnt = 6;
 
 // Step state of a run whose step loop executes on the device (CUDA-graph mode).
 struct Ctl {
@@ -128,6 +131,11 @@ struct Params {
     const uint4 *in_edge;      // {src, edge id, IC threshold, LT weight}
     uint64_t *fdense;          // [n*B] frontier words by node (zero outside the frontier)
     uint32_t *fbits;           // [ceil(n/32)] frontier nodes
+    // LT pull step
+    const uint32_t *lt_in_src;
+    const int4 *lt_items;
+    int32_t n_lt_items, n_lt_long;
+    int32_t fstride;           // words per row of fdense (LT: even, so that rows are 16-byte aligned)
     const uint64_t *wg0;       // [B] per-word trial-block index of bit 0
     uint64_t g_base;           // trial-block index (trial >> 2) of bit 0 of word 0
     unsigned long long *level_counts;
@@ -456,7 +464,13 @@ __global__ void __launch_bounds__(kBlock, MODE == 2 ? 4 : 6) k_finalize(Params p
             int dg = lane < kNPB ? s_deg[lane] : 0;
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) dg += __shfl_xor_sync(kFull, dg, o);
-            if (lane == 0 && dg) atomicAdd(&p.out.cnt[3], dg);
+            unsigned long long ckk = lane < kNPB ? (unsigned long long)s_deg[lane] * (unsigned)s_kept[lane] : 0ull;
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) ckk += __shfl_xor_sync(kFull, ckk, o);
+            if (lane == 0 && dg) {
+                atomicAdd(&p.out.cnt[3], dg);
+                atomicAdd((unsigned long long *)(p.out.cnt + 4), ckk);
+            }
             if (lane == 31) {
                 if (sk) ps0 = atomicAdd((unsigned long long *)p.out.cnt, ((unsigned long long)sh << 32) | (unsigned)sk);
                 if (sc) item0 = atomicAdd(&p.out.cnt[2], sc);
@@ -595,7 +609,13 @@ __global__ void __launch_bounds__(kBlock) k_collect(Params p_) {
             if (sk) ps0 = atomicAdd((unsigned long long *)p.out.cnt, ((unsigned long long)sh << 32) | (unsigned)sk);
             if (sc) item0 = atomicAdd(&p.out.cnt[2], sc);
         }
-        if (lane == 0 && dg) atomicAdd(&p.out.cnt[3], dg);
+        unsigned long long ckk = (unsigned long long)deg * (unsigned)K;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) ckk += __shfl_xor_sync(kFull, ckk, o);
+        if (lane == 0 && dg) {
+            atomicAdd(&p.out.cnt[3], dg);
+            atomicAdd((unsigned long long *)(p.out.cnt + 4), ckk);
+        }
         ps0 = __shfl_sync(kFull, ps0, 31);
         item0 = __shfl_sync(kFull, item0, 31);
         const int n_pairs = __shfl_sync(kFull, sk, 31), n_items = __shfl_sync(kFull, sc, 31);
@@ -1108,6 +1128,366 @@ __global__ void __launch_bounds__(kBlock) k_pull_ic(Params p_) {
     count_add(p, C_UPDATES, n_up);
 }
 
+// ---------------------------------------------------------------- pull (LT counting form)
+// The frontier of the step in node-indexed form for the pull step: a warp per slot writes the node's
+// whole row (zero where it has no bits), so rows need no clearing; the node's bit says the row is this
+// step's.  !SET: clear the bits again.
+template <bool SET>
+__global__ void __launch_bounds__(kBlock) k_frontier_rows(Params p_) {
+    Params p = p_;
+    resolve(p);
+    if (p.ctl && !p.ctl->pull) return;
+    const int lane = lane_id();
+    const int slots = p.in.cnt[1];
+    const int thread = blockIdx.x * blockDim.x + threadIdx.x, n_threads = gridDim.x * blockDim.x;
+    if (!SET) {
+        for (int sl = thread; sl < slots; sl += n_threads) p.fbits[p.in.node[sl] >> 5] = 0u;
+        return;
+    }
+    for (int sl = thread >> 5; sl < slots; sl += n_threads >> 5) {
+        const int u = p.in.node[sl];
+        const int off = p.in.poff[sl], k = p.in.pk[sl];
+        uint64_t *row = p.fdense + (size_t)u * p.fstride;
+        for (int j = lane; j < p.B; j += 32) row[j] = 0ull;
+        __syncwarp();
+        for (int j = lane; j < k; j += 32) row[p.in.pw[off + j]] = p.in.pb[off + j];
+        if (lane == 0) atomicOr(&p.fbits[u >> 5], 1u << (u & 31));
+    }
+}
+
+// Bit-sliced count of up to kPullItem one-bit inputs in each of 64 lanes of trials.
+struct SliceCount {
+    uint64_t s[8];
+
+    __device__ __forceinline__ void clear() {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) s[i] = 0ull;
+    }
+    // full adder: s + a + b -> s, returns the carry
+    static __device__ __forceinline__ uint64_t full(uint64_t &s, uint64_t a, uint64_t b) {
+        const uint64_t t = s ^ a, c = (s & a) | (t & b);
+        s = t ^ b;
+        return c;
+    }
+    // four inputs into planes 0 and 1; returns what carries into plane 2
+    __device__ __forceinline__ uint64_t add4(uint64_t x0, uint64_t x1, uint64_t x2, uint64_t x3) {
+        const uint64_t a = full(s[0], x0, x1), b = full(s[0], x2, x3);
+        return full(s[1], a, b);
+    }
+    __device__ __forceinline__ void carry2(uint64_t e, uint64_t f) {
+        uint64_t g = full(s[2], e, f);
+#pragma unroll
+        for (int i = 3; i < 8; ++i) {
+            const uint64_t h = s[i] & g;
+            s[i] ^= g;
+            g = h;
+        }
+    }
+};
+
+// Words of v that a pull step's counts carry into: vis and nxt of word w gain the trials of c.
+__device__ __forceinline__ void pull_activate(const Params &p, int v, int w, bool shared, uint64_t need, uint64_t c) {
+    const size_t idx = (size_t)v * p.B + w;
+    if (shared) {
+        atomicOr((unsigned long long *)p.vis + idx, (unsigned long long)c);
+        atomicOr((unsigned long long *)p.nxt + idx, (unsigned long long)c);
+    } else {
+        p.vis[idx] = (p.valid[w] & ~need) | c;
+        p.nxt[idx] = c;
+    }
+}
+
+// Add the counts to v's counters of word w (tag: first plane << 5 | planes, as in the edge records) in
+// the trials of `need` (those where v is inactive); what carries out of the top plane is activated and
+// returned.  Other warps may add to the same counters.
+__device__ __forceinline__ uint64_t pull_apply_shared(const Params &p, int v, uint32_t tag, int w, uint64_t need,
+                                                      const SliceCount &a, uint32_t &n_up) {
+    const int L = (int)(tag & 31u);
+    unsigned long long *pl = (unsigned long long *)p.planes + ((size_t)(tag >> 5) * p.B + (size_t)w * L);
+    uint64_t c = 0;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        if (i >= L) break;
+        // two addends of equal weight (count and carry): both set carries whatever the plane
+        const uint64_t s = a.s[i] & need, t = s ^ c;
+        c &= s;
+        if (t) {
+            ++n_up;
+            c |= (uint64_t)atomicXor(pl + i, (unsigned long long)t) & t;
+        }
+    }
+    for (int i = 8; i < L && c; ++i) {
+        ++n_up;
+        c &= (uint64_t)atomicXor(pl + i, (unsigned long long)c);
+    }
+    c &= need;
+    if (c) pull_activate(p, v, w, true, need, c);
+    return c;
+}
+
+// The same for words w and w + 1 of a row that only this warp adds to.  Their planes lie next to each
+// other and load together, four of each word at a time: one load waiting for the other's carry was a
+// third of the kernel's time.
+__device__ __forceinline__ void pull_apply_own(const Params &p, int v, uint32_t tag, int w, uint64_t need0, uint64_t need1,
+                                               SliceCount &a, SliceCount &b, uint32_t &n_up, uint64_t &act0,
+                                               uint64_t &act1) {
+    const int L = (int)(tag & 31u);
+    unsigned long long *pa = (unsigned long long *)p.planes + ((size_t)(tag >> 5) * p.B + (size_t)w * L);
+    unsigned long long *pb = pa + L;
+    uint64_t ca = 0, cb = 0;
+    uint64_t any = 0;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        a.s[i] &= need0;
+        b.s[i] &= need1;
+        any |= a.s[i] | b.s[i];
+    }
+    act0 = act1 = 0ull;
+    if (!any) return;
+#pragma unroll
+    for (int h = 0; h < 8; h += 4) {
+        if (h >= L || (h > 0 && !(a.s[4] | a.s[5] | a.s[6] | a.s[7] | ca | b.s[4] | b.s[5] | b.s[6] | b.s[7] | cb))) break;
+        uint64_t olda[4], oldb[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            olda[i] = need0 && h + i < L ? (uint64_t)__ldcg(pa + h + i) : 0ull;
+            oldb[i] = need1 && h + i < L ? (uint64_t)__ldcg(pb + h + i) : 0ull;
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            if (h + i >= L) break;
+            const uint64_t ta = a.s[h + i] ^ ca, tb = b.s[h + i] ^ cb;
+            ca = (a.s[h + i] & ca) | (olda[i] & ta);
+            cb = (b.s[h + i] & cb) | (oldb[i] & tb);
+            if (ta) {
+                ++n_up;
+                pa[h + i] = olda[i] ^ ta;
+            }
+            if (tb) {
+                ++n_up;
+                pb[h + i] = oldb[i] ^ tb;
+            }
+        }
+    }
+    for (int i = 8; i < L && (ca | cb); ++i) {
+        const uint64_t oa = ca ? (uint64_t)__ldcg(pa + i) : 0ull, ob = cb ? (uint64_t)__ldcg(pb + i) : 0ull;
+        if (ca) pa[i] = oa ^ ca;
+        if (cb) pb[i] = ob ^ cb;
+        n_up += (ca != 0ull) + (cb != 0ull);
+        ca &= oa;
+        cb &= ob;
+    }
+    act0 = ca & need0;
+    act1 = cb & need1;
+    if (act0) pull_activate(p, v, w, false, need0, act0);
+    if (act1) pull_activate(p, v, w + 1, false, need1, act1);
+}
+
+// Bits 2 i of the result: bit i of x (16 bits).
+__device__ __forceinline__ uint32_t spread2(uint32_t x) {
+    x = (x | (x << 8)) & 0x00FF00FFu;
+    x = (x | (x << 4)) & 0x0F0F0F0Fu;
+    x = (x | (x << 2)) & 0x33333333u;
+    return (x | (x << 1)) & 0x55555555u;
+}
+
+// Pull step of LT in the counting form.  A push step toggles one counter plane or more with an atomic
+// for every (edge, word) whose target still counts: scattered 8-byte reads and atomics, whose rate
+// bounds it (41 G checks/s on R-MAT-21).  Here a segment of LN lanes owns 2 LN words of a target, two
+// per lane.  The sources of the target's in-edges that are in the frontier are listed in shared memory;
+// each listed source adds its row of the frontier (16 LN contiguous bytes, mostly from L2), counted in
+// registers by carry-save adders, 8 rows at a time; the list is padded with row n, which is zero.  The
+// counters are then read and written once per target, word and step.  Rows of up to kPullShort in-edges
+// go to a segment each, longer ones to a warp per item, its segments taking turns on 8 listed rows and
+// adding up their counts; the counters of a row split over several items are added to atomically.
+//
+// Latency-bound (ncu, R-MAT-20, a dense step: 32 % issue active, long scoreboard 13 of 19 cycles per
+// issue, 1.4 TB/s DRAM): 36 % of the warps' time goes on gathering rows, a third on the counters, a
+// fifth on listing sources.  2 words per lane and 24 warps per SM at 80 registers; one word per lane at 64
+// registers took 107 against 73 ms per R-MAT-21 call, 32 warps with two words (spilled) the same as 24.
+// R-MAT-21, 1,000 trials (64 of 246 steps pull): expansion 364 -> 115 ms.
+template <int LN>
+__global__ void __launch_bounds__(kBlock, 3) k_pull_lt(Params p_) {
+    Params p = p_;
+    resolve(p);
+    if (p.ctl && !p.ctl->pull) return;
+    constexpr int SEG = 32 / LN;
+    constexpr int kLong = 256 + 8 * SEG;           // list entries of a long item, padded
+    constexpr int kShort = kPullShort + 8;         // ... of a short one
+    constexpr int kList = SEG * kShort > kLong ? SEG * kShort : kLong;
+    __shared__ int32_t s_list[kWarps][64];
+    __shared__ __align__(16) uint32_t s_src[kWarps][kList];
+    const int lane = lane_id();
+    const int wid = threadIdx.x >> 5;
+    const int seg = lane / LN, l = lane % LN;
+    const uint32_t seg_mask = (LN == 32 ? 0xFFFFFFFFu : (1u << (LN & 31)) - 1u) << (seg * LN);
+    const uint32_t below = (1u << lane) - 1u;
+    ListBuf lb{s_list[wid], 0};
+    const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int n_warps = (gridDim.x * blockDim.x) >> 5;
+    const int B = p.B;
+    const int chunks = (B + 2 * LN - 1) / (2 * LN);
+    uint32_t n_edges = 0, n_wc = 0, n_up = 0;
+    auto need_of = [&](int v, int w) {
+        return w < B ? p.valid[w] & ~(uint64_t)__ldcg((const unsigned long long *)p.vis + (size_t)v * B + w) : 0ull;
+    };
+    // list the sources of edges at, at + pitch, ... (4 per lane; `left` edges from `at` on) that are in
+    // the frontier; all loads of a kind are in flight together
+    auto scan = [&](uint32_t *list, int &count, int at, int left, int pitch, uint32_t mask) {
+        uint32_t u[4], f[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) u[i] = i * pitch < left ? __ldg(&p.lt_in_src[at + i * pitch]) : kNoSource;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) f[i] = u[i] != kNoSource ? __ldg(&p.fbits[u[i] >> 5]) : 0u;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const bool in = (f[i] >> (u[i] & 31u)) & 1u;
+            const uint32_t m = __ballot_sync(kFull, in) & mask;
+            if (in) list[count + __popc(m & below)] = u[i];
+            count += __popc(m);
+        }
+    };
+    // chunk ch of v gained trials in the even words m0 and the odd words m1 (bits): into the node's
+    // dirty mask, and the node into the list
+    auto record = [&](int v, int ch, bool leader, uint32_t m0, uint32_t m1) {
+        bool claimed = false;
+        if (leader && (m0 | m1)) {
+            const int w0 = 2 * LN * ch;
+            atomicOr((unsigned long long *)(p.dmask + (size_t)v * p.nq + (w0 >> 6)),
+                     (unsigned long long)(spread2(m0) | (spread2(m1) << 1)) << (w0 & 63));
+            claimed = atomicExch(&p.mark[v], p.stamp) != p.stamp;
+        }
+        lb.put(p, claimed, v);
+    };
+    // add the rows list[first + 8 i .. + 8), i = 0, step, 2 step, ..., below count
+    auto gather = [&](const uint32_t *list, int first, int count, int step, int w, SliceCount &a, SliceCount &b) {
+        const ulonglong2 *rows = reinterpret_cast<const ulonglong2 *>(p.fdense + w);
+        const size_t stride = (size_t)(p.fstride >> 1);
+        for (int i = first; i < count; i += step) {
+            uint64_t ca[2], cb[2];
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const uint4 q = *reinterpret_cast<const uint4 *>(list + i + 4 * h);
+                const ulonglong2 z0 = __ldg(rows + q.x * stride), z1 = __ldg(rows + q.y * stride);
+                const ulonglong2 z2 = __ldg(rows + q.z * stride), z3 = __ldg(rows + q.w * stride);
+                ca[h] = a.add4(z0.x, z1.x, z2.x, z3.x);
+                cb[h] = b.add4(z0.y, z1.y, z2.y, z3.y);
+            }
+            a.carry2(ca[0], ca[1]);
+            b.carry2(cb[0], cb[1]);
+            n_wc += 16;
+        }
+    };
+    // bring the counters of words w, w + 1 into L2 while the rows are counted
+    auto prefetch = [&](uint32_t tag, int w) {
+        const uint64_t *a = p.planes + ((size_t)(tag >> 5) * B + (size_t)w * (tag & 31u));
+        const int bytes = 16 * (int)(tag & 31u);
+        for (int o = 0; o < bytes; o += 128)
+            asm volatile("prefetch.global.L2 [%0];" ::"l"((const char *)a + o));
+    };
+    // ---- long items: a warp each
+    for (int it = warp; it < p.n_lt_long; it += n_warps) {
+        const int4 d = p.lt_items[it];
+        const int v = d.x, len = d.z & 255;
+        uint32_t *list = s_src[wid];
+        // nothing to do where every trial is active
+        bool open = false;
+        for (int w = lane; w < B; w += 32) open |= need_of(v, w) != 0ull;
+        if (!__any_sync(kFull, open)) continue;
+        int count = 0;
+        for (int e = 0; e < len; e += 128) scan(list, count, d.y + e + lane, len - e - lane, 32, kFull);
+        if (lane == 0) n_edges += len;
+        if (count == 0) continue;
+        if (lane < 8 * SEG) list[count + lane] = (uint32_t)p.n;
+        __syncwarp();
+        for (int ch = 0; ch < chunks; ++ch) {
+            const int w = 2 * (ch * LN + l);
+            // one read for all segments: another warp may activate trials of a split row meanwhile
+            const uint64_t need0 = __shfl_sync(kFull, need_of(v, w), l), need1 = __shfl_sync(kFull, need_of(v, w + 1), l);
+            if (seg == 0 && w < B) prefetch((uint32_t)d.w, w);
+            SliceCount a, b;
+            a.clear();
+            b.clear();
+            if (need0 | need1) gather(list, 8 * seg, count, 8 * SEG, w, a, b);
+            __syncwarp();
+#pragma unroll
+            for (int o = LN; o < 32; o <<= 1) {  // add the segments' counts
+                uint64_t c = 0, c1 = 0;
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    const uint64_t x = __shfl_xor_sync(kFull, a.s[i], o), y = __shfl_xor_sync(kFull, b.s[i], o);
+                    c = SliceCount::full(a.s[i], x, c);
+                    c1 = SliceCount::full(b.s[i], y, c1);
+                }
+            }
+            // every segment has the sums: segment 0 adds those of the even words, segment 1 the odd
+            uint64_t act = 0;
+            const uint64_t need = seg == 0 ? need0 : need1;
+            if (seg < 2 && need) {
+                if (seg == 1) a = b;
+                act = pull_apply_shared(p, v, (uint32_t)d.w, w + seg, need, a, n_up);
+            }
+            const uint32_t m = __ballot_sync(kFull, act != 0ull);
+            record(v, ch, lane == 0, m & ((1u << (LN & 31)) - 1u), (m >> LN) & ((1u << (LN & 31)) - 1u));
+        }
+        __syncwarp();
+    }
+    // ---- short items: a segment each; the next items' records and first sources load meanwhile
+    auto item_at = [&](int it) { return it < p.n_lt_items ? __ldg(&p.lt_items[it]) : make_int4(0, 0, 0, 0); };
+    const int step = n_warps * SEG;
+    int base = p.n_lt_long + warp * SEG;
+    int4 d = item_at(base + seg);
+    for (; base < p.n_lt_items; base += step) {
+        const int4 dn = item_at(base + step + seg);
+        const int len = d.z & 255;
+        uint32_t *list = s_src[wid] + seg * kShort;
+        int count = 0;
+        const int longest = __shfl_sync(kFull, len, 0);  // items are in descending order
+        for (int e = 0; e < longest; e += 4 * LN) scan(list, count, d.y + e + l, len - e - l, LN, seg_mask);
+        n_edges += l == 0 ? len : 0;
+        if (__any_sync(kFull, count != 0)) {
+            if (l < 8) list[count + l] = (uint32_t)p.n;
+            __syncwarp();
+            const int v = d.x;
+            for (int ch = 0; ch < chunks; ++ch) {
+                const int w = 2 * (ch * LN + l);
+                uint64_t act0 = 0, act1 = 0;
+                if (count) {
+                    const uint64_t need0 = need_of(v, w), need1 = need_of(v, w + 1);
+                    if (w < B) prefetch((uint32_t)d.w, w);
+                    SliceCount a, b;
+                    a.clear();
+                    b.clear();
+                    gather(list, 0, count, 8, w, a, b);
+                    if (d.z <= 255) {
+                        pull_apply_own(p, v, (uint32_t)d.w, w, need0, need1, a, b, n_up, act0, act1);
+                    } else {
+                        if (need0) act0 = pull_apply_shared(p, v, (uint32_t)d.w, w, need0, a, n_up);
+                        if (need1) act1 = pull_apply_shared(p, v, (uint32_t)d.w, w + 1, need1, b, n_up);
+                    }
+                }
+                record(v, ch, l == 0, (__ballot_sync(kFull, act0 != 0ull) & seg_mask) >> (seg * LN),
+                       (__ballot_sync(kFull, act1 != 0ull) & seg_mask) >> (seg * LN));
+            }
+            __syncwarp();
+        }
+        d = dn;
+    }
+    if (lb.n) lb.flush(p);
+    count_add(p, C_EDGES, n_edges);
+    count_add(p, C_WCHECKS, n_wc);
+    count_add(p, C_UPDATES, n_up);
+}
+
+// Whether the LT step whose frontier makes `checks` (edge, word) checks pulls.  A push step costs its
+// checks; a pull step the scan of all m in-edges and, for every in-edge from the frontier, a row of all
+// B words whether they carry bits or not.  Measured on GB300 (ms per call, push only / pull above
+// checks = m / 3 m / 6 m): R-MAT-21, B = 16: 384 / 154 / 160 / 187; B = 64: 1,470 / 484 / 455 / 446;
+// B = 1: 51.1 / 50.8 (52.1 above 0.3 m); BA 100k, B = 157: 54.7 / 37.8 / 35.4 / 33.8; B = 16: 8.5 / 6.65 / 6.8.
+__host__ __device__ __forceinline__ bool lt_pull_pays(unsigned long long checks, int64_t m, int32_t B) {
+    return checks * 12ull > (unsigned long long)m * (unsigned long long)(B > 12 ? B : 12);
+}
+
 // ---------------------------------------------------------------- device step loop
 // Start of a pass in graph mode: the seed step (-1) with a fresh stamp.
 __global__ void k_pass_begin(Params p) {
@@ -1125,7 +1505,7 @@ __global__ void k_pass_begin(Params p) {
 // stop at an empty frontier, the level cap or the time limit (timeout_ns > 0, measured on the GPU's
 // global timer from the call's first step), else set up the next step.
 __global__ void k_ctl(Params p, cudaGraphConditionalHandle h, int32_t first, int32_t max_levels, int32_t may_pull,
-                      int32_t pull_always, int32_t permille, int64_t m, int32_t tau,
+                      int32_t lt, int32_t pull_always, int32_t permille, int64_t m, int32_t tau,
                       unsigned long long timeout_ns) {
     Ctl *c = p.ctl;
     const unsigned long long now = global_ns();
@@ -1134,6 +1514,7 @@ __global__ void k_ctl(Params p, cudaGraphConditionalHandle h, int32_t first, int
     const bool odd = (L & 1) != 0;
     const int32_t *cnt = odd ? p.fr[1].cnt : p.fr[0].cnt;
     const int32_t slots = cnt[1], items = cnt[2], fedges = cnt[3];
+    const unsigned long long checks = *(const unsigned long long *)(cnt + 4);
     const int32_t waiting = p.lcnt[odd ? 1 : 0];
     c->slots += (unsigned long long)slots;
     c->items += (unsigned long long)items;
@@ -1151,13 +1532,14 @@ __global__ void k_ctl(Params p, cudaGraphConditionalHandle h, int32_t first, int
     }
     if (go) {
         int32_t *ncnt = odd ? p.fr[0].cnt : p.fr[1].cnt;
-        ncnt[0] = ncnt[1] = ncnt[2] = ncnt[3] = 0;
+        for (int i = 0; i < kCnt; ++i) ncnt[i] = 0;
         p.lcnt[odd ? 0 : 1] = 0;
         c->level = L;
         c->stamp += 1u;
         c->force = items == 0 ? 1 : 0;
         c->pull = (may_pull && items > 0 && tau == 0 &&
-                   (pull_always || (int64_t)fedges * 1000 > (int64_t)permille * m))
+                   (pull_always || (lt ? lt_pull_pays(checks, m, p.B)
+                                       : (int64_t)fedges * 1000 > (int64_t)permille * m)))
                       ? 1
                       : 0;
         c->levels += 1ull;
@@ -1382,12 +1764,15 @@ static cnd_status run_items(int model, const cnd_graph_dev &G, const char *fn, s
     // bytes per word column: vis, nxt, two pair pools (+ LT accumulators or counter planes)
     const double per_word = (double)n * (2 * 8 + 2 * 10 + (model == 1 && !lt_cnt ? 256 : 0)) +
                             (lt_cnt ? 8.0 * (double)G.lt_planes : 0.0);
-    // pulling (IC) happens only when asked for: by direction, or by a switch threshold
-    const bool may_pull = model == 0 && G.m > 0 &&
-                          (o.direction == CND_DIR_PULL || (o.direction == CND_DIR_AUTO && o.pull_permille > 0));
+    // IC pulls only when asked to: by direction, or by a switch threshold; LT in the counting form
+    // chooses per step (lt_pull_pays)
+    const bool lt_pull = lt_cnt && G.m > 0 && o.direction != CND_DIR_PUSH && o.defer_bits == 0;
+    const bool ic_pull = model == 0 && G.m > 0 &&
+                         (o.direction == CND_DIR_PULL || (o.direction == CND_DIR_AUTO && o.pull_permille > 0));
+    const bool may_pull = ic_pull || lt_pull;
     int64_t bmax = o.word_bits ? o.word_bits / 64 : kMaxB;
     bmax = std::min<int64_t>(bmax, std::max<int64_t>(1, (int64_t)(budget / per_word)));
-    bmax = std::min<int64_t>(bmax, may_pull ? kPullMaxB : kMaxB);
+    bmax = std::min<int64_t>(bmax, ic_pull ? kPullMaxB : kMaxB);
     bmax = std::min<int64_t>(bmax, std::max<int64_t>(1, (int64_t)0x7FFFFFFF / std::max(n, 1)));
     const int64_t n_pass = (total_words + bmax - 1) / bmax;
     const int B = (int)((total_words + n_pass - 1) / n_pass);
@@ -1517,15 +1902,27 @@ static cnd_status run_items(int model, const cnd_graph_dev &G, const char *fn, s
         CND_CUDA_TRY(W.alloc(&P.acc, nB * 64));
         CND_CUDA_TRY(W.alloc(&P.cvt, (size_t)n * nq));
     }
-    // pull direction (IC only): node-indexed frontier and frontier-node bitmap
+    // pull direction: node-indexed frontier and frontier-node bitmap
     const int permille = o.pull_permille > 0 ? o.pull_permille : kPullPermille;
     if (may_pull) {
-        CND_CUDA_TRY(W.alloc(&P.fdense, nB));
+        // LT: rows of an even number of words, a zero row behind the last, and room for a segment to
+        // read past the end of a row
+        P.fstride = lt_pull ? (B + 1) & ~1 : B;
+        const size_t n_fd = lt_pull ? ((size_t)n + 1) * (size_t)P.fstride + 64 : nB;
+        CND_CUDA_TRY(W.alloc(&P.fdense, n_fd));
+        if (lt_pull) {
+            const size_t zero = (size_t)n * (size_t)P.fstride;
+            CND_CUDA_TRY(cudaMemsetAsync(P.fdense + zero, 0, sizeof(uint64_t) * (n_fd - zero), st));
+        }
         CND_CUDA_TRY(W.alloc(&P.fbits, (size_t)(n + 31) / 32));
-        CND_CUDA_TRY(cudaMemsetAsync(P.fdense, 0, sizeof(uint64_t) * nB, st));
+        if (ic_pull) CND_CUDA_TRY(cudaMemsetAsync(P.fdense, 0, sizeof(uint64_t) * nB, st));
         CND_CUDA_TRY(cudaMemsetAsync(P.fbits, 0, sizeof(uint32_t) * ((size_t)(n + 31) / 32), st));
         P.in_row_ptr = G.in_row_ptr;
         P.in_edge = G.in_edge;
+        P.lt_in_src = G.lt_in_src;
+        P.lt_items = G.lt_pull_items;
+        P.n_lt_items = G.n_lt_pull_items;
+        P.n_lt_long = G.n_lt_long;
     }
     for (int i = 0; i < 2; ++i) {
         CND_CUDA_TRY(W.alloc(&fr[i].node, (size_t)n));
@@ -1534,7 +1931,7 @@ static cnd_status run_items(int model, const cnd_graph_dev &G, const char *fn, s
         CND_CUDA_TRY(W.alloc(&fr[i].pw, nB));
         CND_CUDA_TRY(W.alloc(&fr[i].pb, nB));
         CND_CUDA_TRY(W.alloc(&fr[i].work, work_cap));
-        CND_CUDA_TRY(W.alloc(&fr[i].cnt, 4));
+        CND_CUDA_TRY(W.alloc(&fr[i].cnt, kCnt));
     }
     P.ctr = d_ctr;
     if (S) {
@@ -1545,7 +1942,7 @@ static cnd_status run_items(int model, const cnd_graph_dev &G, const char *fn, s
     CND_CUDA_TRY(cudaMemsetAsync(P.mark, 0xFF, sizeof(uint32_t) * (size_t)n, st));
     CND_CUDA_TRY(cudaMemsetAsync(P.nxt, 0, sizeof(uint64_t) * nB, st));
     CND_CUDA_TRY(cudaMemsetAsync(P.dmask, 0, sizeof(uint64_t) * (size_t)n * nq, st));
-    if (!t_pinned.h) CND_CUDA_TRY(cudaMallocHost(&t_pinned.h, 6 * sizeof(int32_t)));
+    if (!t_pinned.h) CND_CUDA_TRY(cudaMallocHost(&t_pinned.h, 8 * sizeof(int32_t)));
     int32_t *hcnt = t_pinned.h;
 
     // a pass whose columns share one key takes it as launch parameters
@@ -1566,9 +1963,13 @@ static cnd_status run_items(int model, const cnd_graph_dev &G, const char *fn, s
     const int init_blocks = G.num_sms * resident_blocks(k_init_uk);
     const void *k_seedfin = nq <= kCollectNq ? k_col : (const void *)k_finalize<1, false>;
     const int push_blocks = G.num_sms * resident_blocks(k_push_uk);
-    const void *k_pull_pw = (const void *)k_pull_ic<true>, *k_pull_uk = (const void *)k_pull_ic<false>;
+    const void *k_pull_fn_lt = B <= 16 ? (const void *)k_pull_lt<8> : (const void *)k_pull_lt<16>;
+    const void *k_pull_pw = model == 0 ? (const void *)k_pull_ic<true> : k_pull_fn_lt;
+    const void *k_pull_uk = model == 0 ? (const void *)k_pull_ic<false> : k_pull_fn_lt;
+    const void *k_set = model == 0 ? (const void *)k_frontier_dense<true> : (const void *)k_frontier_rows<true>;
+    const void *k_clear = model == 0 ? (const void *)k_frontier_dense<false> : (const void *)k_frontier_rows<false>;
     const int pull_blocks = G.num_sms * resident_blocks(k_pull_uk);
-    const int dense_blocks = G.num_sms * resident_blocks((const void *)k_frontier_dense<true>);
+    const int dense_blocks = G.num_sms * resident_blocks(k_set);
     const int fin_blocks = G.num_sms * resident_blocks(k_fin_uk);
     const int seed_blocks = G.num_sms * resident_blocks(k_seedfin);
     uint32_t stamp = 0;
@@ -1603,7 +2004,7 @@ static cnd_status run_items(int model, const cnd_graph_dev &G, const char *fn, s
 
         // step 0: seeds (finalized from list 1 like an IC step; nothing waits)
         int cur = 0;
-        CND_CUDA_TRY(cudaMemsetAsync(fr[cur].cnt, 0, 4 * sizeof(int32_t), st));
+        CND_CUDA_TRY(cudaMemsetAsync(fr[cur].cnt, 0, kCnt * sizeof(int32_t), st));
         CND_CUDA_TRY(cudaMemsetAsync(d_lcnt, 0, 2 * sizeof(int32_t), st));
         P.out = fr[cur];
         P.lin = lists[1];
@@ -1619,15 +2020,17 @@ static cnd_status run_items(int model, const cnd_graph_dev &G, const char *fn, s
         launches += 2;
         P.force = 0;
         for (int L = 0;; ++L) {
-            CND_CUDA_TRY(cudaMemcpyAsync(hcnt, fr[cur].cnt, 4 * sizeof(int32_t), cudaMemcpyDeviceToHost, st));
-            CND_CUDA_TRY(cudaMemcpyAsync(hcnt + 4, d_lcnt + (L & 1), sizeof(int32_t), cudaMemcpyDeviceToHost, st));
+            CND_CUDA_TRY(cudaMemcpyAsync(hcnt, fr[cur].cnt, kCnt * sizeof(int32_t), cudaMemcpyDeviceToHost, st));
+            CND_CUDA_TRY(cudaMemcpyAsync(hcnt + kCnt, d_lcnt + (L & 1), sizeof(int32_t), cudaMemcpyDeviceToHost, st));
             CND_CUDA_TRY(cudaStreamSynchronize(st));
             if (timing) {
                 const cnd_status ts = collect_timing();
                 if (ts != CND_OK) return ts;
             }
             // slots / work items of step L's frontier; nodes whose words wait
-            const int32_t slots = hcnt[1], n_items_w = hcnt[2], front_edges = hcnt[3], waiting = hcnt[4];
+            const int32_t slots = hcnt[1], n_items_w = hcnt[2], front_edges = hcnt[3], waiting = hcnt[kCnt];
+            unsigned long long checks;
+            memcpy(&checks, hcnt + 4, sizeof(checks));
             if (S) {
                 S->frontier_slots += slots;
                 S->work_items += n_items_w;
@@ -1647,7 +2050,7 @@ static cnd_status run_items(int model, const cnd_graph_dev &G, const char *fn, s
                 }
             }
             const int nx = cur ^ 1;
-            CND_CUDA_TRY(cudaMemsetAsync(fr[nx].cnt, 0, 4 * sizeof(int32_t), st));
+            CND_CUDA_TRY(cudaMemsetAsync(fr[nx].cnt, 0, kCnt * sizeof(int32_t), st));
             CND_CUDA_TRY(cudaMemsetAsync(d_lcnt + ((L + 1) & 1), 0, sizeof(int32_t), st));
             P.in = fr[cur];
             P.out = fr[nx];
@@ -1662,12 +2065,13 @@ static cnd_status run_items(int model, const cnd_graph_dev &G, const char *fn, s
             // direction: pull when the frontier's out-edges are a large share of m
             const bool pull = may_pull && n_items_w > 0 && P.tau == 0 &&
                               (o.direction == CND_DIR_PULL ||
-                               (int64_t)front_edges * 1000 > (int64_t)permille * (int64_t)G.m);
+                               (lt_pull ? lt_pull_pays(checks, G.m, B)
+                                        : (int64_t)front_edges * 1000 > (int64_t)permille * (int64_t)G.m));
             if (timing) CND_CUDA_TRY(cudaEventRecord(ev.e[0], st));
             if (pull) {
-                CND_CUDA_TRY(launch((const void *)k_frontier_dense<true>, dense_blocks, st, P));
+                CND_CUDA_TRY(launch(k_set, dense_blocks, st, P));
                 CND_CUDA_TRY(launch(pw ? k_pull_pw : k_pull_uk, pull_blocks, st, P));
-                CND_CUDA_TRY(launch((const void *)k_frontier_dense<false>, dense_blocks, st, P));
+                CND_CUDA_TRY(launch(k_clear, dense_blocks, st, P));
                 launches += 3;
                 if (S) S->pull_steps += 1;
             } else if (n_items_w > 0) {
@@ -1774,13 +2178,14 @@ static cnd_status run_items(int model, const cnd_graph_dev &G, const char *fn, s
                 CND_CUDA_TRY(cudaMemsetAsync(P.acc, 0, sizeof(uint32_t) * nB * 64, cs));
                 CND_CUDA_TRY(cudaMemsetAsync(P.cvt, 0, sizeof(uint64_t) * (size_t)n * nq, cs));
             }
-            CND_CUDA_TRY(cudaMemsetAsync(fr[0].cnt, 0, 4 * sizeof(int32_t), cs));
+            CND_CUDA_TRY(cudaMemsetAsync(fr[0].cnt, 0, kCnt * sizeof(int32_t), cs));
             CND_CUDA_TRY(cudaMemsetAsync(d_lcnt, 0, 2 * sizeof(int32_t), cs));
             k_pass_begin<<<1, 1, 0, cs>>>(Q);
             k_seed<<<std::max<int>(1, (int)ps.size()), 128, 0, cs>>>(Q, pass_segs(pass), (int32_t)ps.size(),
                                                                       seeds_dev, d_bad);
             CND_CUDA_TRY(launch(k_seedfin, seed_blocks, cs, Q));
-            k_ctl<<<1, 1, 0, cs>>>(Q, h, 1, o.max_levels, may_pull ? 1 : 0, o.direction == CND_DIR_PULL ? 1 : 0,
+            k_ctl<<<1, 1, 0, cs>>>(Q, h, 1, o.max_levels, may_pull ? 1 : 0, lt_pull ? 1 : 0,
+                                   o.direction == CND_DIR_PULL ? 1 : 0,
                                    permille, (int64_t)G.m, P.tau, timeout_ns);
             CND_CUDA_TRY(cudaGetLastError());
             CND_CUDA_TRY(cap_end(&tail));
@@ -1795,13 +2200,14 @@ static cnd_status run_items(int model, const cnd_graph_dev &G, const char *fn, s
             cudaGraph_t body = cp.conditional.phGraph_out[0];
             CND_CUDA_TRY(cap_begin(body, {}));
             if (may_pull) {
-                CND_CUDA_TRY(launch((const void *)k_frontier_dense<true>, dense_blocks, cs, Q));
+                CND_CUDA_TRY(launch(k_set, dense_blocks, cs, Q));
                 CND_CUDA_TRY(launch(pw ? k_pull_pw : k_pull_uk, pull_blocks, cs, Q));
-                CND_CUDA_TRY(launch((const void *)k_frontier_dense<false>, dense_blocks, cs, Q));
+                CND_CUDA_TRY(launch(k_clear, dense_blocks, cs, Q));
             }
             CND_CUDA_TRY(launch(pw ? k_push_pw : k_push_uk, push_blocks, cs, Q));
             CND_CUDA_TRY(launch(pw ? k_fin_pw : k_fin_uk, fin_blocks, cs, Q));
-            k_ctl<<<1, 1, 0, cs>>>(Q, h, 0, o.max_levels, may_pull ? 1 : 0, o.direction == CND_DIR_PULL ? 1 : 0,
+            k_ctl<<<1, 1, 0, cs>>>(Q, h, 0, o.max_levels, may_pull ? 1 : 0, lt_pull ? 1 : 0,
+                                   o.direction == CND_DIR_PULL ? 1 : 0,
                                    permille, (int64_t)G.m, P.tau, timeout_ns);
             CND_CUDA_TRY(cudaGetLastError());
             CND_CUDA_TRY(cap_end(nullptr));
@@ -2362,7 +2768,7 @@ static size_t place_static(Arena &a, Params &P, Frontier (&fr)[2], int32_t n, in
         fr[i].pw = a.take<uint16_t>(nB);
         fr[i].pb = a.take<uint64_t>(nB);
         fr[i].work = a.take<int2>(work_cap);
-        fr[i].cnt = a.take<int32_t>(4);
+        fr[i].cnt = a.take<int32_t>(kCnt);
     }
     return a.used;
 }
@@ -2455,7 +2861,7 @@ static cnd_status simulate_noalloc(const cnd_graph *g, const int32_t *seeds, int
         int64_t *wout = (int64_t *)(desc + B);
         const int64_t *d_wout = (const int64_t *)(d_valid + B);
         const SeedSeg *d_seg = (const SeedSeg *)(d_valid + 2 * B);
-        int32_t hcnt[4];
+        int32_t hcnt[kCnt];
         uint32_t stamp = 0;
         for (int64_t pass = 0; pass < n_pass; ++pass) {
             const int64_t w0 = pass * B;
@@ -2471,7 +2877,7 @@ static cnd_status simulate_noalloc(const cnd_graph *g, const int32_t *seeds, int
             CND_CUDA_TRY(cudaMemsetAsync(P.vis, 0, sizeof(uint64_t) * nB, st));
             P.g_base = (uint64_t)(64 * w0) >> 2;
             int cur = 0;
-            CND_CUDA_TRY(cudaMemsetAsync(fr[cur].cnt, 0, 4 * sizeof(int32_t), st));
+            CND_CUDA_TRY(cudaMemsetAsync(fr[cur].cnt, 0, kCnt * sizeof(int32_t), st));
             CND_CUDA_TRY(cudaMemsetAsync(P.lin_cnt, 0, 2 * sizeof(int32_t), st));
             P.out = fr[cur];
             P.stamp = stamp++;
@@ -2482,11 +2888,11 @@ static cnd_status simulate_noalloc(const cnd_graph *g, const int32_t *seeds, int
             CND_CUDA_TRY(launch(k_fin_fn, fin_blocks, st, P));
             P.force = 0;
             for (;;) {
-                CND_CUDA_TRY(cudaMemcpyAsync(hcnt, fr[cur].cnt, 4 * sizeof(int32_t), cudaMemcpyDeviceToHost, st));
+                CND_CUDA_TRY(cudaMemcpyAsync(hcnt, fr[cur].cnt, kCnt * sizeof(int32_t), cudaMemcpyDeviceToHost, st));
                 CND_CUDA_TRY(cudaStreamSynchronize(st));
                 if (hcnt[1] == 0 || hcnt[2] == 0) break;
                 const int nx = cur ^ 1;
-                CND_CUDA_TRY(cudaMemsetAsync(fr[nx].cnt, 0, 4 * sizeof(int32_t), st));
+                CND_CUDA_TRY(cudaMemsetAsync(fr[nx].cnt, 0, kCnt * sizeof(int32_t), st));
                 CND_CUDA_TRY(cudaMemsetAsync(P.lin_cnt, 0, sizeof(int32_t), st));
                 P.in = fr[cur];
                 P.out = fr[nx];

@@ -1,0 +1,97 @@
+"""The LT pull step (counting form) against the oracle and the push step: in-rows around the lengths at
+which they change hands or are split, zero-weight in-edges, pass widths around the words a segment owns,
+seeds and saturated targets, several passes, the CUDA-graph loop, batches and level caps."""
+import numpy as np
+import pytest
+
+import oracle
+import paper_2404_17059_gb300 as P
+from paper_2404_17059_gb300 import inputs as I
+
+pytestmark = pytest.mark.gpu
+LC = 24
+IN_DEGREES = [1, 2, 7, 8, 9, 63, 64, 65, 96, 254, 255, 256, 257, 300, 510, 511, 766, 1500]
+
+
+def _targets():
+    """One target per in-degree, fed by 1,600 sources that the seeds reach over chains of two steps; some
+    in-edges of weight zero; the targets feed each other and back into the sources."""
+    n_src, rng = 1600, np.random.default_rng(3)
+    k = len(IN_DEGREES)
+    n = n_src + k
+    src, dst = [], []
+    for i, d in enumerate(IN_DEGREES):
+        src.append(rng.permutation(n_src)[:d])
+        dst.append(np.full(d, n_src + i))
+    for _ in range(3):  # sources among themselves
+        src.append(rng.permutation(n_src))
+        dst.append(rng.permutation(n_src))
+    src.append(np.repeat(np.arange(n_src, n), 40))  # targets back into sources and each other
+    dst.append(rng.integers(0, n, 40 * k))
+    g = I.csr_from_edges(n, np.concatenate(src), np.concatenate(dst))
+    w = I.lt_weighted_cascade(g).copy()
+    w[rng.random(g.m) < 0.05] = 0  # the others of a node stay equal
+    return g, w
+
+
+@pytest.fixture(scope="module")
+def graph():
+    g, w = _targets()
+    return g, w, P.cnd_graph_create(g.n, g.row_ptr, g.col, None, w)
+
+
+def _run(G, seeds, T, rng, **kw):
+    return P.cnd_lt_simulate_ex(G, seeds, T, rng, edge_checks=True, level_counts_len=LC, stats=2, **kw)
+
+
+def _same(a, b):
+    assert np.array_equal(a.spread, b.spread)
+    assert np.array_equal(a.node_count, b.node_count)
+    assert a.edge_checks == b.edge_checks
+    assert np.array_equal(a.level_counts, b.level_counts)
+
+
+@pytest.mark.parametrize("words", [1, 2, 15, 16, 17, 31, 32, 33, 65])
+def test_pull_widths_match_oracle(graph, words):
+    g, w, G = graph
+    T = 64 * words - 5
+    seeds = I.uniform_seeds(g.n, 300, words)
+    b = oracle.simulate_threads("lt", g, seeds, T, 7, lt_weight=w, level_counts_len=LC)
+    pull = _run(G, seeds, T, 7, direction="pull")
+    assert pull.stats["pull_steps"] == pull.stats["levels"] > 2 and pull.stats["lt_counters"] == 1
+    push = _run(G, seeds, T, 7, direction="push")
+    assert push.stats["pull_steps"] == 0
+    for a in (pull, push, _run(G, seeds, T, 7), _run(G, seeds, T, 7, direction="pull", graph=1)):
+        _same(a, b)
+    _same(_run(G, seeds, T, 7, direction="pull", word_bits=64 * ((words + 1) // 2)), b)
+
+
+def test_pull_caps_offsets_and_seed_sets(graph):
+    g, w, G = graph
+    for seeds in ([], [0], list(range(1600, g.n)), list(range(0, g.n, 2))):
+        for kw in ({}, {"max_levels": 1}, {"max_levels": 3}, {"first_trial": 6400}):
+            b = oracle.simulate_threads("lt", g, seeds, 200, 5, lt_weight=w, level_counts_len=LC, **kw)
+            _same(_run(G, seeds, 200, 5, direction="pull", **kw), b)
+
+
+def test_pull_batches(graph):
+    g, w, G = graph
+    off, seeds, _, keys = I.batch_items(g.n, 37, 1, 200, (1,), graph_seed=2)
+    trials = np.array([(64, 0, 130, 1000)[i % 4] for i in range(37)], dtype=np.int32)
+    out = [P.cnd_lt_simulate_batch(G, off, seeds, trials, keys, node_count=True, edge_checks=True,
+                                   level_counts_len=LC, direction=d, word_bits=wb)
+           for d, wb in (("push", 0), ("pull", 0), ("auto", 64 * 40), ("pull", 64 * 7))]
+    for a in out[1:]:
+        _same(a, out[0])
+
+
+def test_dense_frontier_pulls_by_itself():
+    g = I.rmat(15, 16 << 15, graph_seed=4)
+    w = I.lt_weighted_cascade(g)
+    G = P.cnd_graph_create(g.n, g.row_ptr, g.col, None, w)
+    seeds = I.top_degree_seeds(g, 100)
+    push = _run(G, seeds, 1000, 2, direction="push")
+    for graph in (0, 1):
+        a = _run(G, seeds, 1000, 2, graph=graph)
+        assert 0 < a.stats["pull_steps"] < a.stats["levels"]
+        _same(a, push)
