@@ -65,6 +65,13 @@ constexpr int kPushMinBlocks = 8;
 constexpr int kStageB = 64;  // pairs of a push work item staged in shared memory (more: read from the pool)
 constexpr int kPullMaxB = 256;  // words per node the pull kernel keeps in registers
 constexpr int kTasks = 256;  // (edge, pair) tasks per push work item
+// ... of a slot of more than 32 pairs in an IC pass of more than 256 words on a graph of kWideNodes nodes
+// and more: its lanes go over the item's edges with the pairs they hold, so more edges per item pay
+// while a step has items enough for all warps (16 seed sets on R-MAT-20, 424 words: 515 / 482 / 472 ms per
+// call at 256 / 1,024 / 2,048 tasks; BA 100k, 157 words, few slots per step: 19.7 / 20.6 / 22.3 ms;
+// Watts-Strogatz 10k p = 0.1, 65,536 trials, 1,024 words: 3.60 / - / 4.03 ms)
+constexpr int kWideTasks = 2048;
+constexpr int kWideNodes = 65536;
 // AUTO without pull_permille: push only -- the pull step measured 1.3x to 3.7x
 // slower than push on every GB300 workload here (hub in-rows scanned by one warp)
 constexpr int kPullPermille = 1001;
@@ -105,6 +112,7 @@ __device__ __forceinline__ unsigned long long global_ns() {
 struct Params {
     int32_t n, B, nq;
     int32_t chunk;             // > 0: fixed edges per work item
+    int32_t wide;              // tasks per work item of a slot with more than 32 pairs
     const int32_t *row_ptr;
     const uint2 *edge;         // {col, IC threshold} or {col, LT weight}
     uint64_t *vis, *nxt, *dmask;
@@ -185,7 +193,7 @@ __device__ __forceinline__ void add_level_count(const Params &p, unsigned long l
 
 // Edges per work item for a slot with k pairs.
 __device__ __forceinline__ int edges_per_item(const Params &p, int k) {
-    return p.chunk > 0 ? p.chunk : max(1, kTasks / max(k, 1));
+    return p.chunk > 0 ? p.chunk : max(1, (k > 32 ? p.wide : kTasks) / max(k, 1));
 }
 
 // t / k for t < 2^32 / k (k <= kMaxB): multiply by ceil-ish reciprocal.
@@ -752,37 +760,183 @@ __global__ void __launch_bounds__(kBlock) k_lt_init(Params p) {
 }
 
 // ---------------------------------------------------------------- push
-// One warp per work item: the item's (edge, pair) tasks are spread over the
-// lanes, task t = (edge t / k, pair t % k).
-// Nibble j of x non-zero -> bit j of the result (16 bits).
-__device__ __forceinline__ uint32_t nibble_mask(uint64_t x) {
-    uint64_t m = (x | (x >> 1) | (x >> 2) | (x >> 3)) & 0x1111111111111111ull;
-    m = (m | (m >> 3)) & 0x0303030303030303ull;
-    m = (m | (m >> 6)) & 0x000F000F000F000Full;
-    m = (m | (m >> 12)) & 0x000000FF000000FFull;
-    m = (m | (m >> 24)) & 0xFFFFull;
-    return (uint32_t)m;
+// ---------------------------------------------------------------- push (IC)
+// Nibbles of x that are not zero, as bits: nibble j of the low half at 4 j, of the high half at 4 j + 1.
+__device__ __forceinline__ uint32_t nibble_bits(uint64_t x) {
+    uint32_t lo = (uint32_t)x, hi = (uint32_t)(x >> 32);
+    lo |= lo >> 1;
+    hi |= hi >> 1;
+    lo |= lo >> 2;
+    hi |= hi >> 2;
+    return (lo & 0x11111111u) | ((hi & 0x11111111u) << 1);
 }
 
-// Per-warp queue that spreads the Philox calls of 32 IC tasks evenly over the
-// lanes: a task with many 4-trial blocks to draw no longer stalls the warp.
-struct DrawQueue {
-    uint16_t q[32 * 16];  // (lane << 4) | block
-    uint8_t res[32 * 16]; // live bits of the block's four trials
-    uint64_t g0[32];
-    uint32_t e[32], thr[32];
-    uint16_t w[32];
+// Per-warp state of the IC push: the pairs the lanes hold, the edges they are at, the queued coin blocks
+// and the live coins.
+template <bool PERWORD>
+struct PushIc {
+    uint16_t q[32 * 16];             // (lane << 5) | bit of nibble_bits
+    uint2 edge[32];                  // {edge id, IC threshold}
+    uint32_t live[32][2];
+    uint4 key[PERWORD ? 32 : 1];     // {trial block of bit 0 (64 bits), Philox key}
+    uint32_t g[PERWORD ? 1 : 32];    // 16 w: trial block of bit 0, less that of the pass
 };
 
+// IC push (k_push<0, PERWORD>).  A lane holds one (word, frontier bits) pair of the item's slot and goes
+// over the item's edges with it; a slot of k <= 16 pairs takes 32 / k edges at a time.  Per edge and
+// pair: c = f & ~vis_v[w]; the 4-trial blocks of c are queued and drawn by all lanes, one Philox block
+// each; drawing lanes or the rare live coins into their owner's word in shared memory.
+//
+// Bound by the ALU pipe and issue slots (ncu, R-MAT-20: 65 % issue active, not-selected the first stall;
+// 3.6 draws per check, each 20 multiplies and 20 three-input xors).  Holding pairs in lanes instead of
+// dealing (edge, pair) tasks to lanes takes the task division, the pair loads and the per-task trial
+// blocks and keys out of the inner loop; or-ing hits takes out the owners' loop that gathered results:
+// R-MAT-21, p = 0.01, 1,024 trials 51.7 -> 46.1 ms, 16 seed sets on R-MAT-20 518 -> 425 ms (with items of
+// kWideTasks; 470 with kTasks), BA 100k, 10,000 trials 16.9 -> 16.5 ms.  8 blocks per SM at 32
+// registers (6 at 40: R-MAT-21 48.2 -> 51.4 ms per call).
+template <bool PERWORD>
+__device__ __forceinline__ void push_ic(Params &p) {
+    __shared__ int32_t s_list[kWarps][64];
+    __shared__ __align__(16) PushIc<PERWORD> s_ic[kWarps];
+    const int lane = lane_id();
+    const int wid = threadIdx.x >> 5;
+    ListBuf lb{s_list[wid], 0};
+    PushIc<PERWORD> &ic = s_ic[wid];
+    const int n_work = p.in.cnt[2];
+    const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int n_warps = (gridDim.x * blockDim.x) >> 5;
+    const int B = p.B;
+    uint32_t n_edges = 0, n_fw = 0, n_wc = 0, n_dr = 0, n_up = 0;
+    ic.live[lane][0] = ic.live[lane][1] = 0u;
+    for (int wi = warp; wi < n_work; wi += n_warps) {
+        const int2 it = p.in.work[wi];
+        const int u = p.in.node[it.x];
+        const int off = p.in.poff[it.x];
+        const int k = p.in.pk[it.x];
+        const int row0 = p.row_ptr[u];
+        const int deg = p.row_ptr[u + 1] - row0;
+        const int e_begin = row0 + it.y;
+        const int e_end = e_begin + min(edges_per_item(p, k), deg - it.y);
+        // lanes hold pairs; with k <= 16 several edges at a time, sub-th edge of each group per lane
+        const int per = k >= 32 ? 1 : 32 / k;
+        const int sub = k >= 32 ? 0 : lane / k;
+        if (lane == 0) {
+            n_edges += e_end - e_begin;
+            n_fw += k;
+        }
+        for (int j0 = 0; j0 < k; j0 += 32) {
+            const int j = k >= 32 ? j0 + lane : lane - sub * k;
+            uint64_t f = 0;
+            int w = 0;
+            if (j < k && sub < per) {
+                f = p.in.pb[off + j];
+                w = (int)p.in.pw[off + j];
+            }
+            __syncwarp();
+            if (PERWORD) {
+                const uint64_t g0 = p.wg0[w];
+                const uint2 key = p.wkey[w];
+                ic.key[lane] = make_uint4((uint32_t)g0, (uint32_t)(g0 >> 32), key.x, key.y);
+            } else {
+                ic.g[lane] = 16u * (uint32_t)w;
+            }
+            const uint64_t *vis_w = p.vis + w;
+            for (int e0 = e_begin; e0 < e_end; e0 += per) {
+                const int e = e0 + sub;
+                uint64_t c = 0;
+                uint32_t thr = 0;
+                int v = 0;
+                if (f != 0ull && e < e_end) {
+                    const uint2 ed = __ldg(&p.edge[e]);
+                    v = (int)ed.x;
+                    thr = ed.y;
+                    if (thr != 0u) {
+                        ++n_wc;
+                        c = f & ~(uint64_t)__ldcg((const unsigned long long *)vis_w + (size_t)v * B);
+                    }
+                }
+                // coins: the 4-trial blocks of c are queued and drawn by all lanes
+                uint32_t rem = thr != kAlways ? nibble_bits(c) : 0u;
+                const int d = __popc(rem);
+                int at = d;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const int x = __shfl_up_sync(kFull, at, o);
+                    if (lane >= o) at += x;
+                }
+                const int D = __shfl_sync(kFull, at, 31);
+                uint64_t nb = c;
+                if (D > 0) {
+                    ic.edge[lane] = make_uint2((uint32_t)e, thr);
+                    uint16_t *q = ic.q + (at - d);
+                    while (rem) {
+                        *q++ = (uint16_t)((lane << 5) | (__ffs(rem) - 1));
+                        rem &= rem - 1u;
+                    }
+                    __syncwarp();
+                    for (int i = lane; i < D; i += 32) {
+                        const uint32_t ent = ic.q[i];
+                        const uint32_t o = ent >> 5, b = ent & 31u;
+                        const uint32_t jj = (b >> 2) | ((b & 1u) << 3);
+                        const uint2 ed = ic.edge[o];
+                        U4 r;
+                        if (PERWORD) {
+                            const uint4 kw = ic.key[o];
+                            const uint64_t g = (((uint64_t)kw.y << 32) | kw.x) + jj;
+                            r = philox4x32_10(ed.x, (uint32_t)g, 0u, (uint32_t)(g >> 32), kw.z, kw.w);
+                        } else {
+                            const uint64_t g = p.g_base + (ic.g[o] + jj);
+                            r = philox4x32_10(ed.x, (uint32_t)g, 0u, (uint32_t)(g >> 32), p.rk);
+                        }
+                        const uint32_t nib = (uint32_t)(r.x < ed.y) | ((uint32_t)(r.y < ed.y) << 1) |
+                                             ((uint32_t)(r.z < ed.y) << 2) | ((uint32_t)(r.w < ed.y) << 3);
+                        ++n_dr;
+                        if (nib) atomicOr(&ic.live[o][b & 1u], nib << (b & 28u));
+                    }
+                    __syncwarp();
+                    if (d) {
+                        const uint2 l = *reinterpret_cast<const uint2 *>(ic.live[lane]);
+                        *reinterpret_cast<uint2 *>(ic.live[lane]) = make_uint2(0u, 0u);
+                        nb = c & (((uint64_t)l.y << 32) | l.x);
+                    }
+                }
+                bool claimed = false;
+                if (nb) {
+                    // vis: a reduction without return (no round trip); bits another task of this
+                    // step has just set are or-ed again into nxt, which is idempotent
+                    const size_t idx = (size_t)v * B + w;
+                    atomicOr((unsigned long long *)p.vis + idx, (unsigned long long)nb);
+                    const uint64_t old = atomicOr((unsigned long long *)p.nxt + idx, (unsigned long long)nb);
+                    claimed = atomicExch(&p.mark[v], p.stamp) != p.stamp;
+                    mark_dirty(p, v, w, old);
+                    ++n_up;
+                }
+                lb.put(p, claimed, v);
+            }
+        }
+    }
+    if (lb.n) lb.flush(p);
+    count_add(p, C_EDGES, n_edges);
+    count_add(p, C_FWORDS, n_fw);
+    count_add(p, C_WCHECKS, n_wc);
+    count_add(p, C_DRAWS, n_dr);
+    count_add(p, C_UPDATES, n_up);
+}
+
+// LT push.  One warp per work item: the item's (edge, pair) tasks are spread over the lanes, task
+// t = (edge t / k, pair t % k).
 template <int MODEL, bool PERWORD>
 __global__ void __launch_bounds__(kBlock, kPushMinBlocks) k_push(Params p_) {
     Params p = p_;
     resolve(p);
     if (p.ctl && p.ctl->pull) return;  // graph mode: this step pulls
+    if constexpr (MODEL == 0) {
+        push_ic<PERWORD>(p);
+        return;
+    }
     __shared__ uint64_t s_b[kWarps][kStageB];
     __shared__ uint16_t s_w[kWarps][kStageB];
     __shared__ int32_t s_list[kWarps][64];
-    __shared__ DrawQueue s_dq[MODEL == 0 ? kWarps : 1];
     const int lane = lane_id();
     const int wid = threadIdx.x >> 5;
     ListBuf lb{s_list[wid], 0};
@@ -818,10 +972,6 @@ __global__ void __launch_bounds__(kBlock, kPushMinBlocks) k_push(Params p_) {
             const uint32_t t = t0 + lane;
             bool hit = false, claimed = false;  // claimed: this lane took mark[v] for the step
             int v = 0;
-            uint64_t ic_c = 0;
-            uint32_t ic_thr = 0;
-            int ic_e = 0, ic_w = 0, ic_v = 0;
-            size_t ic_idx = 0;
             if (t < T) {
                 const uint32_t el = div_by(t, (uint32_t)k, magic);
                 const int j = (int)(t - el * (uint32_t)k);
@@ -831,18 +981,7 @@ __global__ void __launch_bounds__(kBlock, kPushMinBlocks) k_push(Params p_) {
                 const int w = staged ? (int)s_w[wid][j] : (int)p.in.pw[off + j];
                 const uint64_t f = staged ? s_b[wid][j] : p.in.pb[off + j];
                 const size_t idx = (size_t)v * B + w;
-                if (MODEL == 0) {
-                    ic_c = 0;
-                    ic_thr = ed.y;
-                    ic_e = e;
-                    ic_w = w;
-                    ic_v = v;
-                    ic_idx = idx;
-                    if (ic_thr != 0u) {
-                        ++n_wc;
-                        ic_c = f & ~(uint64_t)__ldcg((const unsigned long long *)p.vis + idx);
-                    }
-                } else if (MODEL == 2) {
+                if (MODEL == 2) {
                     // counting form: add 1 to the counters of the trials of c (bit-sliced ripple
                     // carry, plane by plane, atomically); what carries out of the top plane
                     // activates (see k_lt_init)
@@ -920,75 +1059,6 @@ __global__ void __launch_bounds__(kBlock, kPushMinBlocks) k_push(Params p_) {
                         }
                     }
                 }
-            }
-            if (MODEL == 0) {
-                // coins: the 4-trial blocks of c that need a draw, queued and drawn
-                // by all lanes; then the live bits go to vis / nxt
-                DrawQueue &dq = s_dq[MODEL == 0 ? wid : 0];
-                const uint64_t need = (ic_thr != kAlways) ? ic_c : 0ull;
-                const uint32_t nm = nibble_mask(need);
-                const int d = __popc(nm);
-                int base = d;
-#pragma unroll
-                for (int o = 1; o < 32; o <<= 1) {
-                    const int x = __shfl_up_sync(kFull, base, o);
-                    if (lane >= o) base += x;
-                }
-                const int D = __shfl_sync(kFull, base, 31);
-                base -= d;
-                if (D > 0) {
-                    dq.g0[lane] = word_g0<PERWORD>(p, ic_w);
-                    dq.e[lane] = (uint32_t)ic_e;
-                    dq.thr[lane] = ic_thr;
-                    dq.w[lane] = (uint16_t)ic_w;
-                    {
-                        uint32_t mm = nm;
-                        int r = base;
-                        while (mm) {
-                            const int j = __ffs(mm) - 1;
-                            mm &= mm - 1;
-                            dq.q[r++] = (uint16_t)((lane << 4) | j);
-                        }
-                    }
-                    __syncwarp();
-                    for (int qi = lane; qi < D; qi += 32) {
-                        const uint32_t ent = dq.q[qi];
-                        const int o = (int)(ent >> 4), j = (int)(ent & 15u);
-                        const uint32_t th = dq.thr[o];
-                        const U4 r = draw<PERWORD>(p, dq.w[o], dq.e[o], dq.g0[o] + (uint64_t)j, 0u);
-                        dq.res[qi] = (uint8_t)((uint32_t)(r.x < th) | ((uint32_t)(r.y < th) << 1) |
-                                               ((uint32_t)(r.z < th) << 2) | ((uint32_t)(r.w < th) << 3));
-                        ++n_dr;
-                    }
-                    __syncwarp();
-                }
-                uint64_t nb = 0;
-                if (ic_c) {
-                    if (ic_thr == kAlways) {
-                        nb = ic_c;
-                    } else {
-                        uint64_t live = 0;
-                        uint32_t mm = nm;
-                        int r = base;
-                        while (mm) {
-                            const int j = __ffs(mm) - 1;
-                            mm &= mm - 1;
-                            live |= (uint64_t)dq.res[r++] << (4 * j);
-                        }
-                        nb = ic_c & live;
-                    }
-                }
-                if (nb) {
-                    // vis: a reduction without return (no round trip); bits another task of this
-                    // step has just set are or-ed again into nxt, which is idempotent
-                    atomicOr((unsigned long long *)p.vis + ic_idx, (unsigned long long)nb);
-                    const uint64_t old = atomicOr((unsigned long long *)p.nxt + ic_idx, (unsigned long long)nb);
-                    claimed = atomicExch(&p.mark[ic_v], p.stamp) != p.stamp;
-                    mark_dirty(p, ic_v, ic_w, old);
-                    ++n_up;
-                    hit = true;
-                }
-                __syncwarp();
             }
             if (MODEL == 1) lb.add(p, hit, v);
             else lb.put(p, claimed, v);
@@ -1812,6 +1882,7 @@ static cnd_status run_items(int model, const cnd_graph_dev &G, const char *fn, s
     P.B = B;
     P.nq = nq;
     P.chunk = chunk;
+    P.wide = model == 0 && B > 256 && n >= kWideNodes ? kWideTasks : kTasks;
     P.row_ptr = G.row_ptr;
     P.edge = edge;
     P.rk = round_keys(items[0].key);
@@ -2836,6 +2907,7 @@ static cnd_status simulate_noalloc(const cnd_graph *g, const int32_t *seeds, int
         P.B = B;
         P.nq = nq;
         P.chunk = 0;
+        P.wide = kTasks;
         P.tau = 0;
         P.max_wait = 0;
         P.force = 0;
