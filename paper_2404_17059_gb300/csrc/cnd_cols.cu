@@ -483,13 +483,18 @@ bool column_shape(int model, const cnd_graph_dev &G, int per_sm, ColShape &c) {
 }  // namespace
 
 // Calls that run here.  Options that choose a form of the pass engine (width, work items, direction,
-// deferral, statistics, 32-bit sums) get the pass engine.  IC calls of more than kWideTrials trials on
-// graphs of which an SM holds fewer than four columns (n > about 5,500) get it too: with that many
-// trials its words are full, and one check of 64 trials costs it less than two of 32 cost here.
+// deferral, statistics, 32-bit sums) get the pass engine.  So do IC calls of many trials on the larger
+// graphs: with that many the pass engine's words are full, and one check of 64 trials costs it less than
+// two of 32 cost here.  The line is kWideTrials where an SM holds fewer than four columns (n > about
+// 5,500) and there are hub rows (kHub edges and more: one block's work), four times that where it holds
+// one column (n > about 12,000) and there are none.
 // Measured against the pass engine (GB300; host step loop, its default):
 //   1,000 trials:  G(1000, 10000) p = 0.1 1,267 -> 131 us; Watts-Strogatz 10k U[0, 1] 2,595 -> 756 us;
 //                  BA 13k WC 2,067 -> 481 us; BA 20k U[0, 1] 867 -> 683 us; R-MAT 14 p = 0.1 923 -> 789 us
 //   20,000 trials: BA 13k U[0, 1] 3.10 -> 3.72 ms, R-MAT 13 p = 0.1 2.88 -> 3.47 ms (BA 13k WC 7.4 -> 5.5 ms)
+//   65,536 trials: Watts-Strogatz 10k p = 0.1 3.60 -> 1.27 ms, U[0, 1] 30.5 -> 20.0 ms
+//   no hub rows:   G(20000, 200000) p = 0.1 10,000 trials 8.6 -> 2.5 ms; U[0, 1] 10,000 / 30,000 / 65,536 trials
+//                  3.54 -> 3.55 / 8.4 -> 9.5 / 18.7 -> 19.0 ms
 //   LT, any:       BA 5k 1,000 trials 2,395 -> 370 us, 65,536 trials 20.1 -> 8.1 ms
 constexpr int64_t kWideTrials = 4096;
 
@@ -499,7 +504,8 @@ bool columns_fit(int model, const cnd_graph_dev &G, const cnd_sim_opts &o, int64
         return false;
     ColShape c;
     if (!column_shape(model, G, 1, c)) return false;
-    return model == 1 || trials <= kWideTrials || column_shape(model, G, 4, c);
+    if (model == 1 || trials <= kWideTrials || column_shape(model, G, 4, c)) return true;
+    return G.max_out_degree < kHub && (trials <= 4 * kWideTrials || column_shape(model, G, 2, c));
 }
 
 cnd_status run_columns(int model, const cnd_graph_dev &G, const std::vector<ItemDesc> &items, const int32_t *seeds_dev,

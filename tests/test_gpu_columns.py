@@ -82,6 +82,17 @@ def test_long_rows(model):
     _check(model, g, G, list(range(80)), 45, 8, p, w)
 
 
+def test_many_trials_without_hub_rows():
+    g = I.watts_strogatz(9000, 6, 0.05, graph_seed=3)
+    p, w = _weights(g)
+    G = P.cnd_graph_create(g.n, g.row_ptr, g.col, p, w)
+    seeds = I.uniform_seeds(g.n, 5, 3)
+    a = _sim("ic", G, seeds, 20_001, 2)
+    b = _sim("ic", G, seeds, 20_001, 2, word_bits=64 * 128)
+    assert np.array_equal(a.spread, b.spread) and np.array_equal(a.node_count, b.node_count)
+    assert a.edge_checks == b.edge_checks and np.array_equal(a.level_counts, b.level_counts)
+
+
 @pytest.mark.parametrize("model", ["ic", "lt"])
 def test_batches(model):
     g = I.erdos_renyi_m(600, 4000, graph_seed=5)
