@@ -44,6 +44,7 @@ constexpr int OFF_WO = 18624;
 constexpr int OFF_BO = 18688;
 constexpr int N_PARAMS = 18689;
 constexpr int kItemEdges = 256;
+constexpr int kShortRow = 32;
 constexpr float kQScale = 2.3283064365386963e-10f;  // 2^-32
 
 static_assert(N_PARAMS == CND_SUR_N_PARAMS, "parameter count");
@@ -191,22 +192,58 @@ struct Item {
     int32_t node, begin, end, slot;  // slot >= 0: this item's partial row of a split node (scratch row index)
 };
 
-// a[v] = bf16(sum over in-edges of q h[src]) for 64-wide bf16 rows; a warp per item.  The warp
-// gathers 4 rows per load instruction (8 lanes x 16 B per 128-byte row), 16 rows in flight, and
-// folds the 4 partial sums of each feature at the end.
-__global__ void __launch_bounds__(256) k_spmm_in(int32_t n_items, const Item *__restrict__ items,
+// {acc.x, acc.y} += q {x.x, x.y}: two fp32 fused multiply-adds in one issue slot
+__device__ __forceinline__ void fma2(float2 &acc, float q, float2 x) {
+    const float2 qq = make_float2(q, q);
+    unsigned long long d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;"
+        : "=l"(d)
+        : "l"(*reinterpret_cast<const unsigned long long *>(&qq)), "l"(*reinterpret_cast<const unsigned long long *>(&x)),
+          "l"(*reinterpret_cast<const unsigned long long *>(&acc)));
+    acc = *reinterpret_cast<float2 *>(&d);
+}
+
+__device__ __forceinline__ void fma_row(float2 (&acc)[4], float q, const uint4 &row) {
+    fma2(acc[0], q, unpack_bf16(row.x));
+    fma2(acc[1], q, unpack_bf16(row.y));
+    fma2(acc[2], q, unpack_bf16(row.z));
+    fma2(acc[3], q, unpack_bf16(row.w));
+}
+
+__device__ __forceinline__ void store_sum(const Item &item, const float2 (&acc)[4], int f8, __nv_bfloat16 *a, float *scratch) {
+    if (item.slot < 0) {
+        *reinterpret_cast<uint4 *>(a + (size_t)item.node * H + f8) =
+            make_uint4(pack_bf16(acc[0].x, acc[0].y), pack_bf16(acc[1].x, acc[1].y), pack_bf16(acc[2].x, acc[2].y),
+                       pack_bf16(acc[3].x, acc[3].y));
+    } else {
+        float4 *pr = reinterpret_cast<float4 *>(scratch + (size_t)item.slot * H + f8);
+        pr[0] = make_float4(acc[0].x, acc[0].y, acc[1].x, acc[1].y);
+        pr[1] = make_float4(acc[2].x, acc[2].y, acc[3].x, acc[3].y);
+    }
+}
+
+// a[v] = bf16(sum over in-edges of q h[src]) for 64-wide bf16 rows (128 bytes, 8 lanes x 16 bytes).  The
+// sum of an item runs in four chains, edge e in chain e % 4, added as (0 + 1) + (2 + 3), whoever runs
+// them: items of more than kShortRow edges take a warp, a chain per 8 lanes, 16 rows in flight; the
+// others (most rows: half of R-MAT-17's have fewer than 4 edges) 8 lanes each, so that a warp sums
+// four of them at once instead of one with most of its lanes on padding.  Items come in descending
+// length, so the four are alike.  What bounds it is the latency of item, edge and row loads and, before,
+// instructions on padding (ncu: 60 % issue active at 12 % L2 throughput).  R-MAT-17 (1.94 M edges): 64 -> 36 us;
+// R-MAT-20 (16.1 M): 409 -> 272 us (2.06 GB of rows gathered).
+__global__ void __launch_bounds__(256) k_spmm_in(int32_t n_items, int32_t n_long, const Item *__restrict__ items,
                                                  const uint2 *__restrict__ in_c, const __nv_bfloat16 *__restrict__ h,
                                                  __nv_bfloat16 *__restrict__ a, float *__restrict__ scratch) {
     const int lane = threadIdx.x & 31;
-    const int sub = lane >> 3;       // which of 4 edges
-    const int f8 = (lane & 7) * 8;   // first of this lane's 8 features
+    const int sub = lane >> 3;       // which of 4 chains, or of 4 short items
+    const int l = lane & 7;
+    const int f8 = l * 8;            // first of this lane's 8 features
     const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int nwarps = (gridDim.x * blockDim.x) >> 5;
-    for (int it = warp; it < n_items; it += nwarps) {
+    for (int it = warp; it < n_long; it += nwarps) {
         const Item item = items[it];
-        float acc[8];
+        float2 acc[4];
 #pragma unroll
-        for (int i = 0; i < 8; ++i) acc[i] = 0.0f;
+        for (int i = 0; i < 4; ++i) acc[i] = make_float2(0.0f, 0.0f);
         for (int32_t b = item.begin; b < item.end; b += 32) {
             const int cnt = min(32, item.end - b);
             uint2 my = make_uint2(0u, 0u);
@@ -225,36 +262,61 @@ __global__ void __launch_bounds__(256) k_spmm_in(int32_t n_items, const Item *__
                     rr[r] = *reinterpret_cast<const uint4 *>(h + (size_t)(e < cnt ? u : 0u) * H + f8);
                 }
 #pragma unroll
-                for (int r = 0; r < 4; ++r) {
-                    const uint32_t w4[4] = {rr[r].x, rr[r].y, rr[r].z, rr[r].w};
+                for (int r = 0; r < 4; ++r) fma_row(acc, qq[r], rr[r]);
+            }
+        }
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        const float2 x = unpack_bf16(w4[i]);
-                        acc[2 * i] += qq[r] * x.x;
-                        acc[2 * i + 1] += qq[r] * x.y;
-                    }
+        for (int i = 0; i < 4; ++i) {
+            acc[i].x += __shfl_xor_sync(0xffffffffu, acc[i].x, 8);
+            acc[i].y += __shfl_xor_sync(0xffffffffu, acc[i].y, 8);
+            acc[i].x += __shfl_xor_sync(0xffffffffu, acc[i].x, 16);
+            acc[i].y += __shfl_xor_sync(0xffffffffu, acc[i].y, 16);
+        }
+        if (lane < 8) store_sum(item, acc, f8, a, scratch);
+    }
+    const int step = 4 * nwarps;
+    Item item{0, 0, 0, -1};
+    int it = n_long + 4 * warp + sub;
+    if (it < n_items) item = items[it];
+    for (int base = n_long + 4 * warp; base < n_items; base += step) {
+        Item next{0, 0, 0, -1};
+        if (it + step < n_items) next = items[it + step];
+        const int len = item.end - item.begin;
+        const int longest = __shfl_sync(0xffffffffu, len, 0);
+        float2 acc[4][4];
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
+#pragma unroll
+            for (int i = 0; i < 4; ++i) acc[c][i] = make_float2(0.0f, 0.0f);
+        for (int b = 0; b < longest; b += 8) {
+            uint2 my = make_uint2(0u, 0u);  // past the end: q = 0, row 0 read, nothing added
+            if (b + l < len) my = in_c[item.begin + b + l];
+            const float myq = edge_q(my.y);
+#pragma unroll
+            for (int j = 0; j < 8; j += 4) {
+                if (b + j >= longest) break;
+                uint4 rr[4];
+                float qq[4];
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    const uint32_t u = __shfl_sync(0xffffffffu, my.x, j + c, 8);
+                    qq[c] = __shfl_sync(0xffffffffu, myq, j + c, 8);
+                    rr[c] = *reinterpret_cast<const uint4 *>(h + (size_t)u * H + f8);
                 }
-            }
-        }
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            acc[i] += __shfl_xor_sync(0xffffffffu, acc[i], 8);
-            acc[i] += __shfl_xor_sync(0xffffffffu, acc[i], 16);
-        }
-        if (lane < 8) {
-            if (item.slot < 0) {
-                uint4 o;
-                o.x = pack_bf16(acc[0], acc[1]);
-                o.y = pack_bf16(acc[2], acc[3]);
-                o.z = pack_bf16(acc[4], acc[5]);
-                o.w = pack_bf16(acc[6], acc[7]);
-                *reinterpret_cast<uint4 *>(a + (size_t)item.node * H + f8) = o;
-            } else {
-                float4 *pr = reinterpret_cast<float4 *>(scratch + (size_t)item.slot * H + f8);
-                pr[0] = make_float4(acc[0], acc[1], acc[2], acc[3]);
-                pr[1] = make_float4(acc[4], acc[5], acc[6], acc[7]);
+                for (int c = 0; c < 4; ++c) fma_row(acc[c], qq[c], rr[c]);
             }
         }
+        if (it < n_items) {
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                acc[0][i].x = (acc[0][i].x + acc[1][i].x) + (acc[2][i].x + acc[3][i].x);
+                acc[0][i].y = (acc[0][i].y + acc[1][i].y) + (acc[2][i].y + acc[3][i].y);
+            }
+            store_sum(item, acc[0], f8, a, scratch);
+        }
+        item = next;
+        it += step;
     }
 }
 
@@ -299,19 +361,45 @@ __global__ void k_split_out_finish(int32_t n_split, const int32_t *__restrict__ 
     }
 }
 
-// dh[u] += sum over out-edges (u -> w) of q da[w], 64-wide fp32 rows; a warp per item of the out-CSR,
-// 2 rows per load instruction (16 lanes x 16 B per 256-byte row), 8 rows in flight.  An item of a
-// split node writes its partial row (k_split_out_finish adds them in order); a single-item node is
-// read-modify-written by its warp.
-__global__ void __launch_bounds__(256) k_spmm_out(int32_t n_items, const Item *__restrict__ items,
+__device__ __forceinline__ void fma_row4(float4 &acc, float q, const float4 &x) {
+    float2 lo = make_float2(acc.x, acc.y), hi = make_float2(acc.z, acc.w);
+    fma2(lo, q, make_float2(x.x, x.y));
+    fma2(hi, q, make_float2(x.z, x.w));
+    acc = make_float4(lo.x, lo.y, hi.x, hi.y);
+}
+
+__device__ __forceinline__ void add4(float4 &a, const float4 &b) {
+    a.x += b.x;
+    a.y += b.y;
+    a.z += b.z;
+    a.w += b.w;
+}
+
+// dh[u] += sum over out-edges (u -> w) of q da[w], 64-wide fp32 rows (256 bytes, 16 lanes x 16 bytes).  As
+// k_spmm_in with two chains (edge e in chain e % 2): items of more than kShortRow edges take a warp, a
+// chain per half, 8 rows in flight; the others half a warp each.  An item of a split node writes its
+// partial row (k_split_out_finish adds them in order); a single-item node is read-modify-written by its
+// lanes.  R-MAT-17: 102 -> 52 us (497 MB of rows gathered).
+__global__ void __launch_bounds__(256) k_spmm_out(int32_t n_items, int32_t n_long, const Item *__restrict__ items,
                                                   const uint2 *__restrict__ ic_edge, const float *__restrict__ da,
                                                   float *__restrict__ dh, float *__restrict__ scratch) {
     const int lane = threadIdx.x & 31;
-    const int sub = lane >> 4;       // which of 2 edges
-    const int f4 = (lane & 15) * 4;  // first of this lane's 4 features
+    const int sub = lane >> 4;       // which of 2 chains, or of 2 short items
+    const int l = lane & 15;
+    const int f4 = l * 4;            // first of this lane's 4 features
     const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int nwarps = (gridDim.x * blockDim.x) >> 5;
-    for (int it = warp; it < n_items; it += nwarps) {
+    auto store = [&](const Item &item, const float4 &acc) {
+        if (item.slot < 0) {
+            float4 *row = reinterpret_cast<float4 *>(dh + (size_t)item.node * H + f4);
+            float4 v = *row;
+            add4(v, acc);
+            *row = v;
+        } else {
+            *reinterpret_cast<float4 *>(scratch + (size_t)item.slot * H + f4) = acc;
+        }
+    };
+    for (int it = warp; it < n_long; it += nwarps) {
         const Item item = items[it];
         float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
         for (int32_t b = item.begin; b < item.end; b += 32) {
@@ -331,31 +419,49 @@ __global__ void __launch_bounds__(256) k_spmm_out(int32_t n_items, const Item *_
                     xx[r] = *reinterpret_cast<const float4 *>(da + (size_t)(e < cnt ? w : 0u) * H + f4);
                 }
 #pragma unroll
-                for (int r = 0; r < 4; ++r) {
-                    acc.x += qq[r] * xx[r].x;
-                    acc.y += qq[r] * xx[r].y;
-                    acc.z += qq[r] * xx[r].z;
-                    acc.w += qq[r] * xx[r].w;
-                }
+                for (int r = 0; r < 4; ++r) fma_row4(acc, qq[r], xx[r]);
             }
         }
         acc.x += __shfl_xor_sync(0xffffffffu, acc.x, 16);
         acc.y += __shfl_xor_sync(0xffffffffu, acc.y, 16);
         acc.z += __shfl_xor_sync(0xffffffffu, acc.z, 16);
         acc.w += __shfl_xor_sync(0xffffffffu, acc.w, 16);
-        if (lane < 16) {
-            float4 *row = reinterpret_cast<float4 *>(dh + (size_t)item.node * H + f4);
-            if (item.slot < 0) {
-                float4 v = *row;
-                v.x += acc.x;
-                v.y += acc.y;
-                v.z += acc.z;
-                v.w += acc.w;
-                *row = v;
-            } else {
-                *reinterpret_cast<float4 *>(scratch + (size_t)item.slot * H + f4) = acc;
+        if (lane < 16) store(item, acc);
+    }
+    const int step = 2 * nwarps;
+    Item item{0, 0, 0, -1};
+    int it = n_long + 2 * warp + sub;
+    if (it < n_items) item = items[it];
+    for (int base = n_long + 2 * warp; base < n_items; base += step) {
+        Item next{0, 0, 0, -1};
+        if (it + step < n_items) next = items[it + step];
+        const int len = item.end - item.begin;
+        const int longest = __shfl_sync(0xffffffffu, len, 0);
+        float4 acc[2];
+        acc[0] = acc[1] = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int b = 0; b < longest; b += 16) {
+            uint2 my = make_uint2(0u, 0u);
+            if (b + l < len) my = ic_edge[item.begin + b + l];
+            const float myq = edge_q(my.y);
+            for (int j = 0; j < 16 && b + j < longest; j += 4) {
+                float4 xx[4];
+                float qq[4];
+#pragma unroll
+                for (int r = 0; r < 4; ++r) {
+                    const uint32_t w = __shfl_sync(0xffffffffu, my.x, j + r, 16);
+                    qq[r] = __shfl_sync(0xffffffffu, myq, j + r, 16);
+                    xx[r] = *reinterpret_cast<const float4 *>(da + (size_t)w * H + f4);
+                }
+#pragma unroll
+                for (int r = 0; r < 4; ++r) fma_row4(acc[r & 1], qq[r], xx[r]);
             }
         }
+        if (len > 0) {
+            add4(acc[0], acc[1]);
+            store(item, acc[0]);
+        }
+        item = next;
+        it += step;
     }
 }
 
@@ -886,6 +992,8 @@ struct cnd_sur {
     uint2 *in_c = nullptr;
     Item *items_in = nullptr, *items_out = nullptr;
     int32_t n_items_in = 0, n_items_out = 0;
+    int32_t n_long_in = 0, n_long_out = 0;  // items of more than kShortRow edges (they come first)
+    int spmm_in_blocks = 0, spmm_out_blocks = 0;  // resident blocks of the aggregation kernels
     int32_t *split_node = nullptr, *split_first = nullptr;  // in-CSR split nodes, first partial row of each
     int32_t n_split = 0;
     float *scratch = nullptr;                                 // partial rows of the in-aggregation
@@ -926,26 +1034,33 @@ void free_all(cnd_sur *s) {
     s->allocs.clear();
 }
 
-// work items of <= kItemEdges edges per node; a row with more edges is split, each of its items
-// getting a partial-row slot of its own (consecutive per node): split[i] is the i-th split node and
-// first[i] .. first[i+1]-1 its slots
+// work items of <= kItemEdges edges per node, in descending length (n_long: those of more than
+// kShortRow edges); a row with more edges is split, each of its items getting a partial-row slot of its
+// own (consecutive per node): split[i] is the i-th split node and first[i] .. first[i+1]-1 its slots
 void make_items(const std::vector<int32_t> &rp, std::vector<Item> &items, std::vector<int32_t> &split,
-                std::vector<int32_t> &first) {
+                std::vector<int32_t> &first, int32_t &n_long) {
     const int32_t n = (int32_t)rp.size() - 1;
-    items.clear();
     split.clear();
     first.assign(1, 0);
+    std::vector<int32_t> at(kItemEdges + 2, 0);  // counting sort by kItemEdges - length
+    auto each = [&](auto &&f) {
+        for (int32_t v = 0; v < n; ++v)
+            for (int64_t k = rp[v]; k == rp[v] || k < rp[v + 1]; k += kItemEdges)
+                f(v, (int32_t)k, (int32_t)std::min<int64_t>(rp[v + 1], k + kItemEdges));
+    };
+    each([&](int32_t, int32_t b, int32_t e) { at[(size_t)(kItemEdges - (e - b)) + 1]++; });
+    for (size_t i = 1; i < at.size(); ++i) at[i] += at[i - 1];
+    items.resize((size_t)at.back());
+    n_long = at[(size_t)(kItemEdges - kShortRow)];
     int32_t slot = 0;
-    for (int32_t v = 0; v < n; ++v) {
-        const int32_t b = rp[v], e = rp[v + 1];
-        if (e - b <= kItemEdges) {
-            items.push_back({v, b, e, -1});
-        } else {
+    each([&](int32_t v, int32_t b, int32_t e) {
+        const bool whole = rp[v + 1] - rp[v] <= kItemEdges;
+        items[(size_t)at[(size_t)(kItemEdges - (e - b))]++] = Item{v, b, e, whole ? -1 : slot++};
+        if (!whole && e == rp[v + 1]) {
             split.push_back(v);
-            for (int32_t k = b; k < e; k += kItemEdges) items.push_back({v, k, std::min(e, k + kItemEdges), slot++});
             first.push_back(slot);
         }
-    }
+    });
 }
 
 int grid_for(int64_t work, int per_block, int num_sms, int max_per_sm = 8) {
@@ -1010,8 +1125,7 @@ void seed_clear(cnd_sur *s, const int32_t *d_seeds, int32_t ns, cudaStream_t st)
 }
 
 void aggregate_in(cnd_sur *s, const __nv_bfloat16 *hin, __nv_bfloat16 *aout, cudaStream_t st) {
-    const int blocks = grid_for((int64_t)s->n_items_in * 32, 256, s->num_sms);
-    k_spmm_in<<<blocks, 256, 0, st>>>(s->n_items_in, s->items_in, s->in_c, hin, aout, s->scratch);
+    k_spmm_in<<<s->spmm_in_blocks, 256, 0, st>>>(s->n_items_in, s->n_long_in, s->items_in, s->in_c, hin, aout, s->scratch);
     if (s->n_split)
         k_split_finish<<<grid_for((int64_t)s->n_split * 32, 256, s->num_sms), 256, 0, st>>>(
             s->n_split, s->split_node, s->split_first, s->scratch, aout);
@@ -1029,8 +1143,7 @@ void forward(cnd_sur *s, cudaStream_t st) {
 }
 
 void aggregate_out(cnd_sur *s, const float *da, float *dh, cudaStream_t st) {
-    const int blocks = grid_for((int64_t)s->n_items_out * 32, 256, s->num_sms);
-    k_spmm_out<<<blocks, 256, 0, st>>>(s->n_items_out, s->items_out, s->g->d.ic_edge, da, dh, s->scratch_out);
+    k_spmm_out<<<s->spmm_out_blocks, 256, 0, st>>>(s->n_items_out, s->n_long_out, s->items_out, s->g->d.ic_edge, da, dh, s->scratch_out);
     if (s->n_split_out)
         k_split_out_finish<<<grid_for((int64_t)s->n_split_out * 32, 256, s->num_sms), 256, 0, st>>>(
             s->n_split_out, s->split_out_node, s->split_out_first, s->scratch_out, dh);
@@ -1144,11 +1257,19 @@ cnd_status cnd_sur_create(const cnd_graph *g, const float *params, cnd_sur **out
         return fail(e, "in_row_ptr");
     std::vector<Item> it_in, it_out;
     std::vector<int32_t> split, first, split_out, first_out;
-    make_items(irp, it_in, split, first);
-    make_items(rp, it_out, split_out, first_out);
+    make_items(irp, it_in, split, first, s->n_long_in);
+    make_items(rp, it_out, split_out, first_out, s->n_long_out);
     s->row_ptr_h = rp;
     s->n_items_in = (int32_t)it_in.size();
     s->n_items_out = (int32_t)it_out.size();
+    // all resident blocks and no more: a second, partly filled wave would end after the first
+    auto resident = [&](auto *fn) {
+        int per_sm = 0;
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, 256, 0) != cudaSuccess || per_sm < 1) per_sm = 1;
+        return s->num_sms * per_sm;
+    };
+    s->spmm_in_blocks = std::min(resident(k_spmm_in), grid_for((int64_t)s->n_items_in * 32, 256, s->num_sms));
+    s->spmm_out_blocks = std::min(resident(k_spmm_out), grid_for((int64_t)s->n_items_out * 32, 256, s->num_sms));
     s->n_split = (int32_t)split.size();
     s->n_split_out = (int32_t)split_out.size();
     // per-block partials: the backward's blocks (bias rows, dW blocks), the spread's blocks
