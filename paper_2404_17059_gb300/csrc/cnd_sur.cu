@@ -73,6 +73,31 @@ __device__ __forceinline__ void mma16816(float (&d)[4], uint32_t a0, uint32_t a1
         : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
 
+// four 8 x 8 bf16 matrices from shared memory; lane i gives the address of row i % 8 of matrix i / 8
+__device__ __forceinline__ void ldmatrix4(uint32_t (&r)[4], const __nv_bfloat16 *p) {
+    const uint32_t a = (uint32_t)__cvta_generic_to_shared(p);
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"(a)
+                 : "memory");
+}
+
+// ... transposed
+__device__ __forceinline__ void ldmatrix4_trans(uint32_t (&r)[4], const __nv_bfloat16 *p) {
+    const uint32_t a = (uint32_t)__cvta_generic_to_shared(p);
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"(a)
+                 : "memory");
+}
+
+// 16 bytes from global to shared memory without passing registers; zeros if !ok
+__device__ __forceinline__ void copy16(__nv_bfloat16 *dst, const __nv_bfloat16 *src, bool ok) {
+    const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst);
+    const int n = ok ? 16 : 0;
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(src), "r"(n) : "memory");
+}
+
 __device__ __forceinline__ uint32_t ld_u32(const __nv_bfloat16 *p) { return *reinterpret_cast<const uint32_t *>(p); }
 
 // --------------------------------------------------------------------------- setup kernels
@@ -474,7 +499,19 @@ struct WTile {
     static constexpr int LDT = H + 8;       // padded row of wt
 };
 
-// h_out = bf16(relu([h_in | a] W^T + b)); HEAD: also o = w_o . h_out + b_o
+// h_out = bf16(relu([h_in | a] W^T + b)); HEAD: also o = w_o . h_out + b_o.  Reads and writes each row once
+// (400 MB at R-MAT-20, 60 us at the copy rate).  Each warp copies its next tile's 16 rows asynchronously
+// while it works on the current one, takes fragments by ldmatrix and sends the results out as whole
+// 128-byte rows through the tile's buffer; with 4-byte loads and stores straight from and to memory,
+// one tile at a time, the 64-wide layers took 139 us at R-MAT-20, now 71.
+template <int DIN>
+struct FwdSmem {
+    static constexpr int kPitch = (2 * DIN > H ? 2 * DIN : H) + 8;  // of a tile's rows [h | a], or its 64 results
+    __nv_bfloat16 w[H * (2 * DIN + 8)];
+    float b[H], wo[H];
+    __nv_bfloat16 tile[4][2][16 * kPitch];  // [warp][buffer]
+};
+
 template <int DIN, bool HEAD>
 __global__ void __launch_bounds__(128) k_dense_fwd(int32_t n, const __nv_bfloat16 *__restrict__ hin,
                                                    const __nv_bfloat16 *__restrict__ ain,
@@ -482,53 +519,77 @@ __global__ void __launch_bounds__(128) k_dense_fwd(int32_t n, const __nv_bfloat1
                                                    const float *__restrict__ params, int layer,
                                                    __nv_bfloat16 *__restrict__ hout, float *__restrict__ o_out) {
     using T = WTile<DIN>;
-    __shared__ __align__(16) __nv_bfloat16 sw[H * T::LDW];
-    __shared__ float sb[H], swo[H];
-    for (int i = threadIdx.x; i < H * T::K; i += blockDim.x) sw[(i / T::K) * T::LDW + i % T::K] = wcat[i];
-    for (int i = threadIdx.x; i < H; i += blockDim.x) {
-        sb[i] = params[off_b(layer) + i];
-        swo[i] = params[OFF_WO + i];
-    }
-    __syncthreads();
-    const float bo = params[OFF_BO];
-    const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+    extern __shared__ __align__(16) unsigned char fwd_smem[];
+    FwdSmem<DIN> &S = *reinterpret_cast<FwdSmem<DIN> *>(fwd_smem);
+    constexpr int PT = FwdSmem<DIN>::kPitch;
+    const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3, wib = threadIdx.x >> 5;
     const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int nwarps = (gridDim.x * blockDim.x) >> 5;
     const int tiles = (n + 15) >> 4;
-    for (int tile = warp; tile < tiles; tile += nwarps) {
-        const int rA = tile * 16 + g, rB = rA + 8;
-        const bool okA = rA < n, okB = rB < n;
+    auto fetch = [&](int tile, int buf) {
+        if (tile < tiles) {
+#pragma unroll
+            for (int i = lane; i < 16 * (T::K / 8); i += 32) {
+                const int r = i / (T::K / 8), c = (i % (T::K / 8)) * 8;
+                const bool ok = tile * 16 + r < n;
+                const size_t row = (size_t)(ok ? tile * 16 + r : 0) * DIN;
+                copy16(S.tile[wib][buf] + r * PT + c, c < DIN ? hin + row + c : ain + row + (c - DIN), ok);
+            }
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    fetch(warp, 0);
+    for (int i = 8 * threadIdx.x; i < H * T::K; i += 8 * blockDim.x)
+        *reinterpret_cast<uint4 *>(S.w + (i / T::K) * T::LDW + i % T::K) = *reinterpret_cast<const uint4 *>(wcat + i);
+    for (int i = threadIdx.x; i < H; i += blockDim.x) {
+        S.b[i] = params[off_b(layer) + i];
+        S.wo[i] = params[OFF_WO + i];
+    }
+    __syncthreads();
+    const float bo = params[OFF_BO];
+    int buf = 0;
+    for (int tile = warp; tile < tiles; tile += nwarps, buf ^= 1) {
+        fetch(tile + nwarps, buf ^ 1);
+        asm volatile("cp.async.wait_group 1;" ::: "memory");
+        __syncwarp();
+        __nv_bfloat16 *x = S.tile[wib][buf];
         float acc[8][4];
 #pragma unroll
         for (int j = 0; j < 8; ++j) acc[j][0] = acc[j][1] = acc[j][2] = acc[j][3] = 0.0f;
 #pragma unroll
         for (int kk = 0; kk < T::K / 16; ++kk) {
-            const __nv_bfloat16 *src = (kk * 16 < DIN) ? hin : ain;
-            const int c = (kk * 16) % DIN + 2 * t;
-            const uint32_t a0 = okA ? ld_u32(src + (size_t)rA * DIN + c) : 0u;
-            const uint32_t a1 = okB ? ld_u32(src + (size_t)rB * DIN + c) : 0u;
-            const uint32_t a2 = okA ? ld_u32(src + (size_t)rA * DIN + c + 8) : 0u;
-            const uint32_t a3 = okB ? ld_u32(src + (size_t)rB * DIN + c + 8) : 0u;
+            uint32_t a[4];
+            ldmatrix4(a, x + (lane & 15) * PT + kk * 16 + (lane >> 4) * 8);
 #pragma unroll
-            for (int j = 0; j < 8; ++j) {
-                const __nv_bfloat16 *wr = sw + (j * 8 + g) * T::LDW + kk * 16 + 2 * t;
-                mma16816(acc[j], a0, a1, a2, a3, ld_u32(wr), ld_u32(wr + 8));
+            for (int j = 0; j < 8; j += 2) {
+                uint32_t b[4];  // outputs 8 j .. 8 j + 15
+                ldmatrix4(b, S.w + (j * 8 + (lane >> 4) * 8 + (lane & 7)) * T::LDW + kk * 16 + ((lane >> 3) & 1) * 8);
+                mma16816(acc[j], a[0], a[1], a[2], a[3], b[0], b[1]);
+                mma16816(acc[j + 1], a[0], a[1], a[2], a[3], b[2], b[3]);
             }
         }
+        __syncwarp();  // everyone has read the tile: its buffer takes the results
         float pA = 0.0f, pB = 0.0f;
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
             const int col = j * 8 + 2 * t;
-            const float z0 = round_bf16(fmaxf(acc[j][0] + sb[col], 0.0f));
-            const float z1 = round_bf16(fmaxf(acc[j][1] + sb[col + 1], 0.0f));
-            const float z2 = round_bf16(fmaxf(acc[j][2] + sb[col], 0.0f));
-            const float z3 = round_bf16(fmaxf(acc[j][3] + sb[col + 1], 0.0f));
-            if (okA) *reinterpret_cast<uint32_t *>(hout + (size_t)rA * H + col) = pack_bf16(z0, z1);
-            if (okB) *reinterpret_cast<uint32_t *>(hout + (size_t)rB * H + col) = pack_bf16(z2, z3);
+            const float z0 = round_bf16(fmaxf(acc[j][0] + S.b[col], 0.0f));
+            const float z1 = round_bf16(fmaxf(acc[j][1] + S.b[col + 1], 0.0f));
+            const float z2 = round_bf16(fmaxf(acc[j][2] + S.b[col], 0.0f));
+            const float z3 = round_bf16(fmaxf(acc[j][3] + S.b[col + 1], 0.0f));
+            *reinterpret_cast<uint32_t *>(x + g * PT + col) = pack_bf16(z0, z1);
+            *reinterpret_cast<uint32_t *>(x + (g + 8) * PT + col) = pack_bf16(z2, z3);
             if (HEAD) {
-                pA += z0 * swo[col] + z1 * swo[col + 1];
-                pB += z2 * swo[col] + z3 * swo[col + 1];
+                pA += z0 * S.wo[col] + z1 * S.wo[col + 1];
+                pB += z2 * S.wo[col] + z3 * S.wo[col + 1];
             }
+        }
+        __syncwarp();
+#pragma unroll
+        for (int i = lane; i < 16 * (H / 8); i += 32) {
+            const int r = i / (H / 8), c = (i % (H / 8)) * 8;
+            if (tile * 16 + r < n)
+                *reinterpret_cast<uint4 *>(hout + (size_t)(tile * 16 + r) * H + c) = *reinterpret_cast<const uint4 *>(x + r * PT + c);
         }
         if (HEAD) {
             pA += __shfl_xor_sync(0xffffffffu, pA, 1);
@@ -536,10 +597,11 @@ __global__ void __launch_bounds__(128) k_dense_fwd(int32_t n, const __nv_bfloat1
             pB += __shfl_xor_sync(0xffffffffu, pB, 1);
             pB += __shfl_xor_sync(0xffffffffu, pB, 2);
             if (t == 0) {
-                if (okA) o_out[rA] = pA + bo;
-                if (okB) o_out[rB] = pB + bo;
+                if (tile * 16 + g < n) o_out[tile * 16 + g] = pA + bo;
+                if (tile * 16 + g + 8 < n) o_out[tile * 16 + g + 8] = pB + bo;
             }
         }
+        __syncwarp();  // the buffer is free for the tile after next
     }
 }
 
@@ -589,7 +651,8 @@ __global__ void __launch_bounds__(128) k_dense_bwd(int32_t n, const __nv_bfloat1
     __shared__ __align__(16) __nv_bfloat16 swt[(XOUT ? T::K : 1) * T::LDT];
     __shared__ float swo[H];
     if (XOUT)
-        for (int i = threadIdx.x; i < T::K * H; i += blockDim.x) swt[(i / H) * T::LDT + i % H] = wt[i];
+        for (int i = 8 * threadIdx.x; i < T::K * H; i += 8 * blockDim.x)
+            *reinterpret_cast<uint4 *>(swt + (i / H) * T::LDT + i % H) = *reinterpret_cast<const uint4 *>(wt + i);
     for (int i = threadIdx.x; i < H; i += blockDim.x) swo[i] = params[OFF_WO + i];
     __syncthreads();
     const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
@@ -734,18 +797,22 @@ __global__ void __launch_bounds__(128) k_dense_bwd(int32_t n, const __nv_bfloat1
 
 // dW[o][i] = sum_r e[r][o] X[r][i], X = [h_prev | a] (split-K over row chunks; 8 warps per block,
 // warp w owns outputs o in [16 (w % 4), +16) and inputs i in [K/2 (w / 4), +K/2)); block b writes its
-// partial dW (64 x 2 DIN, row-major) to part[b * 128 DIN ..], added up in block order by k_reduce_dw
+// partial dW (64 x 2 DIN, row-major) to part[b * 128 DIN ..], added up in block order by k_reduce_dw.
+// Row chunks are copied asynchronously, kStages - 1 ahead, and both operands are read transposed by ldmatrix.
+// The kernel reads each row once (50 MB at R-MAT-17 for DIN = 64, 7 us at the copy rate); waiting for
+// each chunk and gathering fragments by 2-byte loads took 44 us, now 17.
 template <int DIN>
 __global__ void __launch_bounds__(256) k_dw(int32_t n, const __nv_bfloat16 *__restrict__ e,
                                             const __nv_bfloat16 *__restrict__ hprev,
                                             const __nv_bfloat16 *__restrict__ ain, float *__restrict__ part,
                                             int rows_per_block) {
     constexpr int K = 2 * DIN;
-    constexpr int LE = H + 8, LX = K + 8;
+    constexpr int LE = H + 8, LX = K + 8;  // 16-byte aligned rows, an odd number of 16-byte units apart
     constexpr int NT = K / 2 / 8;  // n-tiles per warp
     constexpr int RC = 32;         // rows per chunk
-    __shared__ __align__(16) __nv_bfloat16 se[RC * LE];
-    __shared__ __align__(16) __nv_bfloat16 sx[RC * LX];
+    constexpr int kStages = 3;
+    __shared__ __align__(16) __nv_bfloat16 se[kStages][RC * LE];
+    __shared__ __align__(16) __nv_bfloat16 sx[kStages][RC * LX];
     const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3, w = threadIdx.x >> 5;
     const int o0 = 16 * (w & 3), i0 = (K / 2) * (w >> 2);
     float acc[NT][4];
@@ -753,43 +820,43 @@ __global__ void __launch_bounds__(256) k_dw(int32_t n, const __nv_bfloat16 *__re
     for (int j = 0; j < NT; ++j) acc[j][0] = acc[j][1] = acc[j][2] = acc[j][3] = 0.0f;
     const int rb = blockIdx.x * rows_per_block;
     const int re = min(n, rb + rows_per_block);
-    for (int r0 = rb; r0 < re; r0 += RC) {
-        // stage e rows (64 bf16 = 8 x 16 B) and X rows (K bf16 = K/8 x 16 B)
-        for (int i = threadIdx.x; i < RC * 8; i += blockDim.x) {
-            const int r = i >> 3, c = (i & 7) * 8;
-            uint4 v = make_uint4(0u, 0u, 0u, 0u);
-            if (r0 + r < re) v = *reinterpret_cast<const uint4 *>(e + (size_t)(r0 + r) * H + c);
-            *reinterpret_cast<uint4 *>(se + r * LE + c) = v;
-        }
-        for (int i = threadIdx.x; i < RC * (K / 8); i += blockDim.x) {
-            const int r = i / (K / 8), c = (i % (K / 8)) * 8;
-            uint4 v = make_uint4(0u, 0u, 0u, 0u);
-            if (r0 + r < re)
-                v = c < DIN ? *reinterpret_cast<const uint4 *>(hprev + (size_t)(r0 + r) * DIN + c)
-                            : *reinterpret_cast<const uint4 *>(ain + (size_t)(r0 + r) * DIN + (c - DIN));
-            *reinterpret_cast<uint4 *>(sx + r * LX + c) = v;
-        }
-        __syncthreads();
-#pragma unroll
-        for (int ks = 0; ks < RC / 16; ++ks) {
-            const int r = ks * 16;
-            auto E = [&](int rr, int oo) { return se[(r + rr) * LE + o0 + oo]; };
-            auto pk = [](__nv_bfloat16 lo, __nv_bfloat16 hi) {
-                return (uint32_t)__bfloat16_as_ushort(lo) | ((uint32_t)__bfloat16_as_ushort(hi) << 16);
-            };
-            const uint32_t a0 = pk(E(2 * t, g), E(2 * t + 1, g));
-            const uint32_t a1 = pk(E(2 * t, g + 8), E(2 * t + 1, g + 8));
-            const uint32_t a2 = pk(E(2 * t + 8, g), E(2 * t + 9, g));
-            const uint32_t a3 = pk(E(2 * t + 8, g + 8), E(2 * t + 9, g + 8));
-#pragma unroll
-            for (int j = 0; j < NT; ++j) {
-                const int col = i0 + j * 8 + g;
-                const uint32_t b0 = pk(sx[(r + 2 * t) * LX + col], sx[(r + 2 * t + 1) * LX + col]);
-                const uint32_t b1 = pk(sx[(r + 2 * t + 8) * LX + col], sx[(r + 2 * t + 9) * LX + col]);
-                mma16816(acc[j], a0, a1, a2, a3, b0, b1);
+    const int chunks = (re - rb + RC - 1) / RC;
+    // e rows (64 bf16 = 8 x 16 B) and X rows (K bf16 = K / 8 x 16 B) of chunk c; zeros past the end
+    auto stage = [&](int c) {
+        if (c < chunks) {
+            const int r0 = rb + c * RC, s = c % kStages;
+            for (int i = threadIdx.x; i < RC * 8; i += blockDim.x) {
+                const int r = i >> 3, col = (i & 7) * 8;
+                const bool ok = r0 + r < re;
+                copy16(se[s] + r * LE + col, e + (size_t)(ok ? r0 + r : rb) * H + col, ok);
+            }
+            for (int i = threadIdx.x; i < RC * (K / 8); i += blockDim.x) {
+                const int r = i / (K / 8), col = (i % (K / 8)) * 8;
+                const bool ok = r0 + r < re;
+                const size_t row = (size_t)(ok ? r0 + r : rb) * DIN;
+                copy16(sx[s] + r * LX + col, col < DIN ? hprev + row + col : ain + row + (col - DIN), ok);
             }
         }
-        __syncthreads();
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    for (int c = 0; c < kStages - 1; ++c) stage(c);
+    for (int c = 0; c < chunks; ++c) {
+        asm volatile("cp.async.wait_group %0;" ::"n"(kStages - 2) : "memory");
+        __syncthreads();  // chunk c has arrived, and everyone is done with chunk c - 1's buffer
+        stage(c + kStages - 1);
+        const __nv_bfloat16 *pe = se[c % kStages], *px = sx[c % kStages];
+#pragma unroll
+        for (int ks = 0; ks < RC / 16; ++ks) {
+            uint32_t a[4];
+            ldmatrix4_trans(a, pe + (ks * 16 + (lane >> 4) * 8 + (lane & 7)) * LE + o0 + ((lane >> 3) & 1) * 8);
+#pragma unroll
+            for (int j = 0; j < NT; j += 2) {
+                uint32_t b[4];
+                ldmatrix4_trans(b, px + (ks * 16 + ((lane >> 3) & 1) * 8 + (lane & 7)) * LX + i0 + j * 8 + (lane >> 4) * 8);
+                mma16816(acc[j], a[0], a[1], a[2], a[3], b[0], b[1]);
+                mma16816(acc[j + 1], a[0], a[1], a[2], a[3], b[2], b[3]);
+            }
+        }
     }
     float *pb = part + (size_t)blockIdx.x * (H * K);
 #pragma unroll
@@ -1133,12 +1200,12 @@ void aggregate_in(cnd_sur *s, const __nv_bfloat16 *hin, __nv_bfloat16 *aout, cud
 
 void forward(cnd_sur *s, cudaStream_t st) {
     const int32_t n = s->n;
-    const int tb = grid_for(((int64_t)n + 15) / 16 * 32, 128, s->num_sms, 16);
-    k_dense_fwd<D0, false><<<tb, 128, 0, st>>>(n, s->x, s->a1, s->wcat, s->p, 0, s->h[0], nullptr);
+    const int tb = grid_for(((int64_t)n + 15) / 16 * 32, 128, s->num_sms, 4);  // what is resident
+    k_dense_fwd<D0, false><<<tb, 128, sizeof(FwdSmem<D0>), st>>>(n, s->x, s->a1, s->wcat, s->p, 0, s->h[0], nullptr);
     aggregate_in(s, s->h[0], s->a[1], st);
-    k_dense_fwd<H, false><<<tb, 128, 0, st>>>(n, s->h[0], s->a[1], s->wcat + 64 * 32, s->p, 1, s->h[1], nullptr);
+    k_dense_fwd<H, false><<<tb, 128, sizeof(FwdSmem<H>), st>>>(n, s->h[0], s->a[1], s->wcat + 64 * 32, s->p, 1, s->h[1], nullptr);
     aggregate_in(s, s->h[1], s->a[2], st);
-    k_dense_fwd<H, true><<<tb, 128, 0, st>>>(n, s->h[1], s->a[2], s->wcat + 64 * 32 + 64 * 128, s->p, 2, s->h[2],
+    k_dense_fwd<H, true><<<tb, 128, sizeof(FwdSmem<H>), st>>>(n, s->h[1], s->a[2], s->wcat + 64 * 32 + 64 * 128, s->p, 2, s->h[2],
                                              s->o);
 }
 
@@ -1169,7 +1236,6 @@ void spread_sum(cnd_sur *s, double *spread, cudaStream_t st) {
 // training backward: gradients accumulate into s->grad; loss adds into s->dsum[1]
 void backward_loss(cnd_sur *s, const float *y, const int32_t *cnt, float inv_t, float batch, cudaStream_t st) {
     const int32_t n = s->n;
-    const int tb = grid_for(((int64_t)n + 15) / 16 * 32, 128, s->num_sms, 16);
     const int tbb = grid_for(((int64_t)n + 15) / 16 * 32, 128, s->num_sms, 4);  // backward: few blocks, few atomics
     const int rpb = (int)std::max<int64_t>(512, (((int64_t)n + 2 * s->num_sms - 1) / (2 * s->num_sms) + 31) / 32 * 32);
     const int db = (int)std::max<int64_t>(1, ((int64_t)n + rpb - 1) / rpb);
@@ -1262,6 +1328,10 @@ cnd_status cnd_sur_create(const cnd_graph *g, const float *params, cnd_sur **out
     s->row_ptr_h = rp;
     s->n_items_in = (int32_t)it_in.size();
     s->n_items_out = (int32_t)it_out.size();
+    // the 64-wide forward layers take more shared memory than a kernel gets by default
+    for (const void *fn : {(const void *)k_dense_fwd<H, false>, (const void *)k_dense_fwd<H, true>})
+        if ((e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(FwdSmem<H>))) != cudaSuccess)
+            return fail(e, "shared memory");
     // all resident blocks and no more: a second, partly filled wave would end after the first
     auto resident = [&](auto *fn) {
         int per_sm = 0;
@@ -1479,7 +1549,7 @@ cnd_status cnd_sur_scores(cnd_sur *s, const int32_t *seeds, int32_t n_seeds, flo
     int32_t ns = 0;
     if ((st = upload_seeds(s, seeds, n_seeds, ns, cs, "cnd_sur_scores")) != CND_OK) return st;
     const int32_t n = s->n;
-    const int tb = grid_for(((int64_t)n + 15) / 16 * 32, 128, s->num_sms, 16);
+    const int tb = grid_for(((int64_t)n + 15) / 16 * 32, 128, s->num_sms, 8);
     seed_set(s, s->seeds, ns, cs);
     forward(s, cs);
     HeadArgs ha{s->o, s->x, nullptr, nullptr, 0.0f, 0.0f, nullptr, 0.0f};
