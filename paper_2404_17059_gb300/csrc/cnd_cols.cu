@@ -67,7 +67,6 @@ struct ColParams {
     unsigned long long *checks, *level_counts;
     int32_t lc_len, max_levels;
     unsigned long long timeout_ns;
-    int32_t *next;            // column counter
     CallFlags *flags;
 };
 
@@ -235,7 +234,7 @@ __global__ void __launch_bounds__(1024, 1) k_columns(ColParams p) {
     const uint32_t lt = (1u << lane) - 1u, le = lt | (1u << lane);
     unsigned long long ck = 0;
     for (;;) {
-        if (tid == 0) S.col = atomicAdd(p.next, 1);
+        if (tid == 0) S.col = atomicAdd(&p.flags->next_column, 1);
         __syncthreads();
         const int col = S.col;
         if (col >= p.n_cols) break;
@@ -508,10 +507,7 @@ bool columns_fit(int model, const cnd_graph_dev &G, const cnd_sim_opts &o, int64
     return G.max_out_degree < kHub && (trials <= 4 * kWideTrials || column_shape(model, G, 2, c));
 }
 
-cnd_status run_columns(int model, const cnd_graph_dev &G, const std::vector<ItemDesc> &items, const int32_t *seeds_dev,
-                       int32_t *spread, int32_t *count, unsigned long long *checks, unsigned long long *level_counts,
-                       CallFlags *flags, const cnd_sim_opts &o, cudaStream_t st) {
-    const void *fn = model == 0 ? (const void *)k_columns<0> : (const void *)k_columns<1>;
+cnd_status plan_columns(int model, const cnd_graph_dev &G, const std::vector<ItemDesc> &items, ColPlan &plan) {
     int64_t trials = 0;
     for (const auto &it : items) trials += it.trials;
     if (trials == 0) return CND_OK;
@@ -520,7 +516,6 @@ cnd_status run_columns(int model, const cnd_graph_dev &G, const std::vector<Item
     // trials (and 2 more: work that a check takes whatever its trials), at a rate in proportion to
     // the block's threads.
     ColShape c;
-    int bits = 32;
     double best = 1e300;
     for (int per_sm = 4; per_sm >= 1; per_sm >>= 1) {
         ColShape k;
@@ -530,47 +525,49 @@ cnd_status run_columns(int model, const cnd_graph_dev &G, const std::vector<Item
             const double cost = waves * (8 + per_sm * (b + 2));
             if (cost < best) {
                 best = cost;
-                bits = b;
+                plan.bits = b;
                 c = k;
             }
         }
     }
-
     const int64_t slots = (int64_t)G.num_sms * c.per_sm;
-    // the same value on every call: threads may launch with different sizes at the same time
-    CND_CUDA_TRY(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxDynamic));
-    std::vector<ColItem> h;
-    h.reserve(items.size());
+    plan.items.resize(sizeof(ColItem) * items.size());
+    ColItem *h = reinterpret_cast<ColItem *>(plan.items.data());
     int64_t cols = 0;
     for (const auto &it : items) {
-        h.push_back(ColItem{it.out0, it.key, (int32_t)it.seed_begin, (int32_t)it.seed_end, (int32_t)it.trials, (int32_t)cols});
-        cols += (it.trials + bits - 1) / bits;
+        *h++ = ColItem{it.out0, it.key, (int32_t)it.seed_begin, (int32_t)it.seed_end, (int32_t)it.trials, (int32_t)cols};
+        cols += (it.trials + plan.bits - 1) / plan.bits;
     }
     if (cols > 0x7FFFFFFF - slots) {
         set_error("too many trials in one call");
         return CND_EINVAL;
     }
-    const int64_t blocks = std::min<int64_t>(cols, slots);
-    // one allocation: the column counter, the items, the blocks' list entries beyond cap
-    const size_t off_bits = (16 + sizeof(ColItem) * h.size() + 15) & ~(size_t)15;
-    const size_t over = c.cap < G.n ? (size_t)blocks * (size_t)G.n : 0;
-    unsigned char *buf = nullptr;
-    CND_CUDA_TRY(cudaMallocAsync((void **)&buf, off_bits + 8 * over, st));
-    struct Free {
-        void *q;
-        cudaStream_t st;
-        ~Free() { cudaFreeAsync(q, st); }
-    } fr{buf, st};
-    CND_CUDA_TRY(cudaMemsetAsync(buf, 0, 16, st));
-    CND_CUDA_TRY(cudaMemcpyAsync(buf + 16, h.data(), sizeof(ColItem) * h.size(), cudaMemcpyHostToDevice, st));
+    plan.n_items = (int32_t)items.size();
+    plan.cols = (int32_t)cols;
+    plan.blocks = (int32_t)std::min<int64_t>(cols, slots);
+    plan.threads = c.threads;
+    plan.cap = c.cap;
+    plan.dyn = c.dyn;
+    plan.over = c.cap < G.n ? (size_t)plan.blocks * (size_t)G.n : 0;  // list entries beyond cap
+    plan.scratch = 8 * plan.over;
+    return CND_OK;
+}
+
+cnd_status run_columns(int model, const cnd_graph_dev &G, const ColPlan &plan, const void *items, void *scratch,
+                       const int32_t *seeds_dev, int32_t *spread, int32_t *count, unsigned long long *checks,
+                       unsigned long long *level_counts, CallFlags *flags, const cnd_sim_opts &o, cudaStream_t st) {
+    if (plan.cols == 0) return CND_OK;
+    const void *fn = model == 0 ? (const void *)k_columns<0> : (const void *)k_columns<1>;
+    // the same value on every call: threads may launch with different sizes at the same time
+    CND_CUDA_TRY(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxDynamic));
     ColParams p{};
     p.n = G.n;
-    p.n_items = (int32_t)h.size();
-    p.bits = bits;
-    p.n_cols = (int32_t)cols;
+    p.n_items = plan.n_items;
+    p.bits = plan.bits;
+    p.n_cols = plan.cols;
     p.row_ptr = G.row_ptr;
     p.edge = model == 0 ? G.ic_edge : G.lt_cnt_edge;
-    p.items = reinterpret_cast<const ColItem *>(buf + 16);
+    p.items = static_cast<const ColItem *>(items);
     p.seeds = seeds_dev;
     p.cnt_off = G.lt_cnt_off;
     p.unit_w = G.lt_unit_w;
@@ -582,13 +579,12 @@ cnd_status run_columns(int model, const cnd_graph_dev &G, const std::vector<Item
     p.lc_len = o.level_counts_len;
     p.max_levels = o.max_levels;
     p.timeout_ns = o.timeout_s > 0 ? (unsigned long long)std::max(1.0, std::min(o.timeout_s * 1e9, 1.8e19)) : 0ull;
-    p.next = reinterpret_cast<int32_t *>(buf);
-    p.cap = c.cap;
-    p.over_bits = reinterpret_cast<uint32_t *>(buf + off_bits);
-    p.over_node = reinterpret_cast<uint16_t *>(p.over_bits + over);
+    p.cap = plan.cap;
+    p.over_bits = static_cast<uint32_t *>(scratch);
+    p.over_node = reinterpret_cast<uint16_t *>(p.over_bits + plan.over);
     p.flags = flags;
     void *args[] = {&p};
-    CND_CUDA_TRY(cudaLaunchKernel(fn, dim3((unsigned)blocks), dim3((unsigned)c.threads), args, c.dyn, st));
+    CND_CUDA_TRY(cudaLaunchKernel(fn, dim3((unsigned)plan.blocks), dim3((unsigned)plan.threads), args, plan.dyn, st));
     return CND_OK;
 }
 

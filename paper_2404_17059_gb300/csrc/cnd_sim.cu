@@ -1735,13 +1735,31 @@ struct Work {
     }
 };
 
-struct PinnedCounters {
+// Per-thread pinned memory: step counters, and staging for the small inputs and outputs of host calls (a
+// copy to or from pageable memory goes through the driver's own staging and waits).  A call waits for
+// its copies before it returns, so the next call of the thread may use it.
+constexpr size_t kStaging = 256 * 1024;
+struct Pinned {
     int32_t *h = nullptr;
-    ~PinnedCounters() {
+    unsigned char *in = nullptr, *out = nullptr;
+    ~Pinned() {
         if (h) cudaFreeHost(h);
+        if (in) cudaFreeHost(in);
+        if (out) cudaFreeHost(out);
     }
 };
-static thread_local PinnedCounters t_pinned;
+static thread_local Pinned t_pinned;
+
+// Copy `bytes` from host to device memory on st, through the pinned staging where they fit.
+static cudaError_t stage_in(void *dst, const void *src, size_t bytes, cudaStream_t st) {
+    if (bytes > kStaging) return cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, st);
+    if (!t_pinned.in) {
+        const cudaError_t e = cudaMallocHost(&t_pinned.in, kStaging);
+        if (e != cudaSuccess) return e;
+    }
+    memcpy(t_pinned.in, src, bytes);
+    return cudaMemcpyAsync(dst, t_pinned.in, bytes, cudaMemcpyHostToDevice, st);
+}
 
 // Keep up to a quarter of the device's memory cached in the stream-ordered
 // pool between calls, so repeated simulations do not go back to the driver.
@@ -2573,35 +2591,44 @@ static cnd_status simulate_common(int model, const cnd_graph *g, const char *fn,
     const int32_t n = G.n;
     const size_t count_rows = batched ? (size_t)n_items : 1;
 
-    // ---- outputs on the device
-    int32_t *d_spread = nullptr, *d_count = nullptr;
-    CallFlags *d_flags = nullptr;
-    const int32_t *d_seeds = nullptr;
-    unsigned long long *d_lc = nullptr, *d_checks = nullptr;
+    // graphs whose per-trial state fits an SM's shared memory: one launch, a block per column of trials
+    const bool columns = columns_fit(model, G, o, total_trials);
+    ColPlan plan;
+    if (columns) {
+        const cnd_status ps = plan_columns(model, G, items, plan);
+        if (ps != CND_OK) return ps;
+    }
+
+    // ---- one allocation: what starts at zero (flags, level counts, and for host calls the spreads and
+    // counts), then the inputs (items of the column engine, seeds of host calls), then scratch
     const int lc_len = o.level_counts_len;
-    if (dev && spread_out) d_spread = spread_out;
-    else CND_CUDA_TRY(W.alloc(&d_spread, (size_t)std::max<int64_t>(total_trials, 1)));
-    if (count_out) {
-        if (dev) d_count = count_out;
-        else CND_CUDA_TRY(W.alloc(&d_count, (size_t)n * count_rows));
+    auto up16 = [](size_t b) { return (b + 15) & ~(size_t)15; };
+    const size_t spread_bytes = sizeof(int32_t) * (size_t)total_trials;
+    const size_t count_bytes = count_out ? sizeof(int32_t) * (size_t)n * count_rows : 0;
+    const size_t off_lc = up16(sizeof(CallFlags));
+    const size_t off_spread = off_lc + up16(sizeof(unsigned long long) * (size_t)lc_len);
+    const size_t off_count = off_spread + (dev && spread_out ? 0 : up16(spread_bytes));
+    const size_t zeroed = off_count + (dev ? 0 : up16(count_bytes));
+    const size_t seed_bytes = dev ? 0 : sizeof(int32_t) * (size_t)n_seeds_total;
+    const size_t off_seeds = zeroed + up16(plan.items.size());
+    const size_t off_scratch = off_seeds + up16(seed_bytes);
+    unsigned char *ws = nullptr;
+    CND_CUDA_TRY(W.alloc(&ws, off_scratch + plan.scratch));
+    CallFlags *d_flags = reinterpret_cast<CallFlags *>(ws);
+    unsigned long long *d_checks = &d_flags->checks;
+    unsigned long long *d_lc = reinterpret_cast<unsigned long long *>(ws + off_lc);
+    int32_t *d_spread = dev && spread_out ? spread_out : reinterpret_cast<int32_t *>(ws + off_spread);
+    int32_t *d_count = !count_out ? nullptr : dev ? count_out : reinterpret_cast<int32_t *>(ws + off_count);
+    const int32_t *d_seeds = dev ? seeds : reinterpret_cast<const int32_t *>(ws + off_seeds);
+    CND_CUDA_TRY(cudaMemsetAsync(ws, 0, zeroed, st));
+    if (dev && spread_out && total_trials && !columns) CND_CUDA_TRY(cudaMemsetAsync(d_spread, 0, spread_bytes, st));
+    if (dev && d_count) CND_CUDA_TRY(cudaMemsetAsync(d_count, 0, count_bytes, st));
+    if (!plan.items.empty() || seed_bytes) {
+        std::vector<unsigned char> in(off_scratch - zeroed);
+        if (!plan.items.empty()) memcpy(in.data(), plan.items.data(), plan.items.size());
+        if (seed_bytes) memcpy(in.data() + (off_seeds - zeroed), seeds, seed_bytes);
+        CND_CUDA_TRY(stage_in(ws + zeroed, in.data(), in.size(), st));
     }
-    CND_CUDA_TRY(W.alloc(&d_lc, (size_t)std::max(lc_len, 1)));
-    CND_CUDA_TRY(W.alloc(&d_checks, 1));
-    CND_CUDA_TRY(W.alloc(&d_flags, 1));
-    if (dev) {
-        d_seeds = seeds;
-    } else {
-        int32_t *tmp = nullptr;
-        CND_CUDA_TRY(W.alloc(&tmp, (size_t)std::max<int64_t>(n_seeds_total, 1)));
-        if (n_seeds_total)
-            CND_CUDA_TRY(cudaMemcpyAsync(tmp, seeds, sizeof(int32_t) * n_seeds_total, cudaMemcpyHostToDevice, st));
-        d_seeds = tmp;
-    }
-    if (total_trials) CND_CUDA_TRY(cudaMemsetAsync(d_spread, 0, sizeof(int32_t) * (size_t)total_trials, st));
-    if (d_count) CND_CUDA_TRY(cudaMemsetAsync(d_count, 0, sizeof(int32_t) * (size_t)n * count_rows, st));
-    CND_CUDA_TRY(cudaMemsetAsync(d_lc, 0, sizeof(unsigned long long) * (size_t)std::max(lc_len, 1), st));
-    CND_CUDA_TRY(cudaMemsetAsync(d_checks, 0, sizeof(unsigned long long), st));
-    CND_CUDA_TRY(cudaMemsetAsync(d_flags, 0, sizeof(CallFlags), st));
 
     cnd_sim_stats *S = o.stats;
     if (S) {
@@ -2610,37 +2637,39 @@ static cnd_status simulate_common(int model, const cnd_graph *g, const char *fn,
         S->flags = flags;
     }
     bool limit_hit = false;
-    // graphs whose per-trial state fits an SM's shared memory: one launch, a block per column of trials
-    const bool columns = columns_fit(model, G, o, total_trials);
-    const cnd_status rs = columns ? run_columns(model, G, items, d_seeds, d_spread, d_count, d_checks, d_lc, d_flags, o, st)
+    const cnd_status rs = columns ? run_columns(model, G, plan, ws + zeroed, ws + off_scratch, d_seeds, d_spread, d_count,
+                                                d_checks, d_lc, d_flags, o, st)
                                   : run_items(model, G, fn, items, d_seeds, batched, d_spread, d_count, d_checks, d_lc,
                                               &d_flags->bad_seed, o, W, limit_hit);
     if (rs != CND_OK) return rs;
 
-    // ---- results
-    CallFlags hf{};
-    CND_CUDA_TRY(cudaMemcpyAsync(&hf, d_flags, sizeof(hf), cudaMemcpyDeviceToHost, st));
-    std::vector<unsigned long long> hlc((size_t)std::max(lc_len, 1));
-    unsigned long long hchecks = 0;
+    // ---- results: one copy through the pinned staging where they fit
+    if (!t_pinned.out) CND_CUDA_TRY(cudaMallocHost(&t_pinned.out, kStaging));
+    const size_t small = dev ? off_spread : zeroed;
+    const bool staged = small <= kStaging;
+    CND_CUDA_TRY(cudaMemcpyAsync(t_pinned.out, ws, staged ? small : sizeof(CallFlags), cudaMemcpyDeviceToHost, st));
     if (dev) {
         if (o.edge_checks_out)
             CND_CUDA_TRY(cudaMemcpyAsync(o.edge_checks_out, d_checks, sizeof(int64_t), cudaMemcpyDeviceToDevice, st));
         if (lc_len)
             CND_CUDA_TRY(cudaMemcpyAsync(o.level_counts_out, d_lc, sizeof(int64_t) * lc_len, cudaMemcpyDeviceToDevice, st));
-    } else {
+    } else if (!staged) {
         if (spread_out && total_trials)
-            CND_CUDA_TRY(cudaMemcpyAsync(spread_out, d_spread, sizeof(int32_t) * total_trials, cudaMemcpyDeviceToHost, st));
-        if (count_out)
-            CND_CUDA_TRY(cudaMemcpyAsync(count_out, d_count, sizeof(int32_t) * (size_t)n * count_rows,
-                                         cudaMemcpyDeviceToHost, st));
-        CND_CUDA_TRY(cudaMemcpyAsync(&hchecks, d_checks, sizeof(hchecks), cudaMemcpyDeviceToHost, st));
+            CND_CUDA_TRY(cudaMemcpyAsync(spread_out, d_spread, spread_bytes, cudaMemcpyDeviceToHost, st));
+        if (count_out) CND_CUDA_TRY(cudaMemcpyAsync(count_out, d_count, count_bytes, cudaMemcpyDeviceToHost, st));
         if (lc_len)
-            CND_CUDA_TRY(cudaMemcpyAsync(hlc.data(), d_lc, sizeof(unsigned long long) * lc_len, cudaMemcpyDeviceToHost, st));
+            CND_CUDA_TRY(cudaMemcpyAsync(o.level_counts_out, d_lc, sizeof(int64_t) * lc_len, cudaMemcpyDeviceToHost, st));
     }
     CND_CUDA_TRY(cudaStreamSynchronize(st));
+    CallFlags hf;
+    memcpy(&hf, t_pinned.out, sizeof(hf));
     if (!dev) {
-        if (o.edge_checks_out) *o.edge_checks_out = (int64_t)hchecks;
-        for (int i = 0; i < lc_len; ++i) o.level_counts_out[i] = (int64_t)hlc[i];
+        if (o.edge_checks_out) *o.edge_checks_out = (int64_t)hf.checks;
+        if (staged) {
+            if (lc_len) memcpy(o.level_counts_out, t_pinned.out + off_lc, sizeof(int64_t) * lc_len);
+            if (spread_out && spread_bytes) memcpy(spread_out, t_pinned.out + off_spread, spread_bytes);
+            if (count_out) memcpy(count_out, t_pinned.out + off_count, count_bytes);
+        }
     }
     if (hf.bad_seed) {
         set_error("%s: a seed id is out of range", fn);
