@@ -783,7 +783,8 @@ struct PushIc {
 };
 
 // IC push (k_push<0, PERWORD>).  A lane holds one (word, frontier bits) pair of the item's slot and goes
-// over the item's edges with it; a slot of k <= 16 pairs takes 32 / k edges at a time.  Per edge and
+// over the item's edges with it; 16 pairs and fewer (a small slot, or the end of a large one) are held
+// several times over, for as many edges at a time.  Per edge and
 // pair: c = f & ~vis_v[w]; the 4-trial blocks of c are queued and drawn by all lanes, one Philox block
 // each; drawing lanes or the rare live coins into their owner's word in shared memory.
 //
@@ -817,20 +818,21 @@ __device__ __forceinline__ void push_ic(Params &p) {
         const int deg = p.row_ptr[u + 1] - row0;
         const int e_begin = row0 + it.y;
         const int e_end = e_begin + min(edges_per_item(p, k), deg - it.y);
-        // lanes hold pairs; with k <= 16 several edges at a time, sub-th edge of each group per lane
-        const int per = k >= 32 ? 1 : 32 / k;
-        const int sub = k >= 32 ? 0 : lane / k;
         if (lane == 0) {
             n_edges += e_end - e_begin;
             n_fw += k;
         }
         for (int j0 = 0; j0 < k; j0 += 32) {
-            const int j = k >= 32 ? j0 + lane : lane - sub * k;
+            // the lanes hold up to 32 pairs; of 16 and fewer, several copies, each for an edge of its own
+            const int held = min(32, k - j0);
+            const int per = 32 / held;
+            const int sub = lane / held;
             uint64_t f = 0;
             int w = 0;
-            if (j < k && sub < per) {
-                f = p.in.pb[off + j];
-                w = (int)p.in.pw[off + j];
+            if (sub < per) {
+                const int j = off + j0 + lane - sub * held;
+                f = p.in.pb[j];
+                w = (int)p.in.pw[j];
             }
             __syncwarp();
             if (PERWORD) {
