@@ -18,15 +18,15 @@
 //
 // A warp takes up to 32 frontier nodes, spreads their out-edges over its lanes (a warp-wide or of the
 // rows' first positions gives each lane the node of its edge), and IC draws the coins of the (edge,
-// 4-trial block) pairs that need one: in place where no lane needs more than one, else from a per-warp
-// queue.  Rows of kHub edges and more are left to the whole block after the others.
+// 4-trial block) pairs that need one from a per-warp queue, 32 at a time.  Rows of kHub edges and more are
+// left to the whole block after the others.
 //
 // Columns are handed out by an atomic counter, since their depths differ.  What bounds a step is the
 // latency of its chain (row offsets, edges, target, coins, three shared-memory atomics, two barriers)
 // where its frontier is small, and issue slots where it is large (62 % issue active, ncu, on a dense
 // Watts-Strogatz 10k).  Against the pass engine's host step loop (GB300): G(1000, 10000), p = 0.1, 1,000
-// trials 1,710 -> 165 us per call, Watts-Strogatz 10k U[0, 1] 2,300 -> 650 us, CELF k = 10 on the
-// 7-regular graph (n = 5,000) 149 -> 21.8 ms.
+// trials 1,766 -> 126 us per call, Watts-Strogatz 10k U[0, 1] 2,184 -> 538 us, CELF k = 10 on the
+// 7-regular graph (n = 5,000) 146 -> 20.7 ms.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -70,9 +70,9 @@ struct ColParams {
     CallFlags *flags;
 };
 
+// Coin blocks to draw, a ring: {edge, threshold, target, (block << 4) | wanted trials of the block}.
 struct __align__(16) WarpQueue {
-    uint4 task[32];    // {edge, threshold, target, wanted trials} of each lane
-    uint8_t q[256];    // (lane << 3) | 4-trial block
+    uint4 q[64];
 };
 
 // The warp's frontier nodes that have edges to expand, in order: {edge id of the warp's t-th edge
@@ -120,6 +120,7 @@ struct StepCtx {
     const uint32_t *rk;
     uint64_t g0;
     uint32_t gained;  // activations of this thread in the step
+    uint32_t qh, qt;  // the warp's queued blocks: entries qh .. qt - 1 (mod 64)
 
     // v becomes active in the trials of `bits` where it is not yet
     __device__ __forceinline__ void activate(uint32_t v, uint32_t bits) {
@@ -155,7 +156,24 @@ __device__ __forceinline__ uint32_t coins(const StepCtx &s, uint32_t e, uint32_t
     return (uint32_t)(c0 < thr) | ((uint32_t)(c1 < thr) << 1) | ((uint32_t)(c2 < thr) << 2) | ((uint32_t)(c3 < thr) << 3);
 }
 
-// Expand one edge per lane, {v, thr} = ed, by the frontier bits f (0: nothing to do in this lane).
+// Draw the first cnt <= 32 queued blocks, one per lane.
+__device__ __forceinline__ void draw_queued(StepCtx &s, const WarpQueue &wq, uint32_t cnt) {
+    const uint32_t lane = threadIdx.x & 31;
+    __syncwarp();
+    if (lane < cnt) {
+        const uint4 t = wq.q[(s.qh + lane) & 63u];
+        const uint32_t j = t.w >> 4;
+        const uint32_t live = coins(s, t.x, t.y, j) & t.w & 15u;
+        if (live) s.activate(t.z, live << (4 * j));
+    }
+    s.qh += cnt;
+    __syncwarp();
+}
+
+// Expand one edge per lane, {v, thr} = ed, by the frontier bits f (0: nothing to do in this lane).  IC: the
+// 4-trial blocks with a trial to decide are queued, one per lane and round, and drawn 32 at a time; fewer than
+// 32 stay queued for the next edges (a chunk of 32 edges has 14 on average on a dense Watts-Strogatz 10k at 8
+// trials per column: drawn chunk by chunk, more than half of the lanes idle, a call took 603 us, now 538).
 template <int MODEL>
 __device__ __forceinline__ void expand(StepCtx &s, WarpQueue &wq, uint32_t e, uint2 ed, uint32_t f) {
     const int lane = threadIdx.x & 31;
@@ -177,40 +195,17 @@ __device__ __forceinline__ void expand(StepCtx &s, WarpQueue &wq, uint32_t e, ui
     }
     uint32_t nm = c | (c >> 1);
     nm = (nm | (nm >> 2)) & 0x11111111u;  // the 4-trial blocks to draw
-    const uint32_t d = __popc(nm);
-    if (!__any_sync(kFull, d > 1u)) {
-        // at most one block per lane: each lane draws its own
-        if (d) {
-            const uint32_t j = (uint32_t)(__ffs(nm) - 1) >> 2;
-            const uint32_t live = (coins(s, e, thr, j) << (4 * j)) & c;
-            if (live) s.activate(v, live);
+    for (;;) {
+        const uint32_t m = __ballot_sync(kFull, nm != 0u);
+        if (m == 0u) return;
+        if (nm) {
+            const uint32_t b = (uint32_t)__ffs(nm) - 1u;
+            nm &= nm - 1u;
+            wq.q[(s.qt + __popc(m & ((1u << lane) - 1u))) & 63u] = make_uint4(e, thr, v, (b << 2) | ((c >> b) & 15u));
         }
-        return;
+        s.qt += __popc(m);
+        if (s.qt - s.qh >= 32u) draw_queued(s, wq, 32u);
     }
-    // queue the blocks: positions from the ballots of the bits of d (0 .. 8)
-    const uint32_t lt = (1u << lane) - 1u;
-    uint32_t D = 0, r = 0;
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        const uint32_t b = __ballot_sync(kFull, (d >> k) & 1u);
-        D += (uint32_t)__popc(b) << k;
-        r += (uint32_t)__popc(b & lt) << k;
-    }
-    wq.task[lane] = make_uint4(e, thr, v, c);
-    while (nm) {
-        const int b = __ffs(nm) - 1;
-        nm &= nm - 1;
-        wq.q[r++] = (uint8_t)((lane << 3) | (b >> 2));
-    }
-    __syncwarp();
-    for (uint32_t i = lane; i < D; i += 32) {
-        const uint32_t ent = wq.q[i];
-        const uint4 t = wq.task[ent >> 3];
-        const uint32_t j = ent & 7u;
-        const uint32_t live = (coins(s, t.x, t.y, j) << (4 * j)) & t.w;
-        if (live) s.activate(t.z, live);
-    }
-    __syncwarp();
 }
 
 template <int MODEL>
@@ -336,7 +331,7 @@ __global__ void __launch_bounds__(1024, 1) k_columns(ColParams p) {
                 nx[u] = 0u;
             }
             __syncthreads();
-            StepCtx s{vis, nx, lnext, gnext, &S.n_list[nslot], cap, planes, p.edge, S.rk, g0, 0u};
+            StepCtx s{vis, nx, lnext, gnext, &S.n_list[nslot], cap, planes, p.edge, S.rk, g0, 0u, 0u, 0u};
             if (tid == 0) {
                 // the slots of the step after next: nobody reads or writes them in this one
                 S.n_list[(step + 2) % 3] = 0;
@@ -411,6 +406,7 @@ __global__ void __launch_bounds__(1024, 1) k_columns(ColParams p) {
                 }
                 __syncwarp();
             }
+            if (MODEL == 0 && s.qt != s.qh) draw_queued(s, wq, s.qt - s.qh);
             __syncthreads();
             const int H = min(S.n_hub[slot], kHubCap);
             if (H) {
@@ -421,6 +417,7 @@ __global__ void __launch_bounds__(1024, 1) k_columns(ColParams p) {
                         expand<MODEL>(s, wq, (uint32_t)(e + lane), e + lane < e1 ? __ldg(&p.edge[e + lane]) : make_uint2(0u, 0u),
                                       e + lane < e1 ? hb.y : 0u);
                 }
+                if (MODEL == 0 && s.qt != s.qh) draw_queued(s, wq, s.qt - s.qh);
                 __syncthreads();
             }
             if (step + 1 < p.lc_len) {
@@ -513,8 +510,10 @@ cnd_status plan_columns(int model, const cnd_graph_dev &G, const std::vector<Ite
     if (trials == 0) return CND_OK;
     // Blocks per SM and trials per column (a multiple of 4, one coin block), by estimated time: a
     // wave of columns takes a constant (the latency of its steps) and work in proportion to the
-    // trials (and 2 more: work that a check takes whatever its trials), at a rate in proportion to
-    // the block's threads.
+    // trials (and 2 more: work that a check takes whatever its trials) and the edges, at a rate in
+    // proportion to the block's threads.  1,000 trials, blocks per SM / trials per column: G(1000, 10000)
+    // 2 / 4 133 us, 1 / 8 148; Watts-Strogatz 10k U[0, 1] 2 / 4 648 us, 1 / 8 575; BA 5k WC 255 and 269.
+    const double size = std::min(1.0, std::max(0.25, (double)G.m / 1e5));
     ColShape c;
     double best = 1e300;
     for (int per_sm = 4; per_sm >= 1; per_sm >>= 1) {
@@ -522,7 +521,7 @@ cnd_status plan_columns(int model, const cnd_graph_dev &G, const std::vector<Ite
         if (!column_shape(model, G, per_sm, k)) continue;
         for (int b = 4; b <= 32; b += 4) {
             const double waves = std::ceil((double)((trials + b - 1) / b) / ((double)G.num_sms * per_sm));
-            const double cost = waves * (8 + per_sm * (b + 2));
+            const double cost = waves * ((per_sm == 1 ? 10 : per_sm == 2 ? 9 : 8) + size * per_sm * (b + 2));
             if (cost < best) {
                 best = cost;
                 plan.bits = b;
