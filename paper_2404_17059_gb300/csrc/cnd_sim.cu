@@ -1558,9 +1558,10 @@ __global__ void __launch_bounds__(kBlock, 3) k_pull_lt(Params p_) {
 // checks; a pull step the scan of all m in-edges and, for every in-edge from the frontier, a row of all
 // B words whether they carry bits or not.  Measured on GB300 (ms per call, push only / pull above
 // checks = m / 3 m / 6 m): R-MAT-21, B = 16: 384 / 154 / 160 / 187; B = 64: 1,470 / 484 / 455 / 446;
-// B = 1: 51.1 / 50.8 (52.1 above 0.3 m); BA 100k, B = 157: 54.7 / 37.8 / 35.4 / 33.8; B = 16: 8.5 / 6.65 / 6.8.
+// B = 1: 51.7 above m, 48.1 / 50.3 above 0.67 m / 0.33 m; BA 100k, B = 157: 54.7 / 37.8 / 35.4 / 33.8;
+// B = 16: 8.5 / 6.65 / 6.8.
 __host__ __device__ __forceinline__ bool lt_pull_pays(unsigned long long checks, int64_t m, int32_t B) {
-    return checks * 12ull > (unsigned long long)m * (unsigned long long)(B > 12 ? B : 12);
+    return checks * 12ull > (unsigned long long)m * (unsigned long long)(B > 8 ? B : 8);
 }
 
 // ---------------------------------------------------------------- device step loop
