@@ -684,6 +684,108 @@ __global__ void __launch_bounds__(kBlock) k_collect(Params p_) {
     add_level_count(p, pc);
 }
 
+// The same for passes of more than kCollectNq dirty-mask words (B up to kMaxB; a node's words hardly fit a
+// lane each).  A warp takes kWideNodesPerWarp listed nodes, lane q holding mask word q of each, places their
+// slots, pool pairs and work items with one atomic each, and goes over a node's words 128 at a time, four
+// coalesced loads of nxt per lane in flight.  Moves 26 bytes per pair; against the block-cooperative
+// finalize, whose lanes search the mask for their words: 35.9 ms ->
+// 5.7 ms a call for 530 words on R-MAT-20; at 157 words k_collect is the faster (2.07 against 3.81 ms a
+// call on BA 100k).
+constexpr int kWideNodesPerWarp = 4;
+
+__global__ void __launch_bounds__(kBlock) k_collect_wide(Params p_) {
+    Params p = p_;
+    resolve(p);
+    constexpr int NN = kWideNodesPerWarp;
+    const int lane = lane_id();
+    const unsigned below = (1u << lane) - 1u;
+    const int count = *p.lin_cnt;
+    const int B = p.B, nq = p.nq;
+    const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int n_warps = (gridDim.x * blockDim.x) >> 5;
+    unsigned long long pc = 0;
+    for (int base = warp * NN; base < count; base += n_warps * NN) {
+        int v[NN], K[NN], deg[NN];
+        uint64_t dm[NN];
+#pragma unroll
+        for (int h = 0; h < NN; ++h) {
+            v[h] = base + h < count ? p.lin[base + h] : -1;
+            dm[h] = 0ull;
+            if (v[h] >= 0 && lane < nq) {
+                uint64_t *d = p.dmask + (size_t)v[h] * nq + lane;
+                dm[h] = *d;
+                if (dm[h]) *d = 0ull;
+            }
+        }
+        int pairs = 0, slots = 0, items = 0, edges = 0;
+        unsigned long long checks = 0;
+#pragma unroll
+        for (int h = 0; h < NN; ++h) {
+            K[h] = __reduce_add_sync(kFull, __popcll(dm[h]));
+            deg[h] = K[h] ? p.row_ptr[v[h] + 1] - p.row_ptr[v[h]] : 0;
+            const int ne = edges_per_item(p, K[h]);
+            pairs += K[h];
+            slots += K[h] > 0;
+            items += (deg[h] + ne - 1) / ne;
+            edges += deg[h];
+            checks += (unsigned long long)deg[h] * (unsigned)K[h];
+        }
+        if (pairs == 0) continue;
+        unsigned long long ps0 = 0;
+        int item0 = 0;
+        if (lane == 0) {
+            ps0 = atomicAdd((unsigned long long *)p.out.cnt, ((unsigned long long)slots << 32) | (unsigned)pairs);
+            if (items) item0 = atomicAdd(&p.out.cnt[2], items);
+            if (edges) {
+                atomicAdd(&p.out.cnt[3], edges);
+                atomicAdd((unsigned long long *)(p.out.cnt + 4), checks);
+            }
+        }
+        ps0 = __shfl_sync(kFull, ps0, 0);
+        item0 = __shfl_sync(kFull, item0, 0);
+        int off = (int)(uint32_t)ps0, slot = (int)(ps0 >> 32);
+#pragma unroll
+        for (int h = 0; h < NN; ++h) {
+            if (K[h] == 0) continue;
+            if (lane == 0) {
+                p.out.node[slot] = v[h];
+                p.out.poff[slot] = off;
+                p.out.pk[slot] = K[h];
+            }
+            const int ne = edges_per_item(p, K[h]);
+            const int nch = (deg[h] + ne - 1) / ne;
+            for (int c = lane; c < nch; c += 32) p.out.work[item0 + c] = make_int2(slot, c * ne);
+            item0 += nch;
+            ++slot;
+            uint64_t *row = p.nxt + (size_t)v[h] * B;
+            for (int q = 0; q < nq; q += 2) {  // 128 words: two mask words, four 32-word groups
+                const uint64_t d0 = __shfl_sync(kFull, dm[h], q);
+                const uint64_t d1 = __shfl_sync(kFull, dm[h], (q + 1) & 31);
+                const uint32_t m[4] = {(uint32_t)d0, (uint32_t)(d0 >> 32), q + 1 < nq ? (uint32_t)d1 : 0u,
+                                       q + 1 < nq ? (uint32_t)(d1 >> 32) : 0u};
+                if ((m[0] | m[1] | m[2] | m[3]) == 0u) continue;
+                uint64_t x[4];
+#pragma unroll
+                for (int g = 0; g < 4; ++g)
+                    x[g] = (m[g] >> lane) & 1u ? (uint64_t)__ldcg((const unsigned long long *)row + 64 * q + 32 * g + lane) : 0ull;
+#pragma unroll
+                for (int g = 0; g < 4; ++g) {
+                    if ((m[g] >> lane) & 1u) {
+                        const int w = 64 * q + 32 * g + lane;
+                        const int at = off + __popc(m[g] & below);
+                        row[w] = 0ull;
+                        p.out.pw[at] = (uint16_t)w;
+                        p.out.pb[at] = x[g];
+                        pc += __popcll(x[g]);
+                    }
+                    off += __popc(m[g]);
+                }
+            }
+        }
+    }
+    add_level_count(p, pc);
+}
+
 // ---------------------------------------------------------------- LT counting form
 // Set-up of a pass in the counting form (every node's non-zero in-weights equal w_v).  With k
 // active in-neighbours, v activates iff k * w_v > theta, i.e. iff k > q = floor(theta / w_v).
@@ -1690,6 +1792,13 @@ static cudaError_t launch(const void *fn, int blocks, cudaStream_t st, Params &p
     return cudaLaunchKernel(fn, dim3(blocks), dim3(kBlock), args, 0, st);
 }
 
+// The frontier collect of a pass of nq dirty-mask words per node, when no word waits.
+static const void *collect_fn(int nq) {
+    return nq == 1            ? (const void *)k_collect<true>
+           : nq <= kCollectNq ? (const void *)k_collect<false>
+                              : (const void *)k_collect_wide;
+}
+
 static int resident_blocks(const void *fn) {
     int b = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, fn, kBlock, 0) != cudaSuccess || b < 1) b = 1;
@@ -2050,13 +2159,12 @@ static cnd_status run_items(int model, const cnd_graph_dev &G, const char *fn, s
     const void *k_fin_uk = model == 0 ? (const void *)k_finalize<1, false>
                            : lt_cnt   ? (const void *)k_finalize<1, false>
                                       : (const void *)k_finalize<2, false>;
-    // nothing waits and a node's words fit one dirty-mask word: the barrier-free collect
-    const bool flat = P.tau == 0 && nq <= kCollectNq;
-    const void *k_col = nq == 1 ? (const void *)k_collect<true> : (const void *)k_collect<false>;
-    if (flat && (model == 0 || lt_cnt)) k_fin_pw = k_fin_uk = k_col;
+    // nothing waits: the barrier-free collects
+    const void *k_col = collect_fn(nq);
+    if (P.tau == 0 && (model == 0 || lt_cnt)) k_fin_pw = k_fin_uk = k_col;
     const void *k_init_pw = (const void *)k_lt_init<true>, *k_init_uk = (const void *)k_lt_init<false>;
     const int init_blocks = G.num_sms * resident_blocks(k_init_uk);
-    const void *k_seedfin = nq <= kCollectNq ? k_col : (const void *)k_finalize<1, false>;
+    const void *k_seedfin = k_col;
     const int push_blocks = G.num_sms * resident_blocks(k_push_uk);
     const void *k_pull_fn_lt = B <= 16 ? (const void *)k_pull_lt<8> : (const void *)k_pull_lt<16>;
     const void *k_pull_pw = model == 0 ? (const void *)k_pull_ic<true> : k_pull_fn_lt;
@@ -2957,10 +3065,7 @@ static cnd_status simulate_noalloc(const cnd_graph *g, const int32_t *seeds, int
         CND_CUDA_TRY(cudaMemsetAsync(P.nxt, 0, sizeof(uint64_t) * nB, st));
         CND_CUDA_TRY(cudaMemsetAsync(P.dmask, 0, sizeof(uint64_t) * (size_t)n * nq, st));
         const void *k_push_fn = (const void *)k_push<0, false>;
-        // nothing waits here (tau = 0): the barrier-free collect where a node's words fit its masks
-        const void *k_fin_fn = nq == 1 ? (const void *)k_collect<true>
-                               : nq <= kCollectNq ? (const void *)k_collect<false>
-                                                  : (const void *)k_finalize<1, false>;
+        const void *k_fin_fn = collect_fn(nq);  // nothing waits here (tau = 0)
         const int push_blocks = G.num_sms * resident_blocks(k_push_fn);
         const int fin_blocks = G.num_sms * resident_blocks(k_fin_fn);
         uint64_t desc[2 * kMaxB + 2];  // valid[B] | wout[B] | one seed run
