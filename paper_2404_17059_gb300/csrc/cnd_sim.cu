@@ -688,9 +688,8 @@ __global__ void __launch_bounds__(kBlock) k_collect(Params p_) {
 // lane each).  A warp takes kWideNodesPerWarp listed nodes, lane q holding mask word q of each, places their
 // slots, pool pairs and work items with one atomic each, and goes over a node's words 128 at a time, four
 // coalesced loads of nxt per lane in flight.  Moves 26 bytes per pair; against the block-cooperative
-// finalize, whose lanes search the mask for their words: 35.9 ms ->
-// 5.7 ms a call for 530 words on R-MAT-20; at 157 words k_collect is the faster (2.07 against 3.81 ms a
-// call on BA 100k).
+// finalize, whose lanes search the mask for their words: 35.9 ms -> 5.7 ms a call for 530 words on R-MAT-20;
+// at 157 words k_collect is the faster (2.07 against 3.81 ms a call on BA 100k).
 constexpr int kWideNodesPerWarp = 4;
 
 __global__ void __launch_bounds__(kBlock) k_collect_wide(Params p_) {
@@ -1727,63 +1726,157 @@ __global__ void k_ctl(Params p, cudaGraphConditionalHandle h, int32_t first, int
 }
 
 // ---------------------------------------------------------------- outputs
-// Per-trial spread: warp k of a block owns word w and reduces 32 nodes at a
-// time with one ballot per trial bit; trial b of word w lands at
-// spread[wout[w] + b] (wout < 0: the word holds no trials).
-__global__ void __launch_bounds__(256) k_spread(const uint64_t *__restrict__ vis, int32_t n, int32_t B,
-                                                int32_t nwords, int32_t nodes_per_block,
-                                                const int64_t *__restrict__ wout, int32_t *__restrict__ spread) {
-    const int lane = threadIdx.x & 31;
-    const int w = blockIdx.x * 8 + (threadIdx.x >> 5);
-    if (w >= nwords) return;
-    const int64_t out = wout[w];
-    if (out < 0) return;
-    const int v0 = blockIdx.y * nodes_per_block;
-    const int v1 = min(n, v0 + nodes_per_block);
-    uint32_t lo = 0, hi = 0;
-    for (int vb = v0; vb < v1; vb += 32) {
-        const int v = vb + lane;
-        const uint64_t x = (v < v1) ? __ldcs((const unsigned long long *)vis + (size_t)v * B + w) : 0ull;
-        const uint32_t xl = (uint32_t)x, xh = (uint32_t)(x >> 32);
-#pragma unroll
-        for (int b = 0; b < 32; ++b) {
-            const uint32_t ml = __ballot_sync(kFull, (xl >> b) & 1u);
-            const uint32_t mh = __ballot_sync(kFull, (xh >> b) & 1u);
-            if (lane == b) {
-                lo += __popc(ml);
-                hi += __popc(mh);
-            }
-        }
-    }
-    if (lo) atomicAdd(&spread[out + lane], (int)lo);
-    if (hi) atomicAdd(&spread[out + 32 + lane], (int)hi);
+// Per-trial spread of a pass.  Bound by one read of vis.  A lane holds one word column and adds its rows as
+// bits, not as numbers: a carry-save tree takes eight rows (seven 3-in-2-out adders, four LOP3 each) and
+// ripples the eights into the upper bit planes, 3.5 instructions per 64 trials, and only at the end of the
+// strip are the kSpreadPlanes planes spelled out as 64 counts.  Lanes are consecutive words (of one row, or of
+// several rows where a row has fewer than 32), so every load is one full line per row; the block's eight
+// strips meet in shared memory and leave with one atomic per trial.  With a ballot per trial and a warp per
+// word before, 405 -> 36 us (BA 100k, 157 words), 690 -> 55 us (R-MAT-21, 16 words), 8.14 -> 0.66 ms
+// (R-MAT-20, 530 words: 6.7 TB/s).
+constexpr int kSpreadPlanes = 10;
+constexpr int kSpreadRows = 1016;  // rows a lane may add: a multiple of 8 below 2^kSpreadPlanes
+static_assert(kSpreadRows % 8 == 0 && kSpreadRows < (1 << kSpreadPlanes), "a strip's counts fit the planes");
+
+__device__ __forceinline__ uint64_t csa(uint64_t &s, uint64_t b, uint64_t c) {  // s += b + c; the carries
+    const uint64_t a = s;
+    s = a ^ b ^ c;
+    return (a & b) | (a & c) | (b & c);
 }
 
-// Per-node activation counts (accumulated over passes) and edge checks; one
-// warp per node, lanes over words.  witem == null: one count row; else the
-// count of word w goes to row witem[w] (one row per batch item).
-__global__ void __launch_bounds__(256) k_counts(const uint64_t *__restrict__ vis, int32_t n, int32_t B,
+__global__ void __launch_bounds__(256, 4) k_spread(const uint64_t *__restrict__ vis, int32_t n, int32_t B,
+                                                   int32_t nwords, int32_t rows, const int64_t *__restrict__ wout,
+                                                   int32_t *__restrict__ spread) {
+    __shared__ int s_cnt[32][65];
+    const int lane = threadIdx.x & 31;
+    const int span = min(B, 32), per = 32 / span;  // words of a row a warp holds, rows it reads at once
+    const int sub = lane / span, wl = lane - sub * span;
+    const int w = blockIdx.y * 32 + wl;
+    for (int i = threadIdx.x; i < 32 * 65; i += 256) (&s_cnt[0][0])[i] = 0;
+    __syncthreads();
+    const int64_t first = ((int64_t)blockIdx.x * 8 + (threadIdx.x >> 5)) * rows * per;
+    if (sub < per && w < nwords && first < n) {
+        const int mine = (int)min((int64_t)rows, ((int64_t)n - first - sub + per - 1) / per);  // rows of this lane
+        const unsigned long long *at = (const unsigned long long *)vis + (size_t)(first + sub) * B + w;
+        const size_t step = (size_t)per * B;
+        uint64_t p[kSpreadPlanes];
+#pragma unroll
+        for (int k = 0; k < kSpreadPlanes; ++k) p[k] = 0ull;
+        for (int r = 0; r < mine; r += 8, at += 8 * step) {
+            uint64_t x[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) x[i] = r + i < mine ? (uint64_t)__ldcs(at + i * step) : 0ull;
+            const uint64_t a = csa(p[0], x[0], x[1]), b = csa(p[0], x[2], x[3]);
+            const uint64_t c = csa(p[0], x[4], x[5]), d = csa(p[0], x[6], x[7]);
+            const uint64_t e = csa(p[1], a, b), f = csa(p[1], c, d);
+            uint64_t up = csa(p[2], e, f);
+#pragma unroll
+            for (int k = 3; k < kSpreadPlanes; ++k) {
+                const uint64_t t = p[k] & up;
+                p[k] ^= up;
+                up = t;
+            }
+        }
+        // lanes of one word start at different trials, so that they do not add to one counter together
+        const int turn = sub * (64 / per);
+#pragma unroll
+        for (int k = 0; k < kSpreadPlanes; ++k) p[k] = (p[k] >> turn) | (p[k] << ((64 - turn) & 63));
+#pragma unroll
+        for (int b = 0; b < 64; ++b) {
+            uint32_t c = 0;
+#pragma unroll
+            for (int k = 0; k < kSpreadPlanes; ++k) {
+                const uint32_t h = (uint32_t)(p[k] >> (b & 32));
+                c |= ((b & 31) >= k ? h >> ((b & 31) - k) : h << (k - (b & 31))) & (1u << k);
+            }
+            if (c) atomicAdd(&s_cnt[wl][(b + turn) & 63], (int)c);
+        }
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < 32 * 64; i += 256) {
+        const int c = s_cnt[i >> 6][i & 63];
+        if (c) {  // only words with trials hold bits
+            const int64_t out = wout[blockIdx.y * 32 + (i >> 6)];
+            if (out >= 0) atomicAdd(&spread[out + (i & 63)], c);
+        }
+    }
+}
+
+// Four blocks per SM, and strips no shorter than the spelling out of the counts (some 150 rows' worth) asks for.
+static cudaError_t launch_spread(const cnd_graph_dev &G, cudaStream_t st, const uint64_t *vis, int32_t B, int32_t nwords,
+                                 const int64_t *wout, int32_t *spread) {
+    const int64_t groups = (nwords + 31) / 32, per = 32 / std::min(B, 32);
+    const int64_t steps = ((int64_t)G.n + per - 1) / per;  // of one row per lane
+    const int64_t strips = std::max<int64_t>(1, (int64_t)G.num_sms * 4 * 8 / groups);
+    const int64_t rows = std::min<int64_t>(kSpreadRows, std::max<int64_t>(64, ((steps + strips - 1) / strips + 7) / 8 * 8));
+    const dim3 grid((unsigned)((steps + 8 * rows - 1) / (8 * rows)), (unsigned)groups);
+    k_spread<<<grid, 256, 0, st>>>(vis, G.n, B, nwords, (int32_t)rows, wout, spread);
+    return cudaGetLastError();
+}
+
+// Per-node activation counts (accumulated over passes) and edge checks.  Bound by one read of vis: 2^lg lanes
+// hold a node's words (a whole warp from 17 words on), so that no lane idles over narrow passes, and a warp
+// has the rows of kCountRows * 32 / 2^lg nodes in flight.  witem == null: one count row; else the count of
+// word w goes to row witem[w] (one row per batch item).  One node per warp and load before: 38 -> 27 us,
+// 203 -> 87 us and 833 -> 572 us on the three cases of k_spread (4 rows: 28, 99, 610 us).
+constexpr int kCountRows = 8;
+
+__global__ void __launch_bounds__(256, 4) k_counts(const uint64_t *__restrict__ vis, int32_t n, int32_t B, int32_t lg,
                                                 const int32_t *__restrict__ row_ptr, const int32_t *__restrict__ witem,
                                                 int32_t *__restrict__ count, unsigned long long *__restrict__ checks) {
     const int lane = threadIdx.x & 31;
-    const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int n_warps = (gridDim.x * blockDim.x) >> 5;
+    const int64_t warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int64_t n_warps = (gridDim.x * blockDim.x) >> 5;
+    const int ln = 1 << lg, per = 32 >> lg;
+    const int sub = lane >> lg, l = lane & (ln - 1);
     unsigned long long ck = 0;
-    for (int v = warp; v < n; v += n_warps) {
-        int s = 0;
-        for (int w = lane; w < B; w += 32) {
-            const int c = __popcll(__ldcs((const unsigned long long *)vis + (size_t)v * B + w));
-            s += c;
-            if (witem && c && count) atomicAdd(&count[(size_t)witem[w] * n + v], c);
-        }
+    for (int64_t base = warp * per * kCountRows; base < n; base += n_warps * per * kCountRows) {
+        int s[kCountRows];
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(kFull, s, o);
-        if (lane == 0 && s) {
-            if (!witem && count) count[v] += s;
-            ck += (unsigned long long)s * (unsigned long long)(row_ptr[v + 1] - row_ptr[v]);
+        for (int u = 0; u < kCountRows; ++u) s[u] = 0;
+        for (int w = l; w < B; w += ln) {
+            const int it = witem && count ? witem[w] : 0;
+            uint64_t x[kCountRows];
+#pragma unroll
+            for (int u = 0; u < kCountRows; ++u) {
+                const int64_t v = base + u * per + sub;
+                x[u] = v < n ? (uint64_t)__ldcs((const unsigned long long *)vis + (size_t)v * B + w) : 0ull;
+            }
+#pragma unroll
+            for (int u = 0; u < kCountRows; ++u) {
+                const int c = __popcll(x[u]);
+                s[u] += c;
+                if (witem && c && count) atomicAdd(&count[(size_t)it * n + base + u * per + sub], c);
+            }
         }
+        __syncwarp();
+#pragma unroll
+        for (int u = 0; u < kCountRows; ++u)
+            for (int o = ln >> 1; o > 0; o >>= 1) s[u] += __shfl_xor_sync(kFull, s[u], o);
+        for (int u = l; u < kCountRows; u += ln) {  // a node's sum is in all of its lanes: a row for each
+            int mine = 0;
+#pragma unroll
+            for (int k = 0; k < kCountRows; ++k) mine = k == u ? s[k] : mine;
+            const int64_t v = base + u * per + sub;
+            if (mine) {  // rows past the last node hold none
+                ck += (unsigned long long)mine * (unsigned long long)(row_ptr[v + 1] - row_ptr[v]);
+                if (!witem && count) count[v] += mine;
+            }
+        }
+        __syncwarp();
     }
+    for (int o = 16; o > 0; o >>= 1) ck += __shfl_xor_sync(kFull, ck, o);
     if (lane == 0 && ck) atomicAdd(checks, ck);
+}
+
+static cudaError_t launch_counts(const cnd_graph_dev &G, cudaStream_t st, const uint64_t *vis, int32_t B, const int32_t *witem,
+                                 int32_t *count, unsigned long long *checks) {
+    int32_t lg = 0;
+    while (lg < 5 && (1 << lg) < B) ++lg;
+    const int64_t per_block = (int64_t)8 * kCountRows * (32 >> lg);
+    const int64_t blocks = std::min<int64_t>((int64_t)G.num_sms * 4, ((int64_t)G.n + per_block - 1) / per_block);
+    k_counts<<<(unsigned)std::max<int64_t>(1, blocks), 256, 0, st>>>(vis, G.n, B, lg, G.row_ptr, witem, count, checks);
+    return cudaGetLastError();
 }
 
 // ---------------------------------------------------------------- dispatch
@@ -2299,13 +2392,8 @@ static cnd_status run_items(int model, const cnd_graph_dev &G, const char *fn, s
             cur = nx;
         }
         // outputs of this pass
-        const int npb = 4096;
-        dim3 grid((unsigned)((nw_here + 7) / 8), (unsigned)((n + npb - 1) / npb));
-        k_spread<<<grid, 256, 0, st>>>(P.vis, n, B, nw_here, npb, d_wout, d_spread);
-        CND_CUDA_TRY(cudaGetLastError());
-        k_counts<<<blocks_for(n, G.num_sms * 8), 256, 0, st>>>(P.vis, n, B, G.row_ptr, batched ? d_witem : nullptr,
-                                                                d_count, d_checks);
-        CND_CUDA_TRY(cudaGetLastError());
+        CND_CUDA_TRY(launch_spread(G, st, P.vis, B, nw_here, d_wout, d_spread));
+        CND_CUDA_TRY(launch_counts(G, st, P.vis, B, batched ? d_witem : nullptr, d_count, d_checks));
         launches += 2;
     }
     if (graph_mode) {
@@ -2417,13 +2505,8 @@ static cnd_status run_items(int model, const cnd_graph_dev &G, const char *fn, s
             tail.assign(1, loop_node);
             // outputs of the pass
             CND_CUDA_TRY(cap_begin(gr.g, tail));
-            const int npb = 4096;
-            dim3 grid((unsigned)((nw_here + 7) / 8), (unsigned)((n + npb - 1) / npb));
-            k_spread<<<grid, 256, 0, cs>>>(P.vis, n, B, nw_here, npb, pass_wout(pass), d_spread);
-            k_counts<<<blocks_for(n, G.num_sms * 8), 256, 0, cs>>>(P.vis, n, B, G.row_ptr,
-                                                                    batched ? pass_witem(pass) : nullptr, d_count,
-                                                                    d_checks);
-            CND_CUDA_TRY(cudaGetLastError());
+            CND_CUDA_TRY(launch_spread(G, cs, P.vis, B, nw_here, pass_wout(pass), d_spread));
+            CND_CUDA_TRY(launch_counts(G, cs, P.vis, B, batched ? pass_witem(pass) : nullptr, d_count, d_checks));
             CND_CUDA_TRY(cap_end(&tail));
             launches += 6;
         }
@@ -3114,13 +3197,8 @@ static cnd_status simulate_noalloc(const cnd_graph *g, const int32_t *seeds, int
                 CND_CUDA_TRY(launch(k_fin_fn, fin_blocks, st, P));
                 cur = nx;
             }
-            const int npb = 4096;
-            dim3 grid((unsigned)((nw_here + 7) / 8), (unsigned)((n + npb - 1) / npb));
-            k_spread<<<grid, 256, 0, st>>>(P.vis, n, B, (int)nw_here, npb, d_wout, spread_out);
-            CND_CUDA_TRY(cudaGetLastError());
-            k_counts<<<blocks_for(n, G.num_sms * 8), 256, 0, st>>>(P.vis, n, B, G.row_ptr, nullptr, count_out,
-                                                                    d_checks);
-            CND_CUDA_TRY(cudaGetLastError());
+            CND_CUDA_TRY(launch_spread(G, st, P.vis, B, (int32_t)nw_here, d_wout, spread_out));
+            CND_CUDA_TRY(launch_counts(G, st, P.vis, B, nullptr, count_out, d_checks));
         }
     }
     int32_t hbad = 0;

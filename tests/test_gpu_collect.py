@@ -31,3 +31,14 @@ def test_wide_pass(graph, words, model, captured):
     b = oracle.simulate_threads(model, g, seeds, T, 5, level_counts_len=12, **kw)
     assert np.array_equal(a.spread, b.spread) and np.array_equal(a.node_count, b.node_count)
     assert a.edge_checks == b.edge_checks and np.array_equal(a.level_counts, b.level_counts)
+
+
+@pytest.mark.parametrize("n,words", [(5_000_003, 33), (1_300_001, 2), (300_001, 31), (70_001, 1), (40_007, 257)])
+def test_full_counters(n, words):
+    """Every node active in every trial: spreads and counts of strips up to their longest, all words full."""
+    row_ptr = np.full(n + 1, n - 1, dtype=np.int32)
+    row_ptr[0] = 0
+    G = P.cnd_graph_create(n, row_ptr, np.arange(1, n, dtype=np.int32), np.ones(n - 1, np.float32), None)
+    T = 64 * words - 1
+    a = P.cnd_ic_simulate_ex(G, np.zeros(1, np.int32), T, 3, edge_checks=True)
+    assert (a.spread == n).all() and (a.node_count == T).all() and a.edge_checks == T * (n - 1)
