@@ -18,7 +18,7 @@
 // trials, and those trials are scattered over its words; the frontier keeps
 // only the words that carry bits: a list of slots (node, pair offset, pair
 // count) over a pool of (word index, frontier bits) pairs.  Work items
-// (slot, edge offset) cover about kTasks (edge, pair) tasks each, and a warp
+// (slot, edge offset) cover about kTasks (LT: kLtTasks) (edge, pair) tasks each, and a warp
 // spreads the tasks of an item evenly over its lanes, so hubs are split over
 // many warps and no lane idles on empty words.
 //
@@ -64,7 +64,17 @@ constexpr int kMaxB = 2048;  // words per node per pass (dirty mask: one 64-bit 
 constexpr int kPushMinBlocks = 8;
 constexpr int kStageB = 64;  // pairs of a push work item staged in shared memory (more: read from the pool)
 constexpr int kPullMaxB = 256;  // words per node the pull kernel keeps in registers
-constexpr int kTasks = 256;  // (edge, pair) tasks per push work item
+constexpr int kTasks = 256;  // (edge, pair) tasks per push work item of IC
+// ... of LT: a lane runs its tasks one after the other, and with few items per warp the step ends with most
+// warps idle (256 / 128 / 64 / 32 tasks: R-MAT-17 with uneven weights 27.0 / 24.9 / 24.7 / 25.6 ms per call,
+// BA 100k 30.3 / 29.3 / 28.8 / 28.2, R-MAT-21 135 / 129 / 127 / 127; two tasks per lane at once are slower).
+// IC's lanes hold the pairs instead and lose by it: BA 100k 18.8 / 19.8 / 20.7 / 21.0, R-MAT-21 47.5 / 48.3 /
+// 50.9 / 57.1.
+constexpr int kLtTasks = 64;
+// Passes of the accumulate form wider than this stay with kTasks: their rows of 64 counters outgrow the L2, and
+// small items spread a step over more of them (R-MAT-18, uneven weights, kTasks / kLtTasks: 16 words 59.6 /
+// 56.8 ms, 24 words 84.1 / 84.7, 32 words 108.6 / 110.7, 63 words 219 / 234).
+constexpr int kLtAccWords = 16;
 // ... of a slot of more than 32 pairs in an IC pass of more than 256 words on a graph of kWideNodes nodes
 // and more: its lanes go over the item's edges with the pairs they hold, so more edges per item pay
 // while a step has items enough for all warps (16 seed sets on R-MAT-20, 424 words: 515 / 482 / 472 ms per
@@ -112,6 +122,7 @@ __device__ __forceinline__ unsigned long long global_ns() {
 struct Params {
     int32_t n, B, nq;
     int32_t chunk;             // > 0: fixed edges per work item
+    int32_t tasks;             // else: (edge, pair) tasks per work item of a slot of up to 32 pairs
     int32_t wide;              // tasks per work item of a slot with more than 32 pairs
     const int32_t *row_ptr;
     const uint2 *edge;         // {col, IC threshold} or {col, LT weight}
@@ -193,7 +204,7 @@ __device__ __forceinline__ void add_level_count(const Params &p, unsigned long l
 
 // Edges per work item for a slot with k pairs.
 __device__ __forceinline__ int edges_per_item(const Params &p, int k) {
-    return p.chunk > 0 ? p.chunk : max(1, (k > 32 ? p.wide : kTasks) / max(k, 1));
+    return p.chunk > 0 ? p.chunk : max(1, (k > 32 ? p.wide : p.tasks) / max(k, 1));
 }
 
 // t / k for t < 2^32 / k (k <= kMaxB): multiply by ceil-ish reciprocal.
@@ -2057,9 +2068,12 @@ static cnd_status run_items(int model, const cnd_graph_dev &G, const char *fn, s
     size_t free_b = 0, total_b = 0;
     CND_CUDA_TRY(cudaMemGetInfo(&free_b, &total_b));
     const double budget = 0.6 * (double)free_b;
-    // bytes per word column: vis, nxt, two pair pools (+ LT accumulators or counter planes)
+    // bytes per word column: vis, nxt, two pair pools (+ LT accumulators or counter planes, and what its work
+    // items take more than IC's)
+    const int tasks_min = model == 0 ? kTasks : kLtTasks;
     const double per_word = (double)n * (2 * 8 + 2 * 10 + (model == 1 && !lt_cnt ? 256 : 0)) +
-                            (lt_cnt ? 8.0 * (double)G.lt_planes : 0.0);
+                            (lt_cnt ? 8.0 * (double)G.lt_planes : 0.0) +
+                            (o.chunk_edges > 0 ? 0.0 : 32.0 * (double)G.m * (1.0 / tasks_min - 1.0 / kTasks));
     // IC pulls only when asked to: by direction, or by a switch threshold; LT in the counting form
     // chooses per step (lt_pull_pays)
     const bool lt_pull = lt_cnt && G.m > 0 && o.direction != CND_DIR_PUSH && o.defer_bits == 0;
@@ -2070,6 +2084,8 @@ static cnd_status run_items(int model, const cnd_graph_dev &G, const char *fn, s
     bmax = std::min<int64_t>(bmax, std::max<int64_t>(1, (int64_t)(budget / per_word)));
     bmax = std::min<int64_t>(bmax, ic_pull ? kPullMaxB : kMaxB);
     bmax = std::min<int64_t>(bmax, std::max<int64_t>(1, (int64_t)0x7FFFFFFF / std::max(n, 1)));
+    if (model == 1 && G.m > 0)  // a step's work items are counted in 32 bits
+        bmax = std::min<int64_t>(bmax, std::max<int64_t>(1, (0x7FFFFFFFll - n - G.m) * tasks_min / (2 * (int64_t)G.m)));
     const int64_t n_pass = (total_words + bmax - 1) / bmax;
     const int B = (int)((total_words + n_pass - 1) / n_pass);
     const int nq = (B + 63) / 64;
@@ -2101,14 +2117,16 @@ static cnd_status run_items(int model, const cnd_graph_dev &G, const char *fn, s
 
     const size_t nB = (size_t)n * B;
     const int chunk = std::min(o.chunk_edges, 16384);  // task index < 2^32 / k in k_push's division
+    const int tasks = model == 0 || (!lt_cnt && B > kLtAccWords) ? kTasks : kLtTasks;
     const size_t work_cap = chunk > 0 ? (size_t)n + (size_t)G.m / chunk + 1
-                                      : (size_t)n + 2 * (size_t)G.m * (size_t)B / kTasks + (size_t)G.m + 1;
+                                      : (size_t)n + 2 * (size_t)G.m * (size_t)B / tasks + (size_t)G.m + 1;
     Params P{};
     P.n = n;
     P.B = B;
     P.nq = nq;
     P.chunk = chunk;
-    P.wide = model == 0 && B > 256 && n >= kWideNodes ? kWideTasks : kTasks;
+    P.tasks = tasks;
+    P.wide = model == 0 && B > 256 && n >= kWideNodes ? kWideTasks : tasks;
     P.row_ptr = G.row_ptr;
     P.edge = edge;
     P.rk = round_keys(items[0].key);
@@ -3133,7 +3151,7 @@ static cnd_status simulate_noalloc(const cnd_graph *g, const int32_t *seeds, int
         P.B = B;
         P.nq = nq;
         P.chunk = 0;
-        P.wide = kTasks;
+        P.tasks = P.wide = kTasks;
         P.tau = 0;
         P.max_wait = 0;
         P.force = 0;
