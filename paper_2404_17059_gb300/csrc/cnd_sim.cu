@@ -33,8 +33,12 @@
 //              (counting form: one bit-sliced increment of v's counter word by
 //              the trials of f & ~vis_v[w]; a carry out of the top plane is
 //              the activation, see k_lt_init)
+//   LT pull    counting form, steps whose frontier is dense: every node with
+//              open trials counts its in-neighbours in the frontier
+//              (k_frontier_rows, k_pull_lt)
 //   collect    per listed node: IC and the LT counting form take the dirty
-//              words of nxt (k_collect; k_finalize where words wait); the LT
+//              words of nxt (k_collect, k_collect_wide above 256 words;
+//              k_finalize where words wait); the LT
 //              accumulate form draws the thresholds of the touched trials and
 //              activates where acc > theta (k_finalize<2>); the non-empty
 //              words become the next frontier
@@ -1557,7 +1561,8 @@ __device__ __forceinline__ uint32_t spread2(uint32_t x) {
 // issue, 1.4 TB/s DRAM): 36 % of the warps' time goes on gathering rows, a third on the counters, a
 // fifth on listing sources.  2 words per lane and 24 warps per SM at 80 registers; one word per lane at 64
 // registers took 107 against 73 ms per R-MAT-21 call, 32 warps with two words (spilled) the same as 24.
-// R-MAT-21, 1,000 trials (64 of 246 steps pull): expansion 364 -> 115 ms.
+// R-MAT-21, 1,000 trials (64 of 246 steps pull): expansion 364 -> 115 ms, 95 ms with the later steps' smaller
+// push items and frontier rows written once.
 template <int LN>
 __global__ void __launch_bounds__(kBlock, 3) k_pull_lt(Params p_) {
     Params p = p_;
@@ -1733,10 +1738,11 @@ __global__ void __launch_bounds__(kBlock, 3) k_pull_lt(Params p_) {
 
 // Whether the LT step whose frontier makes `checks` (edge, word) checks pulls.  A push step costs its
 // checks; a pull step the scan of all m in-edges and, for every in-edge from the frontier, a row of all
-// B words whether they carry bits or not.  Measured on GB300 (ms per call, push only / pull above
-// checks = m / 3 m / 6 m): R-MAT-21, B = 16: 384 / 154 / 160 / 187; B = 64: 1,470 / 484 / 455 / 446;
-// B = 1: 51.7 above m, 48.1 / 50.3 above 0.67 m / 0.33 m; BA 100k, B = 157: 54.7 / 37.8 / 35.4 / 33.8;
-// B = 16: 8.5 / 6.65 / 6.8.
+// B words whether they carry bits or not.  Measured on GB300, ms per call, push only / pull above m B / 6,
+// / 12, / 20 and / 40 checks: R-MAT-21, B = 16: 435 / 161 / 149 / 148 / 151; B = 64: 1,893 / 527 / 475 / 473 /
+// 489; BA 100k with 10 edges a node, B = 157: 151 / 69.5 / 62.7 / 61.7 / 63.4.  Below B = 8 a scan of the
+// in-edges has too few words to pay for it: the line stays at that of 8 words (R-MAT-21, B = 1, above 1.3 m,
+// 0.67 m, 0.4 m, 0.2 m: 42.3 / 42.0 / 45.9 / 52.2).
 __host__ __device__ __forceinline__ bool lt_pull_pays(unsigned long long checks, int64_t m, int32_t B) {
     return checks * 12ull > (unsigned long long)m * (unsigned long long)(B > 8 ? B : 8);
 }
