@@ -718,7 +718,8 @@ def run_surrogate24(args):
 # ----------------------------------------------------------------------------- our arm
 def kernel_name(model, s):
     """The expansion kernel a counted call ran: k_push<0> (IC), k_push<1> (LT, per-trial in-weight
-    sums) or k_push<2> (LT, counting form)."""
+    sums) or k_push<2> (LT, counting form; its dense steps pull with k_frontier_rows and k_pull_lt,
+    and the figures under this name cover those too)."""
     if model == "ic":
         return "k_push<0>"
     return "k_push<2>" if s.get("lt_counters") else "k_push<1>"
@@ -726,7 +727,8 @@ def kernel_name(model, s):
 
 def alg_bytes(model, s):
     """Bytes the expansion kernel must move, from its own work counters: 8 per work item (row_ptr pair),
-    8 per frontier word loaded, 8 per edge read ({col, thr}), 8 per word check (the target's word) and
+    8 per frontier word loaded, 8 per edge read ({col, thr}), 8 per word check (the target's word; of a
+    pull step the words of the frontier rows it adds) and
     16 per IC word update (vis and next read-modify-write), 8 per LT accumulator add (4-byte read-modify-
     write) or 16 per counter-plane update of the LT counting form (8-byte read-modify-write)."""
     base = 8 * s["work_items"] + 8 * s["frontier_words"] + 8 * s["edges_scanned"] + 8 * s["word_checks"]
@@ -936,7 +938,8 @@ def run_ours(args):
                    "note": "reads = word checks, atomics = counter-plane toggles (activations not counted) per "
                            "second of the kernel; *_time_frac = the share of the kernel's time the same accesses "
                            "take at the measured uniformly random rates (cnd_random_access_rate): L2-resident is "
-                           "the ceiling, DRAM-resident the floor"}
+                           "the ceiling, DRAM-resident the floor; pull steps read whole rows of words in one access, so "
+                           "above 1 the reads are not separate random ones"}
 
     cpu = None if args.no_cpu_baseline else cpu_baseline(wl)
     line = {

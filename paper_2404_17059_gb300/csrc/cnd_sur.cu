@@ -976,7 +976,8 @@ __device__ __forceinline__ float out_score(int32_t c, float T, const float *__re
 // Scores of all nodes: 8 lanes per work item of <= 256 out-edges.  The sum is one float per edge at a
 // random node, so it is bound by how many such loads are in flight; a thread per node (the form
 // before) left the whole sum of a hub's out-row to one thread's chain of loads.  8 lanes rather than a
-// warp because most rows are shorter than 32 edges.  R-MAT-17 (1.94 M edges, GB300): 862 -> 23 us.
+// warp because most rows are shorter than 32 edges.  R-MAT-17 (1.94 M edges, GB300): 862 -> 14 us (23 before the items were
+// sorted by length).
 // Items of a split row write their partial sum to scratch[slot]; k_out_scores_split adds them.
 template <int MODE>
 __global__ void __launch_bounds__(256) k_out_scores(int32_t n_items, const Item *__restrict__ items,
