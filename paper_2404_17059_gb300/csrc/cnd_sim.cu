@@ -2187,7 +2187,8 @@ static cnd_status run_items(int model, const cnd_graph_dev &G, const char *fn, s
     }
 
     const size_t nB = (size_t)n * B;
-    const int chunk = std::min(o.chunk_edges, 16384);  // task index < 2^32 / k in k_push's division
+    // LT divides task indices t < chunk * k by a slot's pair count k <= B: t < 2^32 / k keeps div_by exact
+    const int chunk = (int)std::min<int64_t>(o.chunk_edges, model == 0 ? 16384 : std::min(16384ll, 0xFFFFFFFFll / B / B));
     const int tasks = model == 0 || (!lt_cnt && B > kLtAccWords) ? kTasks : kLtTasks;
     const size_t work_cap = chunk > 0 ? (size_t)n + (size_t)G.m / chunk + 1
                                       : (size_t)n + 2 * (size_t)G.m * (size_t)B / tasks + (size_t)G.m + 1;

@@ -29,3 +29,23 @@ def test_work_items(graph, words, form):
                                  direction="push", **kw)
         assert np.array_equal(a.spread, b.spread) and np.array_equal(a.node_count, b.node_count)
         assert a.edge_checks == b.edge_checks and np.array_equal(a.level_counts, b.level_counts)
+
+
+@pytest.mark.parametrize("form", ["equal", "uneven"])
+def test_long_items_of_wide_passes(form):
+    """A row of 6,000 edges as one requested item of 2,047 pairs: 12 M tasks, whose indices have to be divided
+    exactly by the pair count."""
+    n, words = 6002, 2047
+    g = I.csr_from_edges(n, np.concatenate([np.zeros(n - 2, np.int64), np.arange(1, 40)]),
+                         np.concatenate([np.arange(1, n - 1), np.full(39, n - 1)]))
+    w = np.full(g.m, 1 << 31, dtype=np.uint32)  # a spoke follows the hub in half of the trials
+    w[g.col == n - 1] = (1 << 32) // 40 if form == "equal" else np.arange(1, 40) << 21
+    G = P.cnd_graph_create(g.n, g.row_ptr, g.col, None, w)
+    T = 64 * words - 7
+    a, b = (P.cnd_lt_simulate_ex(G, [0], T, 4, edge_checks=True, level_counts_len=4, word_bits=64 * words,
+                                 direction="push", stats=2, chunk_edges=c) for c in (16384, 0))
+    assert a.stats["passes"] == 1 and a.stats["lt_counters"] == (form == "equal")
+    assert np.array_equal(a.spread, b.spread) and np.array_equal(a.node_count, b.node_count)
+    assert a.edge_checks == b.edge_checks and np.array_equal(a.level_counts, b.level_counts)
+    o = oracle.simulate_threads("lt", g, [0], 256, 4, level_counts_len=4, lt_weight=w)
+    assert np.array_equal(a.spread[:256], o.spread)
