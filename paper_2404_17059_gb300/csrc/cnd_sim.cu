@@ -1635,10 +1635,11 @@ __global__ void __launch_bounds__(kBlock, 3) k_pull_lt(Params p_) {
             n_wc += 16;
         }
     };
-    // bring the counters of words w, w + 1 into L2 while the rows are counted
+    // bring the counters of words w, w + 1 (of the last word of an odd pass: its own) into L2 while the rows
+    // are counted
     auto prefetch = [&](uint32_t tag, int w) {
         const uint64_t *a = p.planes + ((size_t)(tag >> 5) * B + (size_t)w * (tag & 31u));
-        const int bytes = 16 * (int)(tag & 31u);
+        const int bytes = (w + 1 < B ? 16 : 8) * (int)(tag & 31u);
         for (int o = 0; o < bytes; o += 128)
             asm volatile("prefetch.global.L2 [%0];" ::"l"((const char *)a + o));
     };
