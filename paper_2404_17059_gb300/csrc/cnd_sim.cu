@@ -2041,9 +2041,14 @@ struct Pinned {
 };
 static thread_local Pinned t_pinned;
 
-// Copy `bytes` from host to device memory on st, through the pinned staging where they fit.
+// Copy `bytes` from host to device memory on st, through the pinned staging where they fit.  The caller may
+// free src on return: a copy from src itself, which a device that reads pageable memory may still be at when
+// cudaMemcpyAsync returns, is waited for.
 static cudaError_t stage_in(void *dst, const void *src, size_t bytes, cudaStream_t st) {
-    if (bytes > kStaging) return cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, st);
+    if (bytes > kStaging) {
+        const cudaError_t e = cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, st);
+        return e != cudaSuccess ? e : cudaStreamSynchronize(st);
+    }
     if (!t_pinned.in) {
         const cudaError_t e = cudaMallocHost(&t_pinned.in, kStaging);
         if (e != cudaSuccess) return e;

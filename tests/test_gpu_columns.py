@@ -121,3 +121,19 @@ def test_time_limit_and_bad_device_seed():
             _sim("ic", G, torch.tensor([1, bad], dtype=torch.int32, device="cuda"), 64, 1)
         assert ei.value.status == P.CND_EINVAL
     _check("ic", g, G, [1, 2], 64, 1, p, w, timeout_s=30.0)
+
+
+def test_inputs_beyond_the_staging():
+    """More than 256 KB of items or seeds: copied from host memory that the call frees before it ends."""
+    g = I.erdos_renyi_m(300, 1500, graph_seed=7)
+    p, w = _weights(g)
+    G = P.cnd_graph_create(g.n, g.row_ptr, g.col, p, w)
+    off, seeds, _, keys = I.batch_items(g.n, 9000, 1, 4, (1,), graph_seed=7)
+    trials = np.array([(4, 9, 0, 33)[i % 4] for i in range(9000)], dtype=np.int32)
+    a, b = (P.cnd_ic_simulate_batch(G, off, seeds, trials, keys, node_count=True, edge_checks=True, word_bits=wb)
+            for wb in (0, 64 * 512))
+    assert np.array_equal(a.spread, b.spread) and np.array_equal(a.node_count, b.node_count)
+    assert a.edge_checks == b.edge_checks
+    many = np.random.default_rng(7).integers(0, 40, 70_000)
+    for model in ("ic", "lt"):
+        _check(model, g, G, many, 70, 4, p, w)
