@@ -1079,6 +1079,7 @@ struct cnd_sur {
           *da0 = nullptr, *yv = nullptr;
     int32_t *seeds = nullptr;
     int32_t seeds_cap = 0;
+    std::vector<int32_t> seeds_h;  // the call's distinct seeds: the source of their copy to the device
     std::vector<int32_t> row_ptr_h;  // host copy of the out-CSR offsets (training-set sampler)
     double *dsum = nullptr;  // [0] spread, [1] loss
     std::vector<void *> allocs;
@@ -1159,7 +1160,9 @@ cnd_status upload_seeds(cnd_sur *s, const int32_t *seeds, int32_t ns, int32_t &n
         set_error("%s: bad seed list", fn);
         return CND_EINVAL;
     }
-    std::vector<int32_t> u(seeds, seeds + ns);
+    // kept by the handle: a device that reads pageable memory may be at it until the call's last wait
+    std::vector<int32_t> &u = s->seeds_h;
+    u.assign(seeds, seeds + ns);
     for (int32_t x : u)
         if (x < 0 || x >= s->n) {
             set_error("%s: seed %d out of range", fn, (int)x);

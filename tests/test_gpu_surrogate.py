@@ -202,3 +202,18 @@ def test_bad_arguments_are_rejected(setup):
     G2 = P.cnd_graph_create(g.n, g.row_ptr, g.col, None, I.lt_weighted_cascade(g))
     with pytest.raises(P.CndError):
         P.cnd_sur_create(G2, params)  # no IC probabilities
+
+
+def test_many_seeds():
+    """Seed lists of 80 KB, duplicates among them, one call after another."""
+    g = I.erdos_renyi_m(30_000, 90_000, graph_seed=6)
+    p = np.full(g.m, 0.1, dtype=np.float32)
+    G = P.cnd_graph_create(g.n, g.row_ptr, g.col, p, None)
+    params = (I.surrogate_init(3) * 3.0).astype(np.float32)
+    sur, OG = P.cnd_sur_create(G, params), S.Graph(g, p)
+    for sd in (1, 2):
+        seeds = np.random.default_rng(sd).integers(0, g.n, 20_000)
+        yh, _ = P.cnd_sur_forward(sur, seeds)
+        ref = S.forward(params.astype(np.float64), OG, np.unique(seeds))["yhat"]
+        np.testing.assert_allclose(yh, ref, rtol=0, atol=5e-3)
+        assert np.all(yh[seeds] == 1.0)
