@@ -97,6 +97,17 @@ __device__ __forceinline__ unsigned long long timer_ns() {
     return t;
 }
 
+// True once the time limit, measured from the call's first step (t0), has passed; the call then times out.  A
+// timer that reads before another SM's t0 is not past it.
+__device__ __forceinline__ bool past_limit(const ColParams &p) {
+    if (p.timeout_ns == 0) return false;
+    if (*(volatile int32_t *)&p.flags->timed_out) return true;
+    const unsigned long long t0 = *(volatile unsigned long long *)&p.flags->t0, now = timer_ns();
+    if (t0 == 0 || now <= t0 || now - t0 <= p.timeout_ns) return false;
+    p.flags->timed_out = 1;
+    return true;
+}
+
 // 32 x 32 bit transpose over a warp: bit i of lane b's result is bit b of lane i's x.
 __device__ __forceinline__ uint32_t transpose32(uint32_t x) {
     const int lane = threadIdx.x & 31;
@@ -229,7 +240,11 @@ __global__ void __launch_bounds__(1024, 1) k_columns(ColParams p) {
     const uint32_t lt = (1u << lane) - 1u, le = lt | (1u << lane);
     unsigned long long ck = 0;
     for (;;) {
-        if (tid == 0) S.col = atomicAdd(&p.flags->next_column, 1);
+        if (tid == 0) {
+            int c = atomicAdd(&p.flags->next_column, 1);
+            if (c < p.n_cols && past_limit(p)) c = p.n_cols;  // the columns left are not run
+            S.col = c;
+        }
         __syncthreads();
         const int col = S.col;
         if (col >= p.n_cols) break;
@@ -336,10 +351,7 @@ __global__ void __launch_bounds__(1024, 1) k_columns(ColParams p) {
                 // the slots of the step after next: nobody reads or writes them in this one
                 S.n_list[(step + 2) % 3] = 0;
                 S.n_hub[nslot] = 0;
-                if (p.timeout_ns && timer_ns() - *(volatile unsigned long long *)&p.flags->t0 > p.timeout_ns) {
-                    p.flags->timed_out = 1;
-                    S.stop = step + 1;  // not this step: other threads may not have read it yet
-                }
+                if (past_limit(p)) S.stop = step + 1;  // not this step: other threads may not have read it yet
             }
             // nodes per warp: all warps get some while there are enough
             const int G = min(32, (F + n_warps - 1) / n_warps);

@@ -137,3 +137,32 @@ def test_inputs_beyond_the_staging():
     many = np.random.default_rng(7).integers(0, 40, 70_000)
     for model in ("ic", "lt"):
         _check(model, g, G, many, 70, 4, p, w)
+
+
+@pytest.mark.parametrize("model", ["ic", "lt"])
+def test_time_limit_ends_a_long_call(model):
+    """The columns that are left when the limit passes are not run."""
+    import time
+    torch = pytest.importorskip("torch")
+    g = I.erdos_renyi_m(1000, 10_000, graph_seed=1)
+    p, w = I.ic_uniform(g, 0.1), I.lt_weighted_cascade(g)
+    G = P.cnd_graph_create(g.n, g.row_ptr, g.col, p, w)
+    f = P.cnd_ic_simulate_ex if model == "ic" else P.cnd_lt_simulate_ex
+    seeds = torch.tensor([1, 2, 3], dtype=torch.int32, device="cuda")
+
+    def seconds(**kw):
+        torch.cuda.synchronize()
+        t0 = time.perf_counter()
+        try:
+            f(G, seeds, 20_000_000, 1, **kw)
+            status = P.CND_OK
+        except P.CndError as e:
+            status = e.status
+        return time.perf_counter() - t0, status
+
+    seconds()
+    full, status = seconds()
+    assert status == P.CND_OK and full > 0.02
+    limited, status = seconds(timeout_s=full / 20)
+    assert status == P.CND_ETIMEOUT
+    assert limited < full / 5, (limited, full)
