@@ -902,23 +902,32 @@ __global__ void __launch_bounds__(256) k_reduce_dw(int32_t nblocks, int32_t din,
     }
 }
 
-// grad (bias of `layer`; head: also w_o, b_o and the loss) += the blocks' partial sums: blocks of 32 x 32
-// threads, 32 values each
+// grad (bias of `layer`; head: also w_o, b_o and the loss, which is summed in 64 bits) += the blocks' partial
+// sums: blocks of 32 x 32 threads, 32 values each
 __global__ void __launch_bounds__(1024) k_reduce_bwd(int32_t nblocks, const float *__restrict__ part, int layer, int head,
                                                      float *__restrict__ grad, double *__restrict__ loss,
                                                      float loss_scale) {
     __shared__ float s[32][33];
+    __shared__ double s_loss[32];
     const int c = blockIdx.x * 32 + threadIdx.x;  // 0 .. 2 H + 1
-    const bool ok = c < (head ? kBwdPart : H);
+    const bool ok = c < (head ? 2 * H + 1 : H), is_loss = head && c == 2 * H + 1;
     float sum = 0.0f;
     if (ok) {
 #pragma unroll 8
         for (int b = threadIdx.y; b < nblocks; b += 32) sum += part[(size_t)b * kBwdPart + c];
     }
+    if (is_loss) {
+        double l = 0.0;
+        for (int b = threadIdx.y; b < nblocks; b += 32) l += (double)part[(size_t)b * kBwdPart + c];
+        s_loss[threadIdx.y] = l;
+    }
     sum = tree_sum(s, sum);
-    if (ok && threadIdx.y == 0) {
-        if (c < 2 * H + 1) grad[c < H ? off_b(layer) + c : (c < 2 * H ? OFF_WO + (c - H) : OFF_BO)] += sum;
-        else *loss += (double)sum * (double)loss_scale;
+    if (threadIdx.y != 0) return;
+    if (ok) grad[c < H ? off_b(layer) + c : (c < 2 * H ? OFF_WO + (c - H) : OFF_BO)] += sum;
+    if (is_loss) {
+        double l = 0.0;
+        for (int i = 0; i < 32; ++i) l += s_loss[i];
+        *loss += l * (double)loss_scale;
     }
 }
 

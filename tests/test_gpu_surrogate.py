@@ -217,3 +217,16 @@ def test_many_seeds():
         ref = S.forward(params.astype(np.float64), OG, np.unique(seeds))["yhat"]
         np.testing.assert_allclose(yh, ref, rtol=0, atol=5e-3)
         assert np.all(yh[seeds] == 1.0)
+
+
+def test_loss_is_summed_in_64_bits():
+    """Zero weights predict 1/2 everywhere; the targets make every term of the loss and every block's sum a whole
+    number below 2^24, and the total an odd number above it."""
+    n = 65_536
+    g = I.csr_from_edges(n, np.arange(9), np.arange(1, 10))
+    G = P.cnd_graph_create(g.n, g.row_ptr, g.col, np.full(9, 0.5, dtype=np.float32), None)
+    sur = P.cnd_sur_create(G, np.zeros(P.CND_SUR_N_PARAMS, dtype=np.float32))
+    y = np.full(n, 64.5, dtype=np.float32)
+    y[12_345] = 1.5
+    loss, _ = P.cnd_sur_loss_grad(sur, [], y)
+    assert loss == ((n - 1) * 64 * 64 + 1) / n
