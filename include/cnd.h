@@ -142,15 +142,18 @@ typedef struct cnd_sim_opts {
                                   steps no longer are activation times, so level counts and
                                   max_levels are refused (CND_EINVAL); 0 = off, at most 64 */
     double timeout_s;          /* > 0: give up with CND_ETIMEOUT after this many seconds (checked
-                                  between steps: by the host, or in a CUDA-graph call by the
-                                  step-control kernel on the GPU's global timer) */
-    cnd_sim_stats *stats;      /* NULL or host struct filled by the call */
+                                  between steps: by the host, or on the GPU's global timer by the
+                                  step-control kernel of a CUDA-graph call and by every block of
+                                  the column engine, which runs no further columns then) */
+    cnd_sim_stats *stats;      /* NULL or host struct filled by the call, which then runs in the pass
+                                  engine (CND_ENGINE_*) */
     int32_t defer_steps;       /* with defer_bits: a word waits at most this many steps (0 = until
                                   nothing else is left to expand) */
     int32_t graph;             /* 1: run the whole call as one CUDA graph launch -- every pass
                                   and its step loop (a device-side WHILE node whose condition a
                                   one-thread control kernel sets after each step), no host round
-                                  trip per step; ignored with CND_STATS_TIMING.  Each host thread
+                                  trip per step; ignored with CND_STATS_TIMING and by the column
+                                  engine, which is one launch without it.  Each host thread
                                   keeps the executable graphs of its recent call shapes (up to 16)
                                   and updates a matching one in place rather than instantiating */
     int32_t autotune;          /* 1: take word_bits, chunk_edges, pull_permille and graph from the
@@ -167,6 +170,21 @@ typedef struct cnd_sim_opts {
 } cnd_sim_opts;
 
 void cnd_sim_opts_init(cnd_sim_opts *opts);
+
+/* The two engines of the simulate calls; both compute exactly the same results.
+ *   passes:  64-trial words of all trials side by side, one step of all of them
+ *            at a time, state in device memory; every graph.
+ *   columns: a block takes a column of up to 32 trials through all of its
+ *            steps, state in shared memory, the whole call one kernel; graphs of
+ *            up to about 23,300 nodes (IC) or 18,000 (LT, and its counting form only).
+ * A call takes the columns where they are the faster by a rule on the graph
+ * and the trials, and only with the engine settings left alone: word_bits,
+ * chunk_edges, pull_permille, defer_bits and lt_accumulate 0, direction
+ * CND_DIR_AUTO and stats NULL.  So a call with stats measures the passes, also
+ * where the same call without takes the columns; `graph` has no effect on
+ * the columns.  cnd_sim_plan tells. */
+#define CND_ENGINE_PASSES 0
+#define CND_ENGINE_COLUMNS 1
 
 /*
  * Build the device copy of a directed CSR graph (Sec. 3 "Data Structures":
@@ -258,6 +276,18 @@ cnd_status cnd_lt_simulate_batch(const cnd_graph *g, int32_t n_items, const int6
 cnd_status cnd_autotune(const cnd_graph *g, int32_t model, int32_t n_items, const int64_t *seed_off,
                         const int32_t *seeds, int32_t n_seeds, const int32_t *n_trials, const uint64_t *rng_seed,
                         const cnd_sim_opts *base, cnd_sim_opts *best_out, double *best_ms_out);
+
+/*
+ * The engine that a simulate call of these sizes and options takes
+ * (CND_ENGINE_*), and the trials that it holds per node at a time: of a pass
+ * (its width for `free_bytes` of free device memory; 0 = what is free now), or
+ * of a column.  Runs nothing.
+ * model: 0 IC, 1 LT.  n_trials: of all n_items seed sets together (1 for
+ * a single one), taken as spread evenly over them.  opts may be NULL; its
+ * autotune is taken as 0.  The outputs may be NULL.
+ */
+cnd_status cnd_sim_plan(const cnd_graph *g, int32_t model, int32_t n_items, int64_t n_trials,
+                        const cnd_sim_opts *opts, int64_t free_bytes, int32_t *engine_out, int32_t *word_bits_out);
 
 /*
  * Influence maximisation by lazy greedy (CELF, Leskovec et al. 2007) on the

@@ -28,7 +28,7 @@ EXPORTS = (
     "cnd_lt_simulate_batch", "cnd_autotune", "cnd_im_opts_init", "cnd_ic_im_celf", "cnd_lt_im_celf",
     "cnd_sur_create", "cnd_sur_destroy", "cnd_sur_set_params", "cnd_sur_get_params", "cnd_sur_forward",
     "cnd_sur_loss_grad", "cnd_sur_adam", "cnd_sur_scores", "cnd_sur_train_opts_init", "cnd_sur_train",
-    "cnd_ic_im_screened", "cnd_sur_onehop", "cnd_philox_rate", "cnd_random_access_rate",
+    "cnd_ic_im_screened", "cnd_sur_onehop", "cnd_philox_rate", "cnd_random_access_rate", "cnd_sim_plan",
 )
 CND_SUR_N_PARAMS = 18689
 
@@ -187,6 +187,8 @@ def load(build_if_missing: bool = True):
         L.cnd_sur_train.restype = i32
         L.cnd_ic_im_screened.argtypes = [vp, vp, C.POINTER(cnd_im_opts), C.POINTER(cnd_screen_opts), vp, vp]
         L.cnd_ic_im_screened.restype = i32
+        L.cnd_sim_plan.argtypes = [vp, i32, i32, i64, C.POINTER(cnd_sim_opts), i64, C.POINTER(i32), C.POINTER(i32)]
+        L.cnd_sim_plan.restype = i32
         L.cnd_lt_weights_wc.argtypes = [i32, i32, vp, vp]
         L.cnd_lt_weights_wc.restype = i32
         L.cnd_philox4x32_10.argtypes = [u64, vp, i64, vp]
@@ -506,6 +508,22 @@ def cnd_autotune(g, model, seeds, n_trials, rng_seed, *, seed_off=None) -> dict:
                           int(seeds.size), _np_ptr(tr), _np_ptr(ks), C.byref(base), C.byref(best), C.byref(ms)))
     return {"word_bits": best.word_bits, "chunk_edges": best.chunk_edges, "pull_permille": best.pull_permille,
             "graph": best.graph, "sample_ms": ms.value}
+
+
+def cnd_sim_plan(g, model, n_trials, *, n_items=1, free_bytes=0, stats=0, **kw):
+    """(engine, trials held per node at a time) of a simulate call with these options: "columns" or
+    "passes", and the trials of a column or of a pass (for free_bytes of free device memory; 0 = now)."""
+    o = cnd_sim_opts_init()
+    for k, v in kw.items():
+        setattr(o, k, _DIRS[v] if k == "direction" and isinstance(v, str) else float(v) if k == "timeout_s" else int(v))
+    stt = cnd_sim_stats()
+    if stats:
+        o.stats = C.cast(C.pointer(stt), C.c_void_p)
+    engine, bits = C.c_int32(), C.c_int32()
+    mdl = {"ic": 0, "lt": 1}[model] if isinstance(model, str) else int(model)
+    _check(load().cnd_sim_plan(g.handle, mdl, int(n_items), int(n_trials), C.byref(o), int(free_bytes),
+                               C.byref(engine), C.byref(bits)))
+    return ("passes", "columns")[engine.value], bits.value
 
 
 @dataclasses.dataclass

@@ -2089,6 +2089,42 @@ static const void *push_fn() {
     return (const void *)k_push<MODEL, PERWORD>;
 }
 
+// LT in the counting form where the graph allows it (unless the caller asks for the sums).
+static bool counting_form(int model, const cnd_graph_dev &G, const cnd_sim_opts &o) {
+    return model == 1 && G.lt_cnt_edge != nullptr && !o.lt_accumulate;
+}
+
+// Words per node and pass of a call of total_words > 0 words, and which pull steps it may take.
+struct PassWidth {
+    int B;
+    bool lt_pull, ic_pull;
+};
+
+static PassWidth pass_width(int model, const cnd_graph_dev &G, const cnd_sim_opts &o, int64_t total_words, size_t free_b) {
+    const int32_t n = G.n;
+    const bool lt_cnt = counting_form(model, G, o);
+    const double budget = 0.6 * (double)free_b;
+    // bytes per word column: vis, nxt, two pair pools (+ LT accumulators or counter planes, and what its work
+    // items take more than IC's)
+    const int tasks_min = model == 0 ? kTasks : kLtTasks;
+    const double per_word = (double)n * (2 * 8 + 2 * 10 + (model == 1 && !lt_cnt ? 256 : 0)) +
+                            (lt_cnt ? 8.0 * (double)G.lt_planes : 0.0) +
+                            (o.chunk_edges > 0 ? 0.0 : 32.0 * (double)G.m * (1.0 / tasks_min - 1.0 / kTasks));
+    // IC pulls only when asked to: by direction, or by a switch threshold; LT in the counting form
+    // chooses per step (lt_pull_pays)
+    const bool lt_pull = lt_cnt && G.m > 0 && o.direction != CND_DIR_PUSH && o.defer_bits == 0;
+    const bool ic_pull = model == 0 && G.m > 0 &&
+                         (o.direction == CND_DIR_PULL || (o.direction == CND_DIR_AUTO && o.pull_permille > 0));
+    int64_t bmax = o.word_bits ? o.word_bits / 64 : kMaxB;
+    bmax = std::min<int64_t>(bmax, std::max<int64_t>(1, (int64_t)(budget / per_word)));
+    bmax = std::min<int64_t>(bmax, ic_pull ? kPullMaxB : kMaxB);
+    bmax = std::min<int64_t>(bmax, std::max<int64_t>(1, (int64_t)0x7FFFFFFF / std::max(n, 1)));
+    if (model == 1 && G.m > 0)  // a step's work items are counted in 32 bits
+        bmax = std::min<int64_t>(bmax, std::max<int64_t>(1, (0x7FFFFFFFll - n - G.m) * tasks_min / (2 * (int64_t)G.m)));
+    const int64_t n_pass = (total_words + bmax - 1) / bmax;
+    return PassWidth{(int)((total_words + n_pass - 1) / n_pass), lt_pull, ic_pull};
+}
+
 // Runs the items' trials: words of all items are packed into passes of B
 // word columns (an item may span passes; trials are independent), and each
 // pass runs the level loop over all its columns at once.
@@ -2101,8 +2137,7 @@ static cnd_status run_items(int model, const cnd_graph_dev &G, const char *fn, s
                             const cnd_sim_opts &o, Work &W, bool &limit_hit) {
     cudaStream_t st = W.st;
     const int32_t n = G.n;
-    // LT in the counting form where the graph allows it (unless the caller asks for the sums)
-    const bool lt_cnt = model == 1 && G.lt_cnt_edge != nullptr && !o.lt_accumulate;
+    const bool lt_cnt = counting_form(model, G, o);
     const uint2 *edge = model == 0 ? G.ic_edge : (lt_cnt ? G.lt_cnt_edge : G.lt_edge);
     int64_t total_words = 0;
     for (const auto &it : items) total_words += (it.trials + 63) / 64;
@@ -2141,30 +2176,11 @@ static cnd_status run_items(int model, const cnd_graph_dev &G, const char *fn, s
         return CND_OK;
     };
 
-    // ---- pass width
     size_t free_b = 0, total_b = 0;
     CND_CUDA_TRY(cudaMemGetInfo(&free_b, &total_b));
-    const double budget = 0.6 * (double)free_b;
-    // bytes per word column: vis, nxt, two pair pools (+ LT accumulators or counter planes, and what its work
-    // items take more than IC's)
-    const int tasks_min = model == 0 ? kTasks : kLtTasks;
-    const double per_word = (double)n * (2 * 8 + 2 * 10 + (model == 1 && !lt_cnt ? 256 : 0)) +
-                            (lt_cnt ? 8.0 * (double)G.lt_planes : 0.0) +
-                            (o.chunk_edges > 0 ? 0.0 : 32.0 * (double)G.m * (1.0 / tasks_min - 1.0 / kTasks));
-    // IC pulls only when asked to: by direction, or by a switch threshold; LT in the counting form
-    // chooses per step (lt_pull_pays)
-    const bool lt_pull = lt_cnt && G.m > 0 && o.direction != CND_DIR_PUSH && o.defer_bits == 0;
-    const bool ic_pull = model == 0 && G.m > 0 &&
-                         (o.direction == CND_DIR_PULL || (o.direction == CND_DIR_AUTO && o.pull_permille > 0));
-    const bool may_pull = ic_pull || lt_pull;
-    int64_t bmax = o.word_bits ? o.word_bits / 64 : kMaxB;
-    bmax = std::min<int64_t>(bmax, std::max<int64_t>(1, (int64_t)(budget / per_word)));
-    bmax = std::min<int64_t>(bmax, ic_pull ? kPullMaxB : kMaxB);
-    bmax = std::min<int64_t>(bmax, std::max<int64_t>(1, (int64_t)0x7FFFFFFF / std::max(n, 1)));
-    if (model == 1 && G.m > 0)  // a step's work items are counted in 32 bits
-        bmax = std::min<int64_t>(bmax, std::max<int64_t>(1, (0x7FFFFFFFll - n - G.m) * tasks_min / (2 * (int64_t)G.m)));
-    const int64_t n_pass = (total_words + bmax - 1) / bmax;
-    const int B = (int)((total_words + n_pass - 1) / n_pass);
+    const PassWidth pw = pass_width(model, G, o, total_words, free_b);
+    const bool lt_pull = pw.lt_pull, ic_pull = pw.ic_pull, may_pull = ic_pull || lt_pull;
+    const int B = pw.B;
     const int nq = (B + 63) / 64;
 
     // ---- pass layout: items by decreasing size, runs of columns
@@ -2800,6 +2816,13 @@ static cnd_status apply_autotune(int model, const cnd_graph *g, int32_t n_items,
     return CND_OK;
 }
 
+static bool bad_opts(const cnd_sim_opts &o) {
+    return o.first_trial < 0 || (o.first_trial & 63) || o.word_bits < 0 || (o.word_bits & 63) || o.word_bits > 64 * kMaxB ||
+           o.level_counts_len < 0 || (o.level_counts_len > 0 && !o.level_counts_out) || o.chunk_edges < 0 ||
+           o.direction < 0 || o.direction > 2 || o.defer_bits < 0 || o.defer_bits > 64 || o.defer_steps < 0 ||
+           o.defer_steps > 255 || o.lt_accumulate < 0 || o.lt_accumulate > 1;
+}
+
 // Shared front end of the single and batched entry points.
 static cnd_status simulate_common(int model, const cnd_graph *g, const char *fn, int32_t n_items,
                                   const int64_t *seed_off, const int32_t *seeds, const int32_t *n_trials_arr,
@@ -2820,11 +2843,7 @@ static cnd_status simulate_common(int model, const cnd_graph *g, const char *fn,
         set_error("%s: graph was created without %s", fn, model == 0 ? "IC probabilities" : "LT weights");
         return CND_EINVAL;
     }
-    if (n_items < 0 || (batched && n_items > 0 && (!seed_off || !keys)) || o.first_trial < 0 ||
-        (o.first_trial & 63) || o.word_bits < 0 || (o.word_bits & 63) || o.word_bits > 64 * kMaxB ||
-        o.level_counts_len < 0 || (o.level_counts_len > 0 && !o.level_counts_out) || o.chunk_edges < 0 ||
-        o.direction < 0 || o.direction > 2 || o.defer_bits < 0 || o.defer_bits > 64 || o.defer_steps < 0 ||
-        o.defer_steps > 255 || o.lt_accumulate < 0 || o.lt_accumulate > 1) {
+    if (n_items < 0 || (batched && n_items > 0 && (!seed_off || !keys)) || bad_opts(o)) {
         set_error("%s: bad arguments (items, first_trial %% 64, word_bits, level_counts, chunk, defer)", fn);
         return CND_EINVAL;
     }
@@ -3064,6 +3083,48 @@ cnd_status cnd_autotune(const cnd_graph *g, int32_t model, int32_t n_items, cons
     o.autotune = 0;
     *best_out = o;
     if (best_ms_out) *best_ms_out = ms;
+    return CND_OK;
+}
+
+cnd_status cnd_sim_plan(const cnd_graph *g, int32_t model, int32_t n_items, int64_t n_trials,
+                        const cnd_sim_opts *opts, int64_t free_bytes, int32_t *engine_out, int32_t *word_bits_out) {
+    clear_error();
+    cnd_sim_opts o;
+    cnd_sim_opts_init(&o);
+    if (opts) o = *opts;
+    if (!g || (model != 0 && model != 1) || n_items < 1 || n_trials < 0 || n_trials > (int64_t)n_items * 0x7FFFFFFF ||
+        free_bytes < 0 || bad_opts(o)) {
+        set_error("cnd_sim_plan: bad arguments");
+        return CND_EINVAL;
+    }
+    const cnd_graph_dev &G = g->d;
+    std::vector<ItemDesc> items((size_t)n_items);
+    int64_t words = 0;
+    for (int32_t i = 0; i < n_items; ++i) {
+        items[i].trials = n_trials / n_items + (i < n_trials % n_items ? 1 : 0);
+        words += (items[i].trials + 63) / 64;
+    }
+    int32_t engine = CND_ENGINE_PASSES, bits = 0;
+    if (words > 0 && columns_fit(model, G, o, n_trials)) {
+        ColPlan plan;
+        const cnd_status st = plan_columns(model, G, items, plan);
+        if (st != CND_OK) return st;
+        engine = CND_ENGINE_COLUMNS;
+        bits = plan.bits;
+    } else if (words > 0) {
+        size_t free_b = (size_t)free_bytes, total_b = 0;
+        if (free_bytes == 0) {
+            int prev = 0;
+            CND_CUDA_TRY(cudaGetDevice(&prev));
+            CND_CUDA_TRY(cudaSetDevice(G.device));
+            const cudaError_t e = cudaMemGetInfo(&free_b, &total_b);
+            cudaSetDevice(prev);
+            CND_CUDA_TRY(e);
+        }
+        bits = 64 * pass_width(model, G, o, words, free_b).B;
+    }
+    if (engine_out) *engine_out = engine;
+    if (word_bits_out) *word_bits_out = bits;
     return CND_OK;
 }
 

@@ -166,3 +166,28 @@ def test_time_limit_ends_a_long_call(model):
     limited, status = seconds(timeout_s=full / 20)
     assert status == P.CND_ETIMEOUT
     assert limited < full / 5, (limited, full)
+
+
+@pytest.mark.parametrize("model", ["ic", "lt"])
+def test_engine_of_a_call(model):
+    """Which of the calls above run in the column engine, and what keeps a call out of it."""
+    engine = {}
+    for n in (1, 33, 6000, 23_300, 24_400, 30_000):
+        rng = np.random.default_rng(n)
+        g = I.csr_from_edges(n, rng.integers(0, n, 4 * n), rng.integers(0, n, 4 * n))
+        p, w = _weights(g)
+        G = P.cnd_graph_create(n, g.row_ptr, g.col, p, w)
+        engine[n], bits = P.cnd_sim_plan(G, model, 100)
+        assert 4 <= bits <= 32 if engine[n] == "columns" else bits == 128
+        if n == 6000:
+            for kw in ({"word_bits": 64}, {"chunk_edges": 8}, {"direction": "push"}, {"defer_bits": 2}, {"stats": 2},
+                       {"pull_permille": 250}):
+                assert P.cnd_sim_plan(G, model, 100, **kw)[0] == "passes"
+            for kw in ({"graph": 1}, {"max_levels": 3}, {"first_trial": 64}, {"n_items": 7}):
+                assert P.cnd_sim_plan(G, model, 100, **kw)[0] == "columns"
+            assert P.cnd_sim_plan(G, model, 0) == ("passes", 0)
+            with pytest.raises(P.CndError):
+                P.cnd_sim_plan(G, model, 100, word_bits=65)
+    assert all(engine[n] == "columns" for n in (1, 33, 6000)) and engine[30_000] == "passes"
+    assert engine[23_300] == ("columns" if model == "ic" else "passes")
+    assert engine[24_400] == "passes"

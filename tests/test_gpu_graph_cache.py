@@ -64,3 +64,45 @@ def test_batches_of_other_compositions():
             assert np.array_equal(np.asarray(r.node_count).reshape(a1 - a0, g.n)[i], b.node_count)
             checks += b.edge_checks
         assert r.edge_checks == checks
+
+
+def test_batches_of_other_compositions_in_the_pass_engine():
+    """As above with statistics, which keep the calls out of the column engine: a batch of the first one's shape
+    finds its executable."""
+    g = I.rmat(12, 16 << 12, graph_seed=3)
+    p = I.ic_uniform_random(g, 0.1, graph_seed=3)
+    G = P.cnd_graph_create(g.n, g.row_ptr, g.col, p, None)
+    so, seeds, tr, keys = I.batch_items(g.n, 24, 1, 30, (64, 128, 640), graph_seed=5)
+    tr[:] = np.array([64, 128, 640])[np.arange(24) % 3]
+    assert P.cnd_sim_plan(G, "ic", int(tr[:9].sum()), n_items=9, graph=1, stats=P.CND_STATS_COUNT)[0] == "passes"
+    reused = []
+    for a0, a1 in ((0, 9), (9, 21), (3, 12), (0, 9)):
+        s2 = so[a0:a1 + 1] - so[a0]
+        r = P.cnd_ic_simulate_batch(G, s2, seeds[so[a0]:so[a1]], tr[a0:a1], keys[a0:a1], graph=1, node_count=True,
+                                    edge_checks=True, stats=P.CND_STATS_COUNT)
+        reused.append(r.stats["graph_reused"])
+        off = np.concatenate([[0], np.cumsum(tr[a0:a1])])
+        checks = 0
+        for i in range(a1 - a0):
+            b = oracle.simulate("ic", g, seeds[so[a0 + i]:so[a0 + i + 1]], int(tr[a0 + i]), int(keys[a0 + i]),
+                                ic_prob=p, level_counts_len=0)
+            assert np.array_equal(r.spread[off[i]:off[i + 1]], b.spread)
+            assert np.array_equal(r.node_count[i], b.node_count)
+            checks += b.edge_checks
+        assert r.edge_checks == checks
+    assert reused[0] == 0 and reused[2:] == [1, 1], reused
+
+
+def test_another_graph_in_between_in_the_pass_engine():
+    """The executables of two graphs, used in turn."""
+    cases = []
+    for g, p in ((I.erdos_renyi_m(1000, 10_000, graph_seed=1), None), (I.barabasi_albert(5000, 3, graph_seed=4), None)):
+        p = I.ic_weighted_cascade(g)
+        cases.append((g, p, P.cnd_graph_create(g.n, g.row_ptr, g.col, p, None)))
+    reused = []
+    for rng in (1, 7, 9):
+        for g, p, G in cases:
+            a = P.cnd_ic_simulate_ex(G, [0, 1, 2], 700, rng, graph=1, edge_checks=True, stats=P.CND_STATS_COUNT)
+            _same(a, oracle.simulate_threads("ic", g, [0, 1, 2], 700, rng, ic_prob=p, level_counts_len=0))
+            reused.append(a.stats["graph_reused"])
+    assert all(r == 1 for r in reused[2:]), reused
