@@ -39,7 +39,6 @@ namespace {
 
 constexpr int kHub = 256;       // out-edges from which the whole block expands a node
 constexpr int kHubCap = 64;     // hubs set aside per step (more are expanded by the warp that finds them)
-constexpr int kColMaxN = 65535; // node ids are kept in 16 bits
 
 struct ColItem {
     int64_t out0;     // position of the item's first trial in the spread output
@@ -488,11 +487,66 @@ bool column_shape(int model, const cnd_graph_dev &G, int per_sm, ColShape &c) {
     return true;
 }
 
+// Blocks per SM and trials per column (a multiple of 4, one coin block), by estimated time: a
+// wave of columns takes a constant (the latency of its steps) and work in proportion to the
+// trials (and 2 more: work that a check takes whatever its trials) and the edges, at a rate in
+// proportion to the block's threads.  1,000 trials, blocks per SM / trials per column: G(1000, 10000)
+// 2 / 4 133 us, 1 / 8 148; Watts-Strogatz 10k U[0, 1] 2 / 4 648 us, 1 / 8 575; BA 5k WC 255 and 269.
+void choose_shape(int model, const cnd_graph_dev &G, int64_t trials, ColShape &c, int32_t &bits) {
+    const double size = std::min(1.0, std::max(0.25, (double)G.m / 1e5));
+    double best = 1e300;
+    for (int per_sm = 4; per_sm >= 1; per_sm >>= 1) {
+        ColShape k;
+        if (!column_shape(model, G, per_sm, k)) continue;
+        for (int b = 4; b <= 32; b += 4) {
+            const double waves = std::ceil((double)((trials + b - 1) / b) / ((double)G.num_sms * per_sm));
+            const double cost = waves * ((per_sm == 1 ? 10 : per_sm == 2 ? 9 : 8) + size * per_sm * (b + 2));
+            if (cost < best) {
+                best = cost;
+                bits = b;
+                c = k;
+            }
+        }
+    }
+}
+
+// Whether the columns of a call on a graph of many edges are faster than its passes.  A column is one
+// block's work, so a wave of columns takes its edges' time on one SM however few trials there are,
+// where a pass spreads them over all; a pass takes some 48 us a step, and how many steps there are
+// follows from how fast a cascade grows, G.ic_branching.
+// IC up to a branching of 1.3, where cascades are long or touch little: always (kColMaxEdges; above 0.8 up to
+// 1,000 edges a node).  Elsewhere by both estimated times, in us, the columns' with 0.4 of it on top: fits to
+// 1,595 calls of 1 to 20,000 trials (G(n, p), Watts-Strogatz, BA and R-MAT, 12,000 to 3 M edges, U[0, 1], WC and
+// uniform p) that leave 30 % (root mean square).  With the rule before, 443 of them took over 1.08 times the
+// passes' time, up to 8 times: G(5000, p) of 1 M edges, p = 0.05, 64 trials 1.3 against 0.4 ms, R-MAT 14 of 776,000
+// edges, p = 0.1, 1,000 trials 2.2 against 0.9 ms, G(20000, p) of 20 M edges, p = 0.1, one trial 13.2 against 0.4 ms.
+// LT: the passes' pull steps count dense rows faster than atomics on shared memory; 1,000 nodes, 20,000 trials,
+// 200 / 400 / 1,000 edges a node: 15.9 against 16.0 / 29.2 against 16.9 / 85 against 31 ms.
+bool columns_pay(int model, const cnd_graph_dev &G, int64_t trials, int64_t words) {
+    if (model == 1) return G.m <= 200ll * G.n;
+    if (G.m > kColMaxEdges) return false;
+    const double r = G.ic_branching;
+    if (r <= 0.8 || (r <= 1.3 && G.m <= 1000ll * G.n)) return true;
+    ColShape c;
+    int32_t bits = 0;
+    choose_shape(model, G, trials, c, bits);
+    const double columns = (double)std::max(words, (trials + bits - 1) / bits);
+    const double waves = std::max(1.0, columns / ((double)G.num_sms * c.per_sm));
+    const double steps = std::min(25.0, 3.0 + std::log((double)G.n) / std::log(r));
+    const double onward = std::pow(r, -0.7);  // the larger r, the fewer checks before a node is active
+    // hub rows are expanded one after the other
+    const double hubs = G.max_out_degree >= kHub ? 1.0 + 0.023 * G.max_out_degree * (double)G.n / (double)G.m : 1.0;
+    const double per_edge = (0.35 + 0.8 * (double)std::min<int64_t>(bits, std::max<int64_t>(2, trials)) * onward) * hubs * 1e-3;
+    const double t_columns = 90.0 + waves * c.per_sm * (double)G.m * per_edge;
+    const double t_passes = 160.0 + 48.0 * steps + 3.8e-4 * (double)G.m * (double)words * onward;
+    return 1.4 * t_columns < t_passes;
+}
+
 }  // namespace
 
 // Calls that run here.  Options that choose a form of the pass engine (width, work items, direction,
-// deferral, statistics, 32-bit sums) get the pass engine.  So do IC calls of many trials on the larger
-// graphs: with that many the pass engine's words are full, and one check of 64 trials costs it less than
+// deferral, statistics, 32-bit sums) get the pass engine.  So do dense graphs (columns_pay), and IC calls of
+// many trials on the larger graphs: with that many the pass engine's words are full, and one check of 64 trials costs it less than
 // two of 32 cost here.  The line is kWideTrials where an SM holds fewer than four columns (n > about
 // 5,500) and there are hub rows (kHub edges and more: one block's work), four times that where it holds
 // one column (n > about 12,000) and there are none.
@@ -506,12 +560,12 @@ bool column_shape(int model, const cnd_graph_dev &G, int per_sm, ColShape &c) {
 //   LT, any:       BA 5k 1,000 trials 2,395 -> 370 us, 65,536 trials 20.1 -> 8.1 ms
 constexpr int64_t kWideTrials = 4096;
 
-bool columns_fit(int model, const cnd_graph_dev &G, const cnd_sim_opts &o, int64_t trials) {
+bool columns_fit(int model, const cnd_graph_dev &G, const cnd_sim_opts &o, int64_t trials, int64_t words) {
     if (model == 1 && (!G.lt_cnt_edge || o.lt_accumulate)) return false;
     if (o.word_bits || o.chunk_edges || o.direction != CND_DIR_AUTO || o.pull_permille || o.defer_bits || o.stats)
         return false;
     ColShape c;
-    if (!column_shape(model, G, 1, c)) return false;
+    if (!column_shape(model, G, 1, c) || !columns_pay(model, G, trials, words)) return false;
     if (model == 1 || trials <= kWideTrials || column_shape(model, G, 4, c)) return true;
     return G.max_out_degree < kHub && (trials <= 4 * kWideTrials || column_shape(model, G, 2, c));
 }
@@ -520,27 +574,8 @@ cnd_status plan_columns(int model, const cnd_graph_dev &G, const std::vector<Ite
     int64_t trials = 0;
     for (const auto &it : items) trials += it.trials;
     if (trials == 0) return CND_OK;
-    // Blocks per SM and trials per column (a multiple of 4, one coin block), by estimated time: a
-    // wave of columns takes a constant (the latency of its steps) and work in proportion to the
-    // trials (and 2 more: work that a check takes whatever its trials) and the edges, at a rate in
-    // proportion to the block's threads.  1,000 trials, blocks per SM / trials per column: G(1000, 10000)
-    // 2 / 4 133 us, 1 / 8 148; Watts-Strogatz 10k U[0, 1] 2 / 4 648 us, 1 / 8 575; BA 5k WC 255 and 269.
-    const double size = std::min(1.0, std::max(0.25, (double)G.m / 1e5));
     ColShape c;
-    double best = 1e300;
-    for (int per_sm = 4; per_sm >= 1; per_sm >>= 1) {
-        ColShape k;
-        if (!column_shape(model, G, per_sm, k)) continue;
-        for (int b = 4; b <= 32; b += 4) {
-            const double waves = std::ceil((double)((trials + b - 1) / b) / ((double)G.num_sms * per_sm));
-            const double cost = waves * ((per_sm == 1 ? 10 : per_sm == 2 ? 9 : 8) + size * per_sm * (b + 2));
-            if (cost < best) {
-                best = cost;
-                plan.bits = b;
-                c = k;
-            }
-        }
-    }
+    choose_shape(model, G, trials, c, plan.bits);
     const int64_t slots = (int64_t)G.num_sms * c.per_sm;
     plan.items.resize(sizeof(ColItem) * items.size());
     ColItem *h = reinterpret_cast<ColItem *>(plan.items.data());

@@ -31,8 +31,8 @@ struct ColPlan {
     size_t dyn = 0, over = 0;
 };
 
-// True if a call of `trials` trials in all runs in the column engine.
-bool columns_fit(int model, const cnd_graph_dev &G, const cnd_sim_opts &o, int64_t trials);
+// True if a call of `trials` trials in all, in `words` words of 64 of the same item, runs in the column engine.
+bool columns_fit(int model, const cnd_graph_dev &G, const cnd_sim_opts &o, int64_t trials, int64_t words);
 
 cnd_status plan_columns(int model, const cnd_graph_dev &G, const std::vector<ItemDesc> &items, ColPlan &plan);
 

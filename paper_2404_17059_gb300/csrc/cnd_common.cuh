@@ -16,6 +16,10 @@ constexpr uint32_t kFull = 0xFFFFFFFFu;    // full warp mask
 constexpr uint32_t kNoSource = 0xFFFFFFFFu;
 constexpr int kPullShort = 64;
 constexpr int kPullItem = 255;  // an 8-bit bit-sliced count holds it
+// Graphs the column engine may take: two words of shared memory a node (so that node ids fit 16 bits), and for
+// IC the edges up to which it was measured (columns_pay)
+constexpr int kColMaxN = 227 * 1024 / 8;
+constexpr int kColMaxEdges = 4000000;
 
 // ---------------------------------------------------------------- Philox4x32-10
 // Counter-based generator of Salmon et al. (SC'11).  One call yields four
@@ -91,6 +95,9 @@ struct cnd_graph_dev {
     int32_t *in_row_ptr = nullptr;  // [n+1] in-CSR (pull direction)
     uint4 *in_edge = nullptr;       // [m] {src, edge id, IC threshold, LT weight}
     int32_t max_out_degree = 0;
+    // IC, graphs the column engine may take: how many out-edges of a node just reached over a live edge are
+    // live, on average (sum over e of p_e times the p of its target's out-edges, over the sum of p)
+    float ic_branching = 0.0f;
     int num_sms = 0;
     // LT counting form, set when every node's non-zero in-weights are equal (the weighted
     // cascade): node v keeps, per 64-trial word, L_v = bits(k_v) bit-sliced counter planes

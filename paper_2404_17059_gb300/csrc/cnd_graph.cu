@@ -266,6 +266,17 @@ cnd_status cnd_graph_create(int32_t n, int32_t m, const int32_t *row_ptr, const 
     d.n = n;
     d.m = m;
     d.max_out_degree = max_deg;
+    if (ic_prob && n <= kColMaxN && m <= kColMaxEdges) {
+        std::vector<double> live((size_t)n, 0.0);
+        for (int32_t u = 0; u < n; ++u)
+            for (int32_t e = row_ptr[u]; e < row_ptr[u + 1]; ++e) live[u] += ic_prob[e];
+        double all = 0.0, onward = 0.0;
+        for (int32_t e = 0; e < m; ++e) {
+            all += ic_prob[e];
+            onward += ic_prob[e] * live[col[e]];
+        }
+        d.ic_branching = all > 0.0 ? (float)(onward / all) : 0.0f;
+    }
     int32_t *d_col = nullptr, *d_tmp_a = nullptr, *d_tmp_b = nullptr;
     float *d_p = nullptr;
     uint32_t *d_w = nullptr;

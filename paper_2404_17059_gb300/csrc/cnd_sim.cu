@@ -2859,7 +2859,7 @@ static cnd_status simulate_common(int model, const cnd_graph *g, const char *fn,
     }
     // ---- items
     std::vector<ItemDesc> items((size_t)n_items);
-    int64_t total_trials = 0, n_seeds_total = 0;
+    int64_t total_trials = 0, total_words = 0, n_seeds_total = 0;
     for (int32_t i = 0; i < n_items; ++i) {
         ItemDesc &it = items[i];
         it.seed_begin = batched ? seed_off[i] : 0;
@@ -2873,6 +2873,7 @@ static cnd_status simulate_common(int model, const cnd_graph *g, const char *fn,
             return CND_EINVAL;
         }
         total_trials += it.trials;
+        total_words += (it.trials + 63) / 64;
         n_seeds_total = std::max(n_seeds_total, it.seed_end);
     }
     if (n_seeds_total > 0 && !seeds) {
@@ -2904,7 +2905,7 @@ static cnd_status simulate_common(int model, const cnd_graph *g, const char *fn,
     const size_t count_rows = batched ? (size_t)n_items : 1;
 
     // graphs whose per-trial state fits an SM's shared memory: one launch, a block per column of trials
-    const bool columns = columns_fit(model, G, o, total_trials);
+    const bool columns = columns_fit(model, G, o, total_trials, total_words);
     ColPlan plan;
     if (columns) {
         const cnd_status ps = plan_columns(model, G, items, plan);
@@ -3105,7 +3106,7 @@ cnd_status cnd_sim_plan(const cnd_graph *g, int32_t model, int32_t n_items, int6
         words += (items[i].trials + 63) / 64;
     }
     int32_t engine = CND_ENGINE_PASSES, bits = 0;
-    if (words > 0 && columns_fit(model, G, o, n_trials)) {
+    if (words > 0 && columns_fit(model, G, o, n_trials, words)) {
         ColPlan plan;
         const cnd_status st = plan_columns(model, G, items, plan);
         if (st != CND_OK) return st;

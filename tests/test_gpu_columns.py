@@ -191,3 +191,20 @@ def test_engine_of_a_call(model):
     assert all(engine[n] == "columns" for n in (1, 33, 6000)) and engine[30_000] == "passes"
     assert engine[23_300] == ("columns" if model == "ic" else "passes")
     assert engine[24_400] == "passes"
+
+
+def test_engine_of_dense_graphs():
+    """A column is one block's work: graphs whose edges take one SM longer than the passes' steps stay with those."""
+    n, rng = 5000, np.random.default_rng(1)
+
+    def engine(d, p_of, trials, model="ic"):
+        g = I.csr_from_edges(n, np.repeat(np.arange(n), d), rng.integers(0, n, n * d))
+        G = P.cnd_graph_create(n, g.row_ptr, g.col, p_of(g), I.lt_weighted_cascade(g))
+        return P.cnd_sim_plan(G, model, trials)[0]
+
+    for trials in (1, 64, 1000):
+        assert engine(200, lambda g: I.ic_uniform(g, 0.05), trials) == "passes"      # branching 10
+        assert engine(200, I.ic_weighted_cascade, trials) == "columns"              # branching 1
+        assert engine(10, lambda g: I.ic_uniform(g, 0.5), trials) == "columns"      # few edges
+        assert engine(400, I.ic_weighted_cascade, trials, "lt") == "passes"
+        assert engine(40, I.ic_weighted_cascade, trials, "lt") == "columns"
