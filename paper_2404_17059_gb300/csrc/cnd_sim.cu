@@ -79,13 +79,16 @@ constexpr int kLtTasks = 64;
 // small items spread a step over more of them (R-MAT-18, uneven weights, kTasks / kLtTasks: 16 words 59.6 /
 // 56.8 ms, 24 words 84.1 / 84.7, 32 words 108.6 / 110.7, 63 words 219 / 234).
 constexpr int kLtAccWords = 16;
-// ... of a slot of more than 32 pairs in an IC pass of more than 256 words on a graph of kWideNodes nodes
-// and more: its lanes go over the item's edges with the pairs they hold, so more edges per item pay
-// while a step has items enough for all warps (16 seed sets on R-MAT-20, 424 words: 515 / 482 / 472 ms per
-// call at 256 / 1,024 / 2,048 tasks; BA 100k, 157 words, few slots per step: 19.7 / 20.6 / 22.3 ms;
-// Watts-Strogatz 10k p = 0.1, 65,536 trials, 1,024 words: 3.60 / - / 4.03 ms)
+// ... of a slot of more than 32 pairs in an IC pass of more than 256 words: its lanes go over the item's edges with
+// the pairs they hold, so more edges per item pay while a step has items enough for all warps, 6 to 7 of them at
+// kWideChecks.  A step's checks decide for the frontier it produces.  ms per call, 256 / 2,048 tasks always / from
+// kWideChecks on: R-MAT-20 p = 0.01, 257 words 426 / 375 / 375, R-MAT-17 p = 0.01, 1,024 words 223 / 212 / 213, BA 100k
+// WC, 257 words 32.2 / 32.6 / 31.7, 1,024 words 112 / 103 / 102; with few slots per step G(100000, 1000000) p = 0.05,
+// 257 words 1.29 / 1.48 to 1.74 / 1.28, BA 100k p = 0.01, 257 words 2.60 / 2.79 / 2.59, Watts-Strogatz 10k p = 0.1,
+// 1,024 words 3.09 / 3.35 / 3.10.  (Sharing a wide item among warps instead, 2 to 8 of them: 1.84 to 2.05 on the
+// G(n, m).)
 constexpr int kWideTasks = 2048;
-constexpr int kWideNodes = 65536;
+constexpr unsigned long long kWideChecks = 128ull << 20;
 // AUTO without pull_permille: push only -- the pull step measured 1.3x to 3.7x
 // slower than push on every GB300 workload here (hub in-rows scanned by one warp)
 constexpr int kPullPermille = 1001;
@@ -111,6 +114,7 @@ struct Ctl {
     uint32_t stamp;  // stamp of that step
     int32_t force;   // 1: every waiting word is expanded now
     int32_t pull;    // 1: this step pulls (IC)
+    int32_t wide, wide_in;  // as in Params
     int32_t limit;   // a pass stopped at max_levels with trials still active
     int32_t timed_out;  // the device loop stopped at its time limit
     unsigned long long slots, items, levels, pull_steps;
@@ -127,7 +131,8 @@ struct Params {
     int32_t n, B, nq;
     int32_t chunk;             // > 0: fixed edges per work item
     int32_t tasks;             // else: (edge, pair) tasks per work item of a slot of up to 32 pairs
-    int32_t wide;              // tasks per work item of a slot with more than 32 pairs
+    int32_t wide, wide_in;     // tasks per work item of a slot with more than 32 pairs: of `out` and of `in`
+    int32_t wide_max;          // ... where the step has enough of them (wide_tasks)
     const int32_t *row_ptr;
     const uint2 *edge;         // {col, IC threshold} or {col, LT weight}
     uint64_t *vis, *nxt, *dmask;
@@ -187,6 +192,8 @@ __device__ __forceinline__ void resolve(Params &p) {
     p.lnext_cnt = p.lcnt + (odd ? 0 : 1);
     p.stamp = p.ctl->stamp;
     p.force = p.ctl->force;
+    p.wide = p.ctl->wide;
+    p.wide_in = p.ctl->wide_in;
     p.level = L + 1;
 }
 
@@ -206,9 +213,15 @@ __device__ __forceinline__ void add_level_count(const Params &p, unsigned long l
     if (lane_id() == 0 && v && p.level < p.lc_len) atomicAdd(&p.level_counts[p.level], v);
 }
 
-// Edges per work item for a slot with k pairs.
-__device__ __forceinline__ int edges_per_item(const Params &p, int k) {
-    return p.chunk > 0 ? p.chunk : max(1, (k > 32 ? p.wide : p.tasks) / max(k, 1));
+// Edges per work item for a slot with k pairs (wide: of the frontier the slot is in).
+__device__ __forceinline__ int edges_per_item(const Params &p, int k, int wide) {
+    return p.chunk > 0 ? p.chunk : max(1, (k > 32 ? wide : p.tasks) / max(k, 1));
+}
+
+// Tasks per work item of the slots of more than 32 pairs that a step produces, from the (edge, word) checks of its
+// own frontier.
+__host__ __device__ __forceinline__ int wide_tasks(const Params &p, unsigned long long checks) {
+    return checks >= kWideChecks ? p.wide_max : p.tasks;
 }
 
 // t / k for t < 2^32 / k (k <= kMaxB): multiply by ceil-ish reciprocal.
@@ -469,7 +482,7 @@ __global__ void __launch_bounds__(kBlock, MODE == 2 ? 4 : 6) k_finalize(Params p
                 }
             }
             const int deg = kept > 0 ? p.row_ptr[v + 1] - p.row_ptr[v] : 0;
-            const int ne = edges_per_item(p, kept);
+            const int ne = edges_per_item(p, kept, p.wide);
             if (lane == 0) {
                 s_kept[wid * kNPW + h] = kept;
                 s_nch[wid * kNPW + h] = deg > 0 ? (deg + ne - 1) / ne : 0;
@@ -563,7 +576,7 @@ __global__ void __launch_bounds__(kBlock, MODE == 2 ? 4 : 6) k_finalize(Params p
                 pos += __popc(bm);
             }
             const int nch = s_nch[e], wb = s_wb[e];
-            const int ne = edges_per_item(p, kept);
+            const int ne = edges_per_item(p, kept, p.wide);
             for (int c = lane; c < nch; c += 32) p.out.work[wb + c] = make_int2(slot, c * ne);
         }
     }
@@ -624,7 +637,7 @@ __global__ void __launch_bounds__(kBlock) k_collect(Params p_) {
             K += __popcll(dm);
         }
         if (K) deg = p.row_ptr[v + 1] - p.row_ptr[v];
-        const int ne = edges_per_item(p, K);
+        const int ne = edges_per_item(p, K, p.wide);
         const int hs = K > 0 ? 1 : 0;
         const int nch = deg > 0 ? (deg + ne - 1) / ne : 0;
         int sk = K, sh = hs, sc = nch, dg = deg;
@@ -751,7 +764,7 @@ __global__ void __launch_bounds__(kBlock) k_collect_wide(Params p_) {
         for (int h = 0; h < NN; ++h) {
             K[h] = __reduce_add_sync(kFull, __popcll(dm[h]));
             deg[h] = K[h] ? p.row_ptr[v[h] + 1] - p.row_ptr[v[h]] : 0;
-            const int ne = edges_per_item(p, K[h]);
+            const int ne = edges_per_item(p, K[h], p.wide);
             pairs += K[h];
             slots += K[h] > 0;
             items += (deg[h] + ne - 1) / ne;
@@ -780,7 +793,7 @@ __global__ void __launch_bounds__(kBlock) k_collect_wide(Params p_) {
                 p.out.poff[slot] = off;
                 p.out.pk[slot] = K[h];
             }
-            const int ne = edges_per_item(p, K[h]);
+            const int ne = edges_per_item(p, K[h], p.wide);
             const int nch = (deg[h] + ne - 1) / ne;
             for (int c = lane; c < nch; c += 32) p.out.work[item0 + c] = make_int2(slot, c * ne);
             item0 += nch;
@@ -950,7 +963,7 @@ __device__ __forceinline__ void push_ic(Params &p) {
         const int row0 = p.row_ptr[u];
         const int deg = p.row_ptr[u + 1] - row0;
         const int e_begin = row0 + it.y;
-        const int e_end = e_begin + min(edges_per_item(p, k), deg - it.y);
+        const int e_end = e_begin + min(edges_per_item(p, k, p.wide_in), deg - it.y);
         if (lane == 0) {
             n_edges += e_end - e_begin;
             n_fw += k;
@@ -1087,7 +1100,7 @@ __global__ void __launch_bounds__(kBlock, kPushMinBlocks) k_push(Params p_) {
         const int k = p.in.pk[it.x];
         const int row0 = p.row_ptr[u];
         const int deg = p.row_ptr[u + 1] - row0;
-        const int ne = edges_per_item(p, k);
+        const int ne = edges_per_item(p, k, p.wide_in);
         const int e_begin = row0 + it.y;
         const int e_cnt = min(ne, deg - it.y);
         const bool staged = k <= kStageB;
@@ -1756,6 +1769,7 @@ __global__ void k_pass_begin(Params p) {
     c->stamp += 1u;
     c->force = 1;
     c->pull = 0;
+    c->wide = c->wide_in = p.tasks;
 }
 
 // The host loop's decision, on the device: run step L (the first step of a
@@ -1797,6 +1811,8 @@ __global__ void k_ctl(Params p, cudaGraphConditionalHandle h, int32_t first, int
         c->level = L;
         c->stamp += 1u;
         c->force = items == 0 ? 1 : 0;
+        c->wide_in = c->wide;
+        c->wide = wide_tasks(p, checks);
         c->pull = (may_pull && items > 0 && tau == 0 &&
                    (pull_always || (lt ? lt_pull_pays(checks, m, p.B)
                                        : (int64_t)fedges * 1000 > (int64_t)permille * m)))
@@ -2220,7 +2236,7 @@ static cnd_status run_items(int model, const cnd_graph_dev &G, const char *fn, s
     P.nq = nq;
     P.chunk = chunk;
     P.tasks = tasks;
-    P.wide = model == 0 && B > 256 && n >= kWideNodes ? kWideTasks : tasks;
+    P.wide_max = model == 0 && B > 256 ? kWideTasks : tasks;
     P.row_ptr = G.row_ptr;
     P.edge = edge;
     P.rk = round_keys(items[0].key);
@@ -2421,6 +2437,7 @@ static cnd_status run_items(int model, const cnd_graph_dev &G, const char *fn, s
         P.lnext_cnt = d_lcnt;
         P.force = 1;
         P.stamp = stamp++;
+        P.wide = tasks;
         P.level = 0;
         k_seed<<<std::max<int>(1, (int)ps.size()), 128, 0, st>>>(P, d_segs, (int32_t)ps.size(), seeds_dev, d_bad);
         CND_CUDA_TRY(cudaGetLastError());
@@ -2462,6 +2479,8 @@ static cnd_status run_items(int model, const cnd_graph_dev &G, const char *fn, s
             CND_CUDA_TRY(cudaMemsetAsync(d_lcnt + ((L + 1) & 1), 0, sizeof(int32_t), st));
             P.in = fr[cur];
             P.out = fr[nx];
+            P.wide_in = P.wide;
+            P.wide = wide_tasks(P, checks);
             P.lin = lists[L & 1];
             P.lin_cnt = d_lcnt + (L & 1);
             P.lnext = lists[(L + 1) & 1];
@@ -3291,7 +3310,7 @@ static cnd_status simulate_noalloc(const cnd_graph *g, const int32_t *seeds, int
         P.B = B;
         P.nq = nq;
         P.chunk = 0;
-        P.tasks = P.wide = kTasks;
+        P.tasks = P.wide = P.wide_in = P.wide_max = kTasks;
         P.tau = 0;
         P.max_wait = 0;
         P.force = 0;

@@ -62,3 +62,26 @@ def test_wide_work_items():
     assert a.edge_checks == b.edge_checks
     c = oracle.simulate_threads("ic", g, seeds, 100, 4, ic_prob=p)
     assert np.array_equal(a.spread[:100], c.spread)
+
+
+def test_items_of_wide_passes_follow_the_step():
+    """Passes of more than 256 words: a frontier of a few seeds is dealt out edge by edge; on a graph whose steps
+    grow past the line of wider items and fall below it again, results stay those of narrow passes."""
+    g = I.erdos_renyi_m(70_000, 700_000, graph_seed=2)
+    G = P.cnd_graph_create(g.n, g.row_ptr, g.col, np.zeros(g.m, dtype=np.float32), None)
+    seeds = I.top_degree_seeds(g, 6)
+    a = P.cnd_ic_simulate_ex(G, seeds, 64 * 300, 1, word_bits=64 * 300, stats=2)
+    assert a.stats["passes"] == 1 and a.stats["work_items"] == g.out_degree()[seeds].sum()
+    g = I.rmat(14, 16 << 14, graph_seed=2)
+    G = P.cnd_graph_create(g.n, g.row_ptr, g.col, I.ic_uniform(g, 0.1), None)
+    seeds, T = I.top_degree_seeds(g, 20), 64 * 1100 - 7
+    kw = dict(edge_checks=True, level_counts_len=16)
+    b = P.cnd_ic_simulate_ex(G, seeds, T, 3, word_bits=64 * 200, **kw)
+    items = {}
+    for graph in (0, 1):
+        a = P.cnd_ic_simulate_ex(G, seeds, T, 3, word_bits=64 * 1100, graph=graph, stats=2, **kw)
+        assert a.stats["passes"] == 1
+        items[graph] = a.stats["work_items"]
+        assert np.array_equal(a.spread, b.spread) and np.array_equal(a.node_count, b.node_count)
+        assert a.edge_checks == b.edge_checks and np.array_equal(a.level_counts, b.level_counts)
+    assert items[0] == items[1]
