@@ -728,7 +728,7 @@ def kernel_name(model, s):
 def alg_bytes(model, s):
     """Bytes the expansion kernel must move, from its own work counters: 8 per work item (row_ptr pair),
     8 per frontier word loaded, 8 per edge read ({col, thr}), 8 per word check (the target's word; of a
-    pull step the words of the frontier rows it adds) and
+    pull step the source's, read for every in-edge from the frontier) and
     16 per IC word update (vis and next read-modify-write), 8 per LT accumulator add (4-byte read-modify-
     write) or 16 per counter-plane update of the LT counting form (8-byte read-modify-write)."""
     base = 8 * s["work_items"] + 8 * s["frontier_words"] + 8 * s["edges_scanned"] + 8 * s["word_checks"]

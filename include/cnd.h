@@ -98,7 +98,9 @@ typedef struct cnd_sim_stats {
     /* CND_STATS_COUNT only: */
     int64_t edges_scanned;     /* frontier out-edges read by the expansion kernels */
     int64_t frontier_words;    /* frontier words loaded by the expansion kernels */
-    int64_t word_checks;       /* (edge, word) pairs with frontier bits: target word read */
+    int64_t word_checks;       /* (edge, word) pairs with frontier bits: target word read; of LT pull
+                                  steps (in-edge from the frontier, word of the pass) pairs: the
+                                  source's word read */
     int64_t draws;             /* Philox blocks drawn (IC coins; LT thresholds) */
     int64_t updates;           /* IC: (edge, target word) pairs with live coins for inactive trials
                                   (each or-ed into the target's words); LT: accumulator adds, or

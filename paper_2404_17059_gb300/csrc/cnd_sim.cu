@@ -1645,7 +1645,6 @@ __global__ void __launch_bounds__(kBlock, 3) k_pull_lt(Params p_) {
             }
             a.carry2(ca[0], ca[1]);
             b.carry2(cb[0], cb[1]);
-            n_wc += 16;
         }
     };
     // bring the counters of words w, w + 1 (of the last word of an odd pass: its own) into L2 while the rows
@@ -1667,7 +1666,10 @@ __global__ void __launch_bounds__(kBlock, 3) k_pull_lt(Params p_) {
         if (!__any_sync(kFull, open)) continue;
         int count = 0;
         for (int e = 0; e < len; e += 128) scan(list, count, d.y + e + lane, len - e - lane, 32, kFull);
-        if (lane == 0) n_edges += len;
+        if (lane == 0) {
+            n_edges += len;
+            n_wc += count;
+        }
         if (count == 0) continue;
         if (lane < 8 * SEG) list[count + lane] = (uint32_t)p.n;
         __syncwarp();
@@ -1716,6 +1718,7 @@ __global__ void __launch_bounds__(kBlock, 3) k_pull_lt(Params p_) {
         const int longest = __shfl_sync(kFull, len, 0);  // items are in descending order
         for (int e = 0; e < longest; e += 4 * LN) scan(list, count, d.y + e + l, len - e - l, LN, seg_mask);
         n_edges += l == 0 ? len : 0;
+        n_wc += count;
         if (__any_sync(kFull, count != 0)) {
             if (l < 8) list[count + l] = (uint32_t)p.n;
             __syncwarp();
@@ -1746,7 +1749,7 @@ __global__ void __launch_bounds__(kBlock, 3) k_pull_lt(Params p_) {
     }
     if (lb.n) lb.flush(p);
     count_add(p, C_EDGES, n_edges);
-    count_add(p, C_WCHECKS, n_wc);
+    count_add(p, C_WCHECKS, l == 0 ? (unsigned long long)n_wc * B : 0ull);  // n_wc listed sources, each of B words
     count_add(p, C_UPDATES, n_up);
 }
 

@@ -95,3 +95,17 @@ def test_dense_frontier_pulls_by_itself():
         a = _run(G, seeds, 1000, 2, graph=graph)
         assert 0 < a.stats["pull_steps"] < a.stats["levels"]
         _same(a, push)
+
+
+@pytest.mark.parametrize("words", [1, 2, 3, 16, 17, 40])
+def test_word_checks_of_a_pull_step(words):
+    """Every in-edge comes from a seed and no target activates: one pull step, which reads the words of the pass
+    once for each in-edge, whatever it pads its lists and lanes with."""
+    k = len(IN_DEGREES)
+    n = 1600 + k
+    g = I.csr_from_edges(n, np.concatenate([np.arange(d) for d in IN_DEGREES]), np.repeat(np.arange(1600, n), IN_DEGREES))
+    G = P.cnd_graph_create(n, g.row_ptr, g.col, None, np.ones(g.m, dtype=np.uint32))
+    seeds = np.arange(1600)
+    a = _run(G, seeds, 64 * words - 5, 1, direction="pull", word_bits=64 * words)
+    assert np.all(a.spread == 1600) and a.stats["pull_steps"] == a.stats["levels"] == 1
+    assert a.stats["word_checks"] == g.m * words
