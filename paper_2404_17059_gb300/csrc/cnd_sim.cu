@@ -2123,17 +2123,17 @@ static PassWidth pass_width(int model, const cnd_graph_dev &G, const cnd_sim_opt
     const int32_t n = G.n;
     const bool lt_cnt = counting_form(model, G, o);
     const double budget = 0.6 * (double)free_b;
-    // bytes per word column: vis, nxt, two pair pools (+ LT accumulators or counter planes, and what its work
-    // items take more than IC's)
-    const int tasks_min = model == 0 ? kTasks : kLtTasks;
-    const double per_word = (double)n * (2 * 8 + 2 * 10 + (model == 1 && !lt_cnt ? 256 : 0)) +
-                            (lt_cnt ? 8.0 * (double)G.lt_planes : 0.0) +
-                            (o.chunk_edges > 0 ? 0.0 : 32.0 * (double)G.m * (1.0 / tasks_min - 1.0 / kTasks));
     // IC pulls only when asked to: by direction, or by a switch threshold; LT in the counting form
     // chooses per step (lt_pull_pays)
     const bool lt_pull = lt_cnt && G.m > 0 && o.direction != CND_DIR_PUSH && o.defer_bits == 0;
     const bool ic_pull = model == 0 && G.m > 0 &&
                          (o.direction == CND_DIR_PULL || (o.direction == CND_DIR_AUTO && o.pull_permille > 0));
+    // bytes per word column: vis, nxt, two pair pools (+ the pull's frontier rows, LT accumulators or counter
+    // planes, and what LT's work items take more than IC's)
+    const int tasks_min = model == 0 ? kTasks : kLtTasks;
+    const double per_word = (double)n * (2 * 8 + 2 * 10 + (lt_pull || ic_pull ? 8 : 0) + (model == 1 && !lt_cnt ? 256 : 0)) +
+                            (lt_cnt ? 8.0 * (double)G.lt_planes : 0.0) +
+                            (o.chunk_edges > 0 ? 0.0 : 32.0 * (double)G.m * (1.0 / tasks_min - 1.0 / kTasks));
     int64_t bmax = o.word_bits ? o.word_bits / 64 : kMaxB;
     bmax = std::min<int64_t>(bmax, std::max<int64_t>(1, (int64_t)(budget / per_word)));
     bmax = std::min<int64_t>(bmax, ic_pull ? kPullMaxB : kMaxB);

@@ -109,3 +109,19 @@ def test_word_checks_of_a_pull_step(words):
     a = _run(G, seeds, 64 * words - 5, 1, direction="pull", word_bits=64 * words)
     assert np.all(a.spread == 1600) and a.stats["pull_steps"] == a.stats["levels"] == 1
     assert a.stats["word_checks"] == g.m * words
+
+
+def test_pass_width_has_room_for_the_frontier_rows():
+    """The words of a pass, planned for little free memory: its state, the pull's rows by node among it, stays
+    within 60 % of that."""
+    g = I.erdos_renyi_m(50_000, 200_000, graph_seed=3)
+    G = P.cnd_graph_create(g.n, g.row_ptr, g.col, I.ic_uniform(g, 0.1), I.lt_weighted_cascade(g))
+    planes = sum(int(k).bit_length() for k in g.in_degree())
+    free = 100 << 20
+    state = 2 * 8 + 2 * 10  # per node and word: vis, nxt, two pools
+    for model, kw, per_word in (("lt", {}, g.n * (state + 8) + 8 * planes), ("lt", {"direction": "push"}, g.n * state + 8 * planes),
+                                ("ic", {"pull_permille": 250}, g.n * (state + 8)), ("ic", {}, g.n * state)):
+        engine, bits = P.cnd_sim_plan(G, model, 10_000_000, free_bytes=free, **kw)
+        words = bits // 64
+        assert engine == "passes" and words > 8
+        assert words * per_word <= 0.6 * free < (words + 4) * per_word, (model, kw, words)
