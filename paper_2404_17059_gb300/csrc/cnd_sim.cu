@@ -2721,9 +2721,23 @@ static int log2_bucket(int64_t x) {
 static cnd_status simulate_common(int model, const cnd_graph *g, const char *fn, int32_t n_items,
                                   const int64_t *seed_off, const int32_t *seeds, const int32_t *n_trials_arr,
                                   int64_t n_trials_one, const uint64_t *keys, uint64_t key_one, int32_t *spread_out,
-                                  int32_t *count_out, const cnd_sim_opts *opts);
+                                  int32_t *count_out, const cnd_sim_opts *opts, int engine = -1);
 
-// Times the candidates on a sample; returns the best settings.
+// The engine of the whole call with the settings of the default candidate (all 0).
+static int default_engine(int model, const cnd_graph_dev &G, int32_t n_items, const int32_t *n_trials_arr,
+                          int64_t n_trials_one, cnd_sim_opts o) {
+    o.word_bits = o.chunk_edges = o.pull_permille = 0;
+    int64_t trials = 0, words = 0;
+    for (int32_t i = 0; i < n_items; ++i) {
+        const int64_t t = n_trials_arr ? n_trials_arr[i] : n_trials_one;
+        trials += t;
+        words += (t + 63) / 64;
+    }
+    return words > 0 && columns_fit(model, G, o, trials, words) ? CND_ENGINE_COLUMNS : CND_ENGINE_PASSES;
+}
+
+// Times the candidates on a sample, each in the engine that the whole call takes with it (fewer trials may suit the
+// other one); returns the best settings.
 static cnd_status tune(int model, const cnd_graph *g, int32_t n_items, const int64_t *seed_off, const int32_t *seeds,
                        const int32_t *n_trials_arr, int64_t n_trials_one, const uint64_t *keys, uint64_t key_one,
                        bool batched, const cnd_sim_opts &base, TuneVal &best, double &best_ms) {
@@ -2755,6 +2769,7 @@ static cnd_status tune(int model, const cnd_graph *g, int32_t n_items, const int
     o.level_counts_len = 0;
     o.max_levels = 0;
     o.direction = CND_DIR_AUTO;
+    const int plain = default_engine(model, g->d, batched ? n_items : 1, n_trials_arr, n_trials_one, base);
     const bool dev = o.device_ptrs != 0;
     // outputs of the sample runs
     int32_t *d_sp = nullptr;
@@ -2771,11 +2786,14 @@ static cnd_status tune(int model, const cnd_graph *g, int32_t n_items, const int
     best_ms = 1e300;
     // one untimed run first (first-call costs: pool growth, module load)
     cnd_status st = simulate_common(model, g, "cnd_autotune", batched ? ns_items : 1, seed_off, seeds,
-                                    batched ? tr.data() : nullptr, batched ? 0 : tr[0], keys, key_one, sp, nullptr, &o);
+                                    batched ? tr.data() : nullptr, batched ? 0 : tr[0], keys, key_one, sp, nullptr, &o,
+                                    plain);
     for (int32_t wb : widths)
         for (int32_t ch : chunks)
             for (int32_t pm : pulls)
                 for (int32_t gr : {0, 1}) {
+                    const int engine = wb == 0 && ch == 0 && pm == 0 ? plain : CND_ENGINE_PASSES;
+                    if (engine == CND_ENGINE_COLUMNS && gr) continue;  // the same call
                     o.word_bits = wb;
                     o.chunk_edges = ch;
                     o.pull_permille = pm;
@@ -2785,7 +2803,7 @@ static cnd_status tune(int model, const cnd_graph *g, int32_t n_items, const int
                         const auto t0 = std::chrono::steady_clock::now();
                         st = simulate_common(model, g, "cnd_autotune", batched ? ns_items : 1, seed_off, seeds,
                                              batched ? tr.data() : nullptr, batched ? 0 : tr[0], keys, key_one, sp,
-                                             nullptr, &o);
+                                             nullptr, &o, engine);
                         if (st == CND_OK && dev) st = cudaStreamSynchronize((cudaStream_t)o.stream) == cudaSuccess
                                                           ? CND_OK
                                                           : CND_ECUDA;
@@ -2811,7 +2829,8 @@ static cnd_status apply_autotune(int model, const cnd_graph *g, int32_t n_items,
         total += batched ? n_trials_arr[i] : n_trials_one;
         n_seeds += batched ? seed_off[i + 1] - seed_off[i] : seed_off[1];
     }
-    const auto key = std::make_tuple((const void *)g, model, batched ? 1 : 0, log2_bucket(total),
+    const int plain = default_engine(model, g->d, batched ? n_items : 1, n_trials_arr, n_trials_one, o);
+    const auto key = std::make_tuple((const void *)g, model, (batched ? 1 : 0) | plain << 1, log2_bucket(total),
                                      log2_bucket(std::max<int64_t>(1, n_seeds / std::max(1, batched ? n_items : 1))));
     TuneVal tv{};
     bool hit = false;
@@ -2845,11 +2864,11 @@ static bool bad_opts(const cnd_sim_opts &o) {
            o.defer_steps > 255 || o.lt_accumulate < 0 || o.lt_accumulate > 1;
 }
 
-// Shared front end of the single and batched entry points.
+// Shared front end of the single and batched entry points (engine: CND_ENGINE_*, -1 by rule).
 static cnd_status simulate_common(int model, const cnd_graph *g, const char *fn, int32_t n_items,
                                   const int64_t *seed_off, const int32_t *seeds, const int32_t *n_trials_arr,
                                   int64_t n_trials_one, const uint64_t *keys, uint64_t key_one, int32_t *spread_out,
-                                  int32_t *count_out, const cnd_sim_opts *opts) {
+                                  int32_t *count_out, const cnd_sim_opts *opts, int engine) {
     clear_error();
     cnd_sim_opts o;
     cnd_sim_opts_init(&o);
@@ -2927,7 +2946,7 @@ static cnd_status simulate_common(int model, const cnd_graph *g, const char *fn,
     const size_t count_rows = batched ? (size_t)n_items : 1;
 
     // graphs whose per-trial state fits an SM's shared memory: one launch, a block per column of trials
-    const bool columns = columns_fit(model, G, o, total_trials, total_words);
+    const bool columns = engine < 0 ? columns_fit(model, G, o, total_trials, total_words) : engine == CND_ENGINE_COLUMNS;
     ColPlan plan;
     if (columns) {
         const cnd_status ps = plan_columns(model, G, items, plan);

@@ -410,3 +410,24 @@ def test_timeout_stops_the_call_and_leaves_the_context_usable(ba, graph):
     assert ei.value.status == P.CND_ETIMEOUT
     assert "timed out" in P.cnd_last_error()
     assert_same(sim("lt", G, seeds, 640, 1, graph=graph), ref("lt", g, seeds, 640, 1, w=w))
+
+
+def test_autotune_times_the_engine_of_the_whole_call():
+    """More trials than the sample's 4,096 take the pass engine on this graph, where 4,096 take the columns: the
+    sample has to run in the engine of the whole call.  A time limit that every call passes tells which it was: the
+    pass engine's host loop does not report a device loop."""
+    import ctypes as C
+    from paper_2404_17059_gb300 import binding
+    g = I.barabasi_albert(7000, 10, graph_seed=3)
+    G = P.cnd_graph_create(g.n, g.row_ptr, g.col, I.ic_weighted_cascade(g), None)
+    seeds = np.ascontiguousarray(I.top_degree_seeds(g, 20), dtype=np.int32)
+    base, best, ms = P.cnd_sim_opts_init(), P.cnd_sim_opts_init(), C.c_double()
+    base.timeout_s = 1e-9
+    for trials, engine in ((4096, "columns"), (20_000, "passes")):
+        assert P.cnd_sim_plan(G, "ic", trials)[0] == engine
+        tr, key = np.array([trials], dtype=np.int32), np.array([1], dtype=np.uint64)
+        st = binding.load().cnd_autotune(G.handle, 0, 0, None, seeds.ctypes.data, seeds.size, tr.ctypes.data,
+                                         key.ctypes.data, C.byref(base), C.byref(best), C.byref(ms))
+        assert st == P.CND_ETIMEOUT
+        assert ("device loop" in P.cnd_last_error()) == (engine == "columns")
+    assert P.cnd_autotune(G, "ic", seeds, 20_000, 1)["sample_ms"] > 0
