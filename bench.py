@@ -138,6 +138,13 @@ class Workload:
                                                       stats=stats, graph=graph)))
         return out
 
+    def engines(self, P, G):
+        """The engine that each model's calls take without statistics (statistics keep a call in the passes)."""
+        if self.batch is not None:
+            tr = np.asarray(self.batch[2], dtype=np.int64)
+            return {"ic": P.cnd_sim_plan(G, "ic", int(tr.sum()), n_items=len(tr))[0]}
+        return {m: P.cnd_sim_plan(G, m, self.trials[m])[0] for m in ("ic", "lt") if self.models.get(m) is not None}
+
     def host_seeds(self):
         return self.seeds if self.batch is None else self.batch[1]
 
@@ -788,6 +795,10 @@ def run_ours(args):
 
     # step indices: 0 the counted call, then warm-up, timed, graph-mode and end-to-end steps, so that
     # single-seed-set workloads rotate through their trial ranges (Workload.first_trial)
+    # Statistics keep a call in the pass engine: where the calls run in the column engine without, the steps that
+    # give `value` go without, and the kernels' event times come from further steps
+    engines = wl.engines(P, G)
+    in_columns = "columns" in engines.values()
     step = 0
     counted = dict(wl.calls(P, G, seeds_d, rank, stats=CND_STATS_COUNT, step=step, world=world))  # work counts
     for _ in range(args.warmup):
@@ -801,22 +812,29 @@ def run_ours(args):
     ev = [(torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)) for _ in range(args.steps)]
     checks = launches = 0
     exp_ms, exp_n, fin_ms, set_ms, mchecks = {}, {}, {}, {}, {}
+
+    def add_kernel_times(res):
+        for model, r in res:
+            exp_ms[model] = exp_ms.get(model, 0.0) + r.stats["expand_ms"]
+            exp_n[model] = exp_n.get(model, 0) + r.stats["expand_launches"]
+            fin_ms[model] = fin_ms.get(model, 0.0) + r.stats["finalize_ms"]
+            set_ms[model] = set_ms.get(model, 0.0) + r.stats["setup_ms"]
+            mchecks[model] = mchecks.get(model, 0) + r.edge_checks
+
     wall0 = time.perf_counter()
     with ClockSampler(local) as clk:
         for i in range(args.steps):
             step += 1
             flush.zero_()  # L2 flush (256 MiB write) outside the timed events
             ev[i][0].record(stream)
-            res = wl.calls(P, G, seeds_d, rank, stats=CND_STATS_TIMING, step=step, world=world)
+            res = wl.calls(P, G, seeds_d, rank, stats=0 if in_columns else CND_STATS_TIMING, step=step, world=world)
             ev[i][1].record(stream)
-            for model, r in res:
-                checks += r.edge_checks
-                launches += r.stats["launches"]
-                exp_ms[model] = exp_ms.get(model, 0.0) + r.stats["expand_ms"]
-                exp_n[model] = exp_n.get(model, 0) + r.stats["expand_launches"]
-                fin_ms[model] = fin_ms.get(model, 0.0) + r.stats["finalize_ms"]
-                set_ms[model] = set_ms.get(model, 0.0) + r.stats["setup_ms"]
-                mchecks[model] = mchecks.get(model, 0) + r.edge_checks
+            checks += sum(r.edge_checks for _, r in res)
+            if in_columns:  # a call is one launch (of a model whose calls are not, at least one)
+                launches += len(res)
+            else:
+                launches += sum(r.stats["launches"] for _, r in res)
+                add_kernel_times(res)
         torch.cuda.synchronize()
     wall = time.perf_counter() - wall0
     if dist:
@@ -833,6 +851,13 @@ def run_ours(args):
         checks_all = float(c.item())
     value = checks_all / (total_ms / 1e3)
     trials_per_s = world * wl.trials_per_step() * args.steps / (total_ms / 1e3)
+
+    kern_steps = args.steps
+    if in_columns:
+        kern_steps = max(1, args.graph_steps)
+        for _ in range(kern_steps):
+            step += 1
+            add_kernel_times(wl.calls(P, G, seeds_d, rank, stats=CND_STATS_TIMING, step=step, world=world))
 
     # ---- a few more steps as one CUDA-graph launch per call (device-side step loop; no per-kernel events)
     ng = max(1, args.graph_steps)
@@ -874,16 +899,16 @@ def run_ours(args):
         b_per_check = alg_bytes(model, cs) / max(1, r.edge_checks)
         tb = b_per_check * mchecks[model]  # algorithmic bytes of the timed steps
         n_l = max(1, exp_n[model])
-        kern[model] = {"kernel": name, "launches_per_step": n_l / args.steps, "avg_launch_ms": exp_ms[model] / n_l,
+        kern[model] = {"kernel": name, "launches_per_step": n_l / kern_steps, "avg_launch_ms": exp_ms[model] / n_l,
                        "alg_bytes_per_launch": tb / n_l, "alg_bytes_per_edge_check": b_per_check,
                        "achieved_gbs": tb / (exp_ms[model] * 1e-3) / 1e9 if exp_ms[model] > 0 else None,
-                       "expand_ms_per_step": exp_ms[model] / args.steps,
-                       "edge_checks_per_step": mchecks[model] / args.steps,
+                       "expand_ms_per_step": exp_ms[model] / kern_steps,
+                       "edge_checks_per_step": mchecks[model] / kern_steps,
                        "edge_checks_per_s_expand": mchecks[model] / (exp_ms[model] * 1e-3)
                        if exp_ms[model] > 0 else None,
                        "hbm_bound_edge_checks_per_s": hbm_bound_rate(peak, r.edge_checks, alg_bytes(model, cs)),
-                       "finalize_ms_per_step": fin_ms[model] / args.steps,
-                       "setup_ms_per_step": set_ms[model] / args.steps,
+                       "finalize_ms_per_step": fin_ms[model] / kern_steps,
+                       "setup_ms_per_step": set_ms[model] / kern_steps,
                        "lt_counters": cs.get("lt_counters", 0) if model == "lt" else None,
                        "passes": cs["passes"], "word_bits": cs["word_bits"], "levels": cs["levels"],
                        "counted_call": {"edge_checks": r.edge_checks,
@@ -898,6 +923,9 @@ def run_ours(args):
             "traffic": ncu_traffic(K["kernel"], traffic_key(wl, args), wc_per_launch), "kernel": K["kernel"],
             "peak_source": f"{peak_kind} (MEASURED_PEAKS.json hbm_gbs, burst copy)" if peak_kind == "measured"
             else "fallback"}
+    if roof["traffic"] and K["avg_launch_ms"] > 0:  # what of that reaches the HBM
+        roof["traffic_gbs"] = roof["traffic"] / (K["avg_launch_ms"] * 1e-3) / 1e9
+        roof["traffic_frac"] = roof["traffic_gbs"] / peak
     # the IC push draws Philox-4x32-10 blocks for its coins: where its draws outweigh its bytes it is
     # bound by integer arithmetic, and its roofline is the Philox rate, measured here on this device
     # with the engine's own generator (cnd_philox_rate)
@@ -949,11 +977,15 @@ def run_ours(args):
         "config": {"workload": wl.desc, "name": wl.name, "graph_nodes": wl.g.n, "graph_edges": wl.g.m,
                    "graph_sha256": wl.g.digest(), "trials_per_step_per_rank": wl.trials_per_step(),
                    "trials_per_model_per_step": wl.trials, "parallelism": f"trial-sharded x{world}",
-                   "call_mode": "host step loop (the default), CUDA events around each expansion launch",
+                   "engines": engines,
+                   "call_mode": "column engine (the default here), no statistics; kernel figures from further steps in "
+                                "the pass engine" if in_columns else
+                                "host step loop (the default), CUDA events around each expansion launch",
                    "l2": "flushed between timed steps (256 MiB write, outside the step events)"},
         "trials_per_s": trials_per_s,
         "graph_mode": {"steps": ng, "ms_per_step": graph_ms / ng, "value": g_checks * world / (graph_ms / 1e3),
-                       "note": "further steps (their own trial ranges), one CUDA-graph launch per call (opts.graph=1)"},
+                       "note": "further steps (their own trial ranges), opts.graph=1: one CUDA-graph launch per call in "
+                               "the pass engine, no effect in the column engine (config.engines)"},
         "edge_checks_per_step": checks_all / args.steps,
         "clocks": clk.summary(),
         "e2e": {"value": world * e2e_checks / e2e_s, "unit": UNIT, "h2d_bytes_per_step": h2d,
