@@ -255,7 +255,9 @@ __device__ __forceinline__ void store_sum(const Item &item, const float2 (&acc)[
 // length, so the four are alike.  What bounds it is the latency of item, edge and row loads and, before,
 // instructions on padding (ncu: 60 % issue active at 12 % L2 throughput).  R-MAT-17 (1.94 M edges): 64 -> 36 us;
 // R-MAT-20 (16.1 M): 409 -> 272 us (2.06 GB of rows gathered).
-__global__ void __launch_bounds__(256) k_spmm_in(int32_t n_items, int32_t n_long, const Item *__restrict__ items,
+// Past an item's end q is 0 and the row is row n, which is zero: 0 is added whatever any node's row holds (with a
+// node's row there, 0 times its overflown features would make the sum NaN).
+__global__ void __launch_bounds__(256) k_spmm_in(int32_t n, int32_t n_items, int32_t n_long, const Item *__restrict__ items,
                                                  const uint2 *__restrict__ in_c, const __nv_bfloat16 *__restrict__ h,
                                                  __nv_bfloat16 *__restrict__ a, float *__restrict__ scratch) {
     const int lane = threadIdx.x & 31;
@@ -271,20 +273,19 @@ __global__ void __launch_bounds__(256) k_spmm_in(int32_t n_items, int32_t n_long
         for (int i = 0; i < 4; ++i) acc[i] = make_float2(0.0f, 0.0f);
         for (int32_t b = item.begin; b < item.end; b += 32) {
             const int cnt = min(32, item.end - b);
-            uint2 my = make_uint2(0u, 0u);
+            uint2 my = make_uint2((uint32_t)n, 0u);
             if (lane < cnt) my = in_c[b + lane];
             const float myq = edge_q(my.y);
             for (int j = 0; j < cnt; j += 16) {
-                // edges j + sub + 4 r, r = 0..3 (q = 0 past the end: row 0 read, nothing added)
+                // edges j + sub + 4 r, r = 0..3
                 uint4 rr[4];
                 float qq[4];
 #pragma unroll
                 for (int r = 0; r < 4; ++r) {
                     const int e = j + sub + 4 * r;
-                    const uint32_t u = __shfl_sync(0xffffffffu, my.x, e & 31);
-                    const float q = __shfl_sync(0xffffffffu, myq, e & 31);
-                    qq[r] = e < cnt ? q : 0.0f;
-                    rr[r] = *reinterpret_cast<const uint4 *>(h + (size_t)(e < cnt ? u : 0u) * H + f8);
+                    const uint32_t u = __shfl_sync(0xffffffffu, my.x, e);
+                    qq[r] = __shfl_sync(0xffffffffu, myq, e);
+                    rr[r] = *reinterpret_cast<const uint4 *>(h + (size_t)u * H + f8);
                 }
 #pragma unroll
                 for (int r = 0; r < 4; ++r) fma_row(acc, qq[r], rr[r]);
@@ -314,7 +315,7 @@ __global__ void __launch_bounds__(256) k_spmm_in(int32_t n_items, int32_t n_long
 #pragma unroll
             for (int i = 0; i < 4; ++i) acc[c][i] = make_float2(0.0f, 0.0f);
         for (int b = 0; b < longest; b += 8) {
-            uint2 my = make_uint2(0u, 0u);  // past the end: q = 0, row 0 read, nothing added
+            uint2 my = make_uint2((uint32_t)n, 0u);
             if (b + l < len) my = in_c[item.begin + b + l];
             const float myq = edge_q(my.y);
 #pragma unroll
@@ -405,7 +406,7 @@ __device__ __forceinline__ void add4(float4 &a, const float4 &b) {
 // chain per half, 8 rows in flight; the others half a warp each.  An item of a split node writes its
 // partial row (k_split_out_finish adds them in order); a single-item node is read-modify-written by its
 // lanes.  R-MAT-17: 102 -> 52 us (497 MB of rows gathered).
-__global__ void __launch_bounds__(256) k_spmm_out(int32_t n_items, int32_t n_long, const Item *__restrict__ items,
+__global__ void __launch_bounds__(256) k_spmm_out(int32_t n, int32_t n_items, int32_t n_long, const Item *__restrict__ items,
                                                   const uint2 *__restrict__ ic_edge, const float *__restrict__ da,
                                                   float *__restrict__ dh, float *__restrict__ scratch) {
     const int lane = threadIdx.x & 31;
@@ -429,7 +430,7 @@ __global__ void __launch_bounds__(256) k_spmm_out(int32_t n_items, int32_t n_lon
         float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
         for (int32_t b = item.begin; b < item.end; b += 32) {
             const int cnt = min(32, item.end - b);
-            uint2 my = make_uint2(0u, 0u);
+            uint2 my = make_uint2((uint32_t)n, 0u);
             if (lane < cnt) my = ic_edge[b + lane];
             const float myq = edge_q(my.y);
             for (int j = 0; j < cnt; j += 8) {
@@ -438,10 +439,9 @@ __global__ void __launch_bounds__(256) k_spmm_out(int32_t n_items, int32_t n_lon
 #pragma unroll
                 for (int r = 0; r < 4; ++r) {
                     const int e = j + sub + 2 * r;
-                    const uint32_t w = __shfl_sync(0xffffffffu, my.x, e & 31);
-                    const float q = __shfl_sync(0xffffffffu, myq, e & 31);
-                    qq[r] = e < cnt ? q : 0.0f;
-                    xx[r] = *reinterpret_cast<const float4 *>(da + (size_t)(e < cnt ? w : 0u) * H + f4);
+                    const uint32_t w = __shfl_sync(0xffffffffu, my.x, e);
+                    qq[r] = __shfl_sync(0xffffffffu, myq, e);
+                    xx[r] = *reinterpret_cast<const float4 *>(da + (size_t)w * H + f4);
                 }
 #pragma unroll
                 for (int r = 0; r < 4; ++r) fma_row4(acc, qq[r], xx[r]);
@@ -465,7 +465,7 @@ __global__ void __launch_bounds__(256) k_spmm_out(int32_t n_items, int32_t n_lon
         float4 acc[2];
         acc[0] = acc[1] = make_float4(0.f, 0.f, 0.f, 0.f);
         for (int b = 0; b < longest; b += 16) {
-            uint2 my = make_uint2(0u, 0u);
+            uint2 my = make_uint2((uint32_t)n, 0u);
             if (b + l < len) my = ic_edge[item.begin + b + l];
             const float myq = edge_q(my.y);
             for (int j = 0; j < 16 && b + j < longest; j += 4) {
@@ -1205,7 +1205,7 @@ void seed_clear(cnd_sur *s, const int32_t *d_seeds, int32_t ns, cudaStream_t st)
 }
 
 void aggregate_in(cnd_sur *s, const __nv_bfloat16 *hin, __nv_bfloat16 *aout, cudaStream_t st) {
-    k_spmm_in<<<s->spmm_in_blocks, 256, 0, st>>>(s->n_items_in, s->n_long_in, s->items_in, s->in_c, hin, aout, s->scratch);
+    k_spmm_in<<<s->spmm_in_blocks, 256, 0, st>>>(s->n, s->n_items_in, s->n_long_in, s->items_in, s->in_c, hin, aout, s->scratch);
     if (s->n_split)
         k_split_finish<<<grid_for((int64_t)s->n_split * 32, 256, s->num_sms), 256, 0, st>>>(
             s->n_split, s->split_node, s->split_first, s->scratch, aout);
@@ -1223,7 +1223,7 @@ void forward(cnd_sur *s, cudaStream_t st) {
 }
 
 void aggregate_out(cnd_sur *s, const float *da, float *dh, cudaStream_t st) {
-    k_spmm_out<<<s->spmm_out_blocks, 256, 0, st>>>(s->n_items_out, s->n_long_out, s->items_out, s->g->d.ic_edge, da, dh, s->scratch_out);
+    k_spmm_out<<<s->spmm_out_blocks, 256, 0, st>>>(s->n, s->n_items_out, s->n_long_out, s->items_out, s->g->d.ic_edge, da, dh, s->scratch_out);
     if (s->n_split_out)
         k_split_out_finish<<<grid_for((int64_t)s->n_split_out * 32, 256, s->num_sms), 256, 0, st>>>(
             s->n_split_out, s->split_out_node, s->split_out_first, s->scratch_out, dh);
@@ -1384,7 +1384,7 @@ cnd_status cnd_sur_create(const cnd_graph *g, const float *params, cnd_sur **out
     SUR_ALLOC(s->part_d, (size_t)grid_for(n, 256, s->num_sms));
     SUR_ALLOC(s->x, nr * D0);
     SUR_ALLOC(s->a1, nr * D0);
-    for (int l = 0; l < 3; ++l) SUR_ALLOC(s->h[l], nr * H);
+    for (int l = 0; l < 3; ++l) SUR_ALLOC(s->h[l], (nr + 1) * H);  // a row of zeros behind the last (aggregations)
     SUR_ALLOC(s->a[1], nr * H);
     SUR_ALLOC(s->a[2], nr * H);
     SUR_ALLOC(s->e, nr * H);
@@ -1392,7 +1392,7 @@ cnd_status cnd_sur_create(const cnd_graph *g, const float *params, cnd_sur **out
     SUR_ALLOC(s->acc0, nr);
     SUR_ALLOC(s->dhA, nr * H);
     SUR_ALLOC(s->dhB, nr * H);
-    SUR_ALLOC(s->da, nr * H);
+    SUR_ALLOC(s->da, (nr + 1) * H);
     SUR_ALLOC(s->ds0, nr);
     SUR_ALLOC(s->da0, nr);
     SUR_ALLOC(s->yv, nr);
@@ -1411,6 +1411,9 @@ cnd_status cnd_sur_create(const cnd_graph *g, const float *params, cnd_sur **out
         (e = up(s->split_out_node, split_out)) != cudaSuccess || (e = up(s->split_out_first, first_out)) != cudaSuccess)
         return fail(e, "split rows");
     if ((e = cudaMemset(s->acc0, 0, sizeof(unsigned long long) * nr)) != cudaSuccess) return fail(e, "memset");
+    for (auto *h : s->h)
+        if ((e = cudaMemset(h + nr * H, 0, sizeof(*h) * H)) != cudaSuccess) return fail(e, "memset");
+    if ((e = cudaMemset(s->da + nr * H, 0, sizeof(float) * H)) != cudaSuccess) return fail(e, "memset");
     const int sms = s->num_sms;
     if (m > 0) k_in_compact<<<grid_for(m, 256, sms), 256>>>(m, G.in_edge, s->in_c);
     k_features<<<grid_for(n, 256, sms), 256>>>(n, G.row_ptr, G.in_row_ptr, s->x);
