@@ -90,18 +90,12 @@ struct BlockState {
     __align__(16) uint32_t rk[20];
 };
 
-__device__ __forceinline__ unsigned long long timer_ns() {
-    unsigned long long t;
-    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-    return t;
-}
-
 // True once the time limit, measured from the call's first step (t0), has passed; the call then times out.  A
 // timer that reads before another SM's t0 is not past it.
 __device__ __forceinline__ bool past_limit(const ColParams &p) {
     if (p.timeout_ns == 0) return false;
     if (*(volatile int32_t *)&p.flags->timed_out) return true;
-    const unsigned long long t0 = *(volatile unsigned long long *)&p.flags->t0, now = timer_ns();
+    const unsigned long long t0 = *(volatile unsigned long long *)&p.flags->t0, now = global_ns();
     if (t0 == 0 || now <= t0 || now - t0 <= p.timeout_ns) return false;
     p.flags->timed_out = 1;
     return true;
@@ -321,7 +315,7 @@ __global__ void __launch_bounds__(1024, 1) k_columns(ColParams p) {
                 (i < cap ? la : ga)[i] = (uint16_t)u;
             }
         }
-        if (tid == 0 && p.timeout_ns) atomicCAS(&p.flags->t0, 0ull, timer_ns());
+        if (tid == 0 && p.timeout_ns) atomicCAS(&p.flags->t0, 0ull, global_ns());
         __syncthreads();
         if (tid == 0 && p.lc_len > 0 && S.n_list[0]) atomicAdd(&p.level_counts[0], (unsigned long long)S.n_list[0] * nt);
         uint16_t *lcur = la, *lnext = lb, *gcur = ga, *gnext = gb;

@@ -115,6 +115,13 @@ struct cnd_graph_dev {
     int32_t n_lt_pull_items = 0, n_lt_long = 0;
 };
 
+// the GPU's global timer
+__device__ __forceinline__ unsigned long long global_ns() {
+    unsigned long long t;
+    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+    return t;
+}
+
 // ---------------------------------------------------------------- errors
 void set_error(const char *fmt, ...);
 void clear_error();

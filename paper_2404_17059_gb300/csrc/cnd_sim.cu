@@ -113,19 +113,13 @@ struct Ctl {
     int32_t level;   // step being run: frontier fr[level & 1] -> fr[(level + 1) & 1]; -1: the seed step
     uint32_t stamp;  // stamp of that step
     int32_t force;   // 1: every waiting word is expanded now
-    int32_t pull;    // 1: this step pulls (IC)
+    int32_t pull;    // 1: this step pulls
     int32_t wide, wide_in;  // as in Params
     int32_t limit;   // a pass stopped at max_levels with trials still active
     int32_t timed_out;  // the device loop stopped at its time limit
     unsigned long long slots, items, levels, pull_steps;
     unsigned long long t0;  // global timer (ns) when the call's first step began
 };
-
-__device__ __forceinline__ unsigned long long global_ns() {
-    unsigned long long t;
-    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-    return t;
-}
 
 struct Params {
     int32_t n, B, nq;
@@ -1581,6 +1575,7 @@ __global__ void __launch_bounds__(kBlock, 3) k_pull_lt(Params p_) {
     Params p = p_;
     resolve(p);
     if (p.ctl && !p.ctl->pull) return;
+    static_assert(LN == 8 || LN == 16, "long items add their odd words in a second segment");
     constexpr int SEG = 32 / LN;
     constexpr int kLong = 256 + 8 * SEG;           // list entries of a long item, padded
     constexpr int kShort = kPullShort + 8;         // ... of a short one
@@ -1590,7 +1585,8 @@ __global__ void __launch_bounds__(kBlock, 3) k_pull_lt(Params p_) {
     const int lane = lane_id();
     const int wid = threadIdx.x >> 5;
     const int seg = lane / LN, l = lane % LN;
-    const uint32_t seg_mask = (LN == 32 ? 0xFFFFFFFFu : (1u << (LN & 31)) - 1u) << (seg * LN);
+    constexpr uint32_t kSeg = (1u << LN) - 1u;
+    const uint32_t seg_mask = kSeg << (seg * LN);
     const uint32_t below = (1u << lane) - 1u;
     ListBuf lb{s_list[wid], 0};
     const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -1701,7 +1697,7 @@ __global__ void __launch_bounds__(kBlock, 3) k_pull_lt(Params p_) {
                 act = pull_apply_shared(p, v, (uint32_t)d.w, w + seg, need, a, n_up);
             }
             const uint32_t m = __ballot_sync(kFull, act != 0ull);
-            record(v, ch, lane == 0, m & ((1u << (LN & 31)) - 1u), (m >> LN) & ((1u << (LN & 31)) - 1u));
+            record(v, ch, lane == 0, m & kSeg, (m >> LN) & kSeg);
         }
         __syncwarp();
     }
