@@ -902,33 +902,34 @@ __global__ void __launch_bounds__(256) k_reduce_dw(int32_t nblocks, int32_t din,
     }
 }
 
-// grad (bias of `layer`; head: also w_o, b_o and the loss, which is summed in 64 bits) += the blocks' partial
-// sums: blocks of 32 x 32 threads, 32 values each
+// grad (bias of `layer`; head: also w_o, b_o and the loss) += the blocks' partial sums: blocks of 32 x 32
+// threads, 32 values each; the loss, which is summed in 64 bits, is the last block's, a thread per partial sum
 __global__ void __launch_bounds__(1024) k_reduce_bwd(int32_t nblocks, const float *__restrict__ part, int layer, int head,
                                                      float *__restrict__ grad, double *__restrict__ loss,
                                                      float loss_scale) {
+    if (head && blockIdx.x == gridDim.x - 1) {
+        __shared__ double s_loss[32];
+        double l = 0.0;
+        for (int b = 32 * threadIdx.y + threadIdx.x; b < nblocks; b += 1024) l += (double)part[(size_t)b * kBwdPart + 2 * H + 1];
+        for (int o = 16; o; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
+        if (threadIdx.x == 0) s_loss[threadIdx.y] = l;
+        __syncthreads();
+        if (threadIdx.y != 0) return;
+        l = s_loss[threadIdx.x];
+        for (int o = 16; o; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
+        if (threadIdx.x == 0) *loss += l * (double)loss_scale;
+        return;
+    }
     __shared__ float s[32][33];
-    __shared__ double s_loss[32];
-    const int c = blockIdx.x * 32 + threadIdx.x;  // 0 .. 2 H + 1
-    const bool ok = c < (head ? 2 * H + 1 : H), is_loss = head && c == 2 * H + 1;
+    const int c = blockIdx.x * 32 + threadIdx.x;  // 0 .. 2 H
+    const bool ok = c < (head ? 2 * H + 1 : H);
     float sum = 0.0f;
     if (ok) {
 #pragma unroll 8
         for (int b = threadIdx.y; b < nblocks; b += 32) sum += part[(size_t)b * kBwdPart + c];
     }
-    if (is_loss) {
-        double l = 0.0;
-        for (int b = threadIdx.y; b < nblocks; b += 32) l += (double)part[(size_t)b * kBwdPart + c];
-        s_loss[threadIdx.y] = l;
-    }
     sum = tree_sum(s, sum);
-    if (threadIdx.y != 0) return;
-    if (ok) grad[c < H ? off_b(layer) + c : (c < 2 * H ? OFF_WO + (c - H) : OFF_BO)] += sum;
-    if (is_loss) {
-        double l = 0.0;
-        for (int i = 0; i < 32; ++i) l += s_loss[i];
-        *loss += l * (double)loss_scale;
-    }
+    if (ok && threadIdx.y == 0) grad[c < H ? off_b(layer) + c : (c < 2 * H ? OFF_WO + (c - H) : OFF_BO)] += sum;
 }
 
 // yhat and the predicted spread; screening scores
@@ -1257,8 +1258,8 @@ void backward_loss(cnd_sur *s, const float *y, const int32_t *cnt, float inv_t, 
     __nv_bfloat16 *wt2 = s->wt + 64 * 32 + 64 * 128, *wt1 = s->wt + 64 * 32;
     // each gradient kernel writes per-block partial sums; the reduce kernels add them up in block order
     auto bias = [&](int layer, int head) {
-        k_reduce_bwd<<<head ? (kBwdPart + 31) / 32 : H / 32, dim3(32, 32), 0, st>>>(tbb, s->part, layer, head, s->grad,
-                                                                                    ha.loss, ha.loss_scale);
+        k_reduce_bwd<<<head ? (2 * H + 1 + 31) / 32 + 1 : H / 32, dim3(32, 32), 0, st>>>(tbb, s->part, layer, head, s->grad,
+                                                                                         ha.loss, ha.loss_scale);
     };
     auto weights = [&](int layer, int din) {
         k_reduce_dw<<<H * 2 * din / 32, dim3(32, 8), 0, st>>>(db, din, s->part, layer, s->grad);
