@@ -118,6 +118,7 @@ struct Ctl {
     int32_t limit;   // a pass stopped at max_levels with trials still active
     int32_t timed_out;  // the device loop stopped at its time limit
     unsigned long long slots, items, levels, pull_steps;
+    unsigned long long pull_bodies;  // steps of a loop whose body has the pull's kernels
     unsigned long long t0;  // global timer (ns) when the call's first step began
 };
 
@@ -1755,9 +1756,14 @@ __global__ void __launch_bounds__(kBlock, 3) k_pull_lt(Params p_) {
 // / 12, / 20 and / 40 checks: R-MAT-21, B = 16: 435 / 161 / 149 / 148 / 151; B = 64: 1,893 / 527 / 475 / 473 /
 // 489; BA 100k with 10 edges a node, B = 157: 151 / 69.5 / 62.7 / 61.7 / 63.4.  Below B = 8 a scan of the
 // in-edges has too few words to pay for it: the line stays at that of 8 words (R-MAT-21, B = 1, above 1.3 m,
-// 0.67 m, 0.4 m, 0.2 m: 42.3 / 42.0 / 45.9 / 52.2).
+// 0.67 m, 0.4 m, 0.2 m: 42.3 / 42.0 / 45.9 / 52.2).  Steps of fewer than kPullMin checks have too little to save
+// for two more launches: us per call, push only / no such line / 1 M / 2 M / 4 M checks: R-MAT 15 x 8, 400 trials
+// 4,401 / 4,961 / 4,492 / 4,499 / 4,483, BA 30k, 4,096 trials, 2 seeds 3,071 / 3,366 / 3,359 / 3,163 / 3,087, R-MAT 16,
+// 1,000 trials 13,091 / 10,978 / 10,953 / 10,988 / 11,456, BA 100k, 400 trials 3,973 / 3,321 / 3,316 / 3,339 / 3,450.
+constexpr unsigned long long kPullMin = 2000000ull;
+
 __host__ __device__ __forceinline__ bool lt_pull_pays(unsigned long long checks, int64_t m, int32_t B) {
-    return checks * 12ull > (unsigned long long)m * (unsigned long long)(B > 8 ? B : 8);
+    return checks >= kPullMin && checks * 12ull > (unsigned long long)m * (unsigned long long)(B > 8 ? B : 8);
 }
 
 // ---------------------------------------------------------------- device step loop
@@ -1771,19 +1777,34 @@ __global__ void k_pass_begin(Params p) {
     c->wide = c->wide_in = p.tasks;
 }
 
+// The step loops of a pass: one, or for LT that may pull two: pushes, and from the first step on that pulls and has
+// kPullLoop checks, steps whose body also has the pull's three kernels.  Those take 6 us a step also where they
+// return at once, so that a long cascade of small steps should never get there.  us per call, push only / one loop /
+// two, the second from the first pull on / from kPullLoop checks on: G(30000, 300000), 64 trials, 340 steps without
+// a pull 8,984 / 11,183 / 9,250 / 9,250; G(30000, 120000), 1,000 trials, 53 of 321 steps pull 7,719 / - / 9,327 / 7,603;
+// R-MAT 16, 1,000 trials, 37 of 93 7,869 / - / 4,708 / 4,745; R-MAT 19, 1,000 trials 80,266 / - / 30,987 / 30,988.
+// A second loop that is not entered takes 15 us a pass and 0.7 us a step, so a call whose steps cannot reach the
+// line has one, of pushes (pass_width).
+constexpr unsigned long long kPullLoop = 4000000ull;
+struct Loops {
+    cudaGraphConditionalHandle h[2];
+    int32_t n;
+};
+
 // The host loop's decision, on the device: run step L (the first step of a
 // pass, or the one after the step just finalized)?  Prepares its counters and
-// sets the WHILE condition of the pass's step loop.
+// sets the WHILE conditions of the pass's step loops.
 // The device loop's step control (one thread): census of the frontier the last step produced,
 // stop at an empty frontier, the level cap or the time limit (timeout_ns > 0, measured on the GPU's
-// global timer from the call's first step), else set up the next step.
-__global__ void k_ctl(Params p, cudaGraphConditionalHandle h, int32_t first, int32_t max_levels, int32_t may_pull,
+// global timer from the call's first step), else set up the next step and the loop that runs it.  at: the loop of
+// the step just run, -1 after the seed step.
+__global__ void k_ctl(Params p, Loops loops, int32_t at, int32_t max_levels, int32_t may_pull,
                       int32_t lt, int32_t pull_always, int32_t permille, int64_t m, int32_t tau,
                       unsigned long long timeout_ns) {
     Ctl *c = p.ctl;
     const unsigned long long now = global_ns();
     if (c->t0 == 0ull) c->t0 = now;
-    const int L = first ? 0 : c->level + 1;
+    const int L = at < 0 ? 0 : c->level + 1;
     const bool odd = (L & 1) != 0;
     const int32_t *cnt = odd ? p.fr[1].cnt : p.fr[0].cnt;
     const int32_t slots = cnt[1], items = cnt[2], fedges = cnt[3];
@@ -1817,10 +1838,19 @@ __global__ void k_ctl(Params p, cudaGraphConditionalHandle h, int32_t first, int
                                        : (int64_t)fedges * 1000 > (int64_t)permille * m)))
                       ? 1
                       : 0;
+        if (loops.n == 2 && at < 1 && !pull_always && checks < kPullLoop) c->pull = 0;
         c->levels += 1ull;
         c->pull_steps += (unsigned long long)c->pull;
     }
-    cudaGraphSetConditional(h, (unsigned)go);
+    const int next = loops.n == 2 && (at == 1 || c->pull) ? 1 : 0;
+    if (go && may_pull && next == loops.n - 1) c->pull_bodies += 1ull;
+    // conditions keep their values: only what changes is set (1 us each)
+    if (at < 0) {
+        for (int i = 0; i < loops.n; ++i) cudaGraphSetConditional(loops.h[i], go && i == next ? 1u : 0u);
+    } else if (!go || next != at) {
+        cudaGraphSetConditional(loops.h[at], 0u);
+        if (go) cudaGraphSetConditional(loops.h[next], 1u);
+    }
 }
 
 // ---------------------------------------------------------------- outputs
@@ -2137,7 +2167,10 @@ static PassWidth pass_width(int model, const cnd_graph_dev &G, const cnd_sim_opt
     if (model == 1 && G.m > 0)  // a step's work items are counted in 32 bits
         bmax = std::min<int64_t>(bmax, std::max<int64_t>(1, (0x7FFFFFFFll - n - G.m) * tasks_min / (2 * (int64_t)G.m)));
     const int64_t n_pass = (total_words + bmax - 1) / bmax;
-    return PassWidth{(int)((total_words + n_pass - 1) / n_pass), lt_pull, ic_pull};
+    const int B = (int)((total_words + n_pass - 1) / n_pass);
+    // a step has m B checks at most
+    const bool ever = o.direction == CND_DIR_PULL || (uint64_t)G.m * (uint64_t)B >= (o.graph ? kPullLoop : kPullMin);
+    return PassWidth{B, lt_pull && ever, ic_pull};
 }
 
 // Runs the items' trials: words of all items are packed into passes of B
@@ -2578,7 +2611,6 @@ static cnd_status run_items(int model, const cnd_graph_dev &G, const char *fn, s
             cudaGraph_t gout = nullptr;
             return cudaStreamEndCapture(cs, &gout);
         };
-        const int body_kernels = (may_pull ? 3 : 0) + 3;
         const unsigned long long timeout_ns =
             o.timeout_s > 0 ? (unsigned long long)std::max(1.0, std::min(o.timeout_s * 1e9, 1.8e19)) : 0ull;
         for (size_t pass = 0; pass < passes.size(); ++pass) {
@@ -2586,8 +2618,14 @@ static cnd_status run_items(int model, const cnd_graph_dev &G, const char *fn, s
             Params Q = pass_params(pass, P);
             const bool pw = pinfo[pass].perword;
             const int32_t nw_here = pinfo[pass].nw_here;
-            cudaGraphConditionalHandle h;
-            CND_CUDA_TRY(cudaGraphConditionalHandleCreate(&h, gr.g, 0, 0));
+            Loops loops{};
+            loops.n = lt_pull ? 2 : 1;
+            for (int i = 0; i < loops.n; ++i) CND_CUDA_TRY(cudaGraphConditionalHandleCreate(&loops.h[i], gr.g, 0, 0));
+            auto control = [&](int at) {
+                k_ctl<<<1, 1, 0, cs>>>(Q, loops, at, o.max_levels, may_pull ? 1 : 0, lt_pull ? 1 : 0,
+                                       o.direction == CND_DIR_PULL ? 1 : 0, permille, (int64_t)G.m, P.tau, timeout_ns);
+                return cudaGetLastError();
+            };
             // set-up and seed step
             CND_CUDA_TRY(cap_begin(gr.g, tail));
             CND_CUDA_TRY(cudaMemsetAsync(P.vis, 0, sizeof(uint64_t) * nB, cs));
@@ -2605,34 +2643,30 @@ static cnd_status run_items(int model, const cnd_graph_dev &G, const char *fn, s
             k_seed<<<std::max<int>(1, (int)ps.size()), 128, 0, cs>>>(Q, pass_segs(pass), (int32_t)ps.size(),
                                                                       seeds_dev, d_bad);
             CND_CUDA_TRY(launch(k_seedfin, seed_blocks, cs, Q));
-            k_ctl<<<1, 1, 0, cs>>>(Q, h, 1, o.max_levels, may_pull ? 1 : 0, lt_pull ? 1 : 0,
-                                   o.direction == CND_DIR_PULL ? 1 : 0,
-                                   permille, (int64_t)G.m, P.tau, timeout_ns);
-            CND_CUDA_TRY(cudaGetLastError());
+            CND_CUDA_TRY(control(-1));
             CND_CUDA_TRY(cap_end(&tail));
-            // the step loop
-            cudaGraphNodeParams cp = {};
-            cp.type = cudaGraphNodeTypeConditional;
-            cp.conditional.handle = h;
-            cp.conditional.type = cudaGraphCondTypeWhile;
-            cp.conditional.size = 1;
-            cudaGraphNode_t loop_node;
-            CND_CUDA_TRY(cudaGraphAddNode(&loop_node, gr.g, tail.data(), nullptr, tail.size(), &cp));
-            cudaGraph_t body = cp.conditional.phGraph_out[0];
-            CND_CUDA_TRY(cap_begin(body, {}));
-            if (may_pull) {
-                CND_CUDA_TRY(launch(k_set, dense_blocks, cs, Q));
-                CND_CUDA_TRY(launch(pw ? k_pull_pw : k_pull_uk, pull_blocks, cs, Q));
-                CND_CUDA_TRY(launch(k_clear, dense_blocks, cs, Q));
+            // the step loops
+            for (int i = 0; i < loops.n; ++i) {
+                cudaGraphNodeParams cp = {};
+                cp.type = cudaGraphNodeTypeConditional;
+                cp.conditional.handle = loops.h[i];
+                cp.conditional.type = cudaGraphCondTypeWhile;
+                cp.conditional.size = 1;
+                cudaGraphNode_t loop_node;
+                CND_CUDA_TRY(cudaGraphAddNode(&loop_node, gr.g, tail.data(), nullptr, tail.size(), &cp));
+                cudaGraph_t body = cp.conditional.phGraph_out[0];
+                CND_CUDA_TRY(cap_begin(body, {}));
+                if (may_pull && i == loops.n - 1) {
+                    CND_CUDA_TRY(launch(k_set, dense_blocks, cs, Q));
+                    CND_CUDA_TRY(launch(pw ? k_pull_pw : k_pull_uk, pull_blocks, cs, Q));
+                    CND_CUDA_TRY(launch(k_clear, dense_blocks, cs, Q));
+                }
+                CND_CUDA_TRY(launch(pw ? k_push_pw : k_push_uk, push_blocks, cs, Q));
+                CND_CUDA_TRY(launch(pw ? k_fin_pw : k_fin_uk, fin_blocks, cs, Q));
+                CND_CUDA_TRY(control(i));
+                CND_CUDA_TRY(cap_end(nullptr));
+                tail.assign(1, loop_node);
             }
-            CND_CUDA_TRY(launch(pw ? k_push_pw : k_push_uk, push_blocks, cs, Q));
-            CND_CUDA_TRY(launch(pw ? k_fin_pw : k_fin_uk, fin_blocks, cs, Q));
-            k_ctl<<<1, 1, 0, cs>>>(Q, h, 0, o.max_levels, may_pull ? 1 : 0, lt_pull ? 1 : 0,
-                                   o.direction == CND_DIR_PULL ? 1 : 0,
-                                   permille, (int64_t)G.m, P.tau, timeout_ns);
-            CND_CUDA_TRY(cudaGetLastError());
-            CND_CUDA_TRY(cap_end(nullptr));
-            tail.assign(1, loop_node);
             // outputs of the pass
             CND_CUDA_TRY(cap_begin(gr.g, tail));
             CND_CUDA_TRY(launch_spread(G, cs, P.vis, B, nw_here, pass_wout(pass), d_spread));
@@ -2672,7 +2706,7 @@ static cnd_status run_items(int model, const cnd_graph_dev &G, const char *fn, s
             return CND_ETIMEOUT;
         }
         if (hc.limit) limit_hit = true;
-        launches += (int64_t)hc.levels * body_kernels;
+        launches += 3 * (int64_t)(hc.levels + hc.pull_bodies);
         if (S) {
             S->levels = (int32_t)hc.levels;
             S->frontier_slots = (int64_t)hc.slots;

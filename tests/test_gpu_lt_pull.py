@@ -125,3 +125,30 @@ def test_pass_width_has_room_for_the_frontier_rows():
         words = bits // 64
         assert engine == "passes" and words > 8
         assert words * per_word <= 0.6 * free < (words + 4) * per_word, (model, kw, words)
+
+
+def test_graph_loop_without_pulls_launches_none():
+    """The CUDA-graph loop of a sparse cascade runs three kernels a step; from the first step that pulls on, six."""
+    for g, pulls in ((I.erdos_renyi_m(30_000, 300_000, graph_seed=4), False), (I.rmat(15, 16 << 15, graph_seed=4), True)):
+        w = I.lt_weighted_cascade(g)
+        G = P.cnd_graph_create(g.n, g.row_ptr, g.col, None, w)
+        seeds = I.top_degree_seeds(g, 100 if pulls else 2)
+        push = _run(G, seeds, 1000, 2, direction="push", graph=1)
+        a = _run(G, seeds, 1000, 2, graph=1)
+        _same(a, push)
+        s, base = a.stats, push.stats["launches"] - 3 * push.stats["levels"]  # outside the loop
+        assert s["levels"] == push.stats["levels"] and (s["pull_steps"] > 0) == pulls
+        extra = s["launches"] - base - 3 * s["levels"]
+        assert extra == 0 if not pulls else 3 * s["pull_steps"] <= extra <= 3 * s["levels"]
+
+
+def test_small_steps_push():
+    """Steps of few checks have nothing to save by pulling, however dense their frontier."""
+    g = I.erdos_renyi_m(30_000, 120_000, graph_seed=4)
+    w = I.lt_weighted_cascade(g)
+    G = P.cnd_graph_create(g.n, g.row_ptr, g.col, None, w)
+    seeds = I.top_degree_seeds(g, 3000)
+    for T in (64, 400):
+        a = _run(G, seeds, T, 2)
+        assert a.stats["pull_steps"] == 0
+        _same(a, _run(G, seeds, T, 2, direction="pull"))
