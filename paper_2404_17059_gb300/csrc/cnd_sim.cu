@@ -722,11 +722,14 @@ __global__ void __launch_bounds__(kBlock) k_collect(Params p_) {
 }
 
 // The same for passes of more than kCollectNq dirty-mask words (B up to kMaxB; a node's words hardly fit a
-// lane each).  A warp takes kWideNodesPerWarp listed nodes, lane q holding mask word q of each, places their
+// lane each).  A warp takes up to kWideNodesPerWarp listed nodes, lane q holding mask word q of each, places their
 // slots, pool pairs and work items with one atomic each, and goes over a node's words 128 at a time, four
-// coalesced loads of nxt per lane in flight.  Moves 26 bytes per pair; against the block-cooperative
-// finalize, whose lanes search the mask for their words: 35.9 ms -> 5.7 ms a call for 530 words on R-MAT-20;
-// at 157 words k_collect is the faster (2.07 against 3.81 ms a call on BA 100k).
+// coalesced loads of nxt per lane in flight, or, where the nodes have few of them, over their pairs, a lane each.
+// Moves 26 bytes per pair; against the block-cooperative finalize, whose lanes search the mask for their words: 35.9 ->
+// 5.7 ms a call for 530 words on R-MAT-20, and, over pairs and with the census added once per block (four additions
+// of every warp at one address took a third of a step's time), batches on G(20000, 100000), 100 items of 1,000 trials
+// IC 5.2 -> 3.9 ms, LT 16.0 -> 11.7 ms; 500 items of 33 trials 2.93 -> 2.79 and 8.6 -> 8.2 ms (over words alone 8.2,
+// 24.5, 4.1 and 11.9 ms).  At 157 words k_collect is the faster (2.07 against 3.81 ms a call on BA 100k).
 constexpr int kWideNodesPerWarp = 4;
 
 __global__ void __launch_bounds__(kBlock) k_collect_wide(Params p_) {
@@ -739,13 +742,15 @@ __global__ void __launch_bounds__(kBlock) k_collect_wide(Params p_) {
     const int B = p.B, nq = p.nq;
     const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int n_warps = (gridDim.x * blockDim.x) >> 5;
-    unsigned long long pc = 0;
-    for (int base = warp * NN; base < count; base += n_warps * NN) {
+    unsigned long long pc = 0, checks = 0;
+    int edges = 0;
+    const int per = min(NN, (count + n_warps - 1) / n_warps);  // short lists: all warps get some
+    for (int base = warp * per; base < count; base += n_warps * per) {
         int v[NN], K[NN], deg[NN];
         uint64_t dm[NN];
 #pragma unroll
         for (int h = 0; h < NN; ++h) {
-            v[h] = base + h < count ? p.lin[base + h] : -1;
+            v[h] = h < per && base + h < count ? p.lin[base + h] : -1;
             dm[h] = 0ull;
             if (v[h] >= 0 && lane < nq) {
                 uint64_t *d = p.dmask + (size_t)v[h] * nq + lane;
@@ -753,8 +758,7 @@ __global__ void __launch_bounds__(kBlock) k_collect_wide(Params p_) {
                 if (dm[h]) *d = 0ull;
             }
         }
-        int pairs = 0, slots = 0, items = 0, edges = 0;
-        unsigned long long checks = 0;
+        int pairs = 0, slots = 0, items = 0;
 #pragma unroll
         for (int h = 0; h < NN; ++h) {
             K[h] = __reduce_add_sync(kFull, __popcll(dm[h]));
@@ -772,14 +776,64 @@ __global__ void __launch_bounds__(kBlock) k_collect_wide(Params p_) {
         if (lane == 0) {
             ps0 = atomicAdd((unsigned long long *)p.out.cnt, ((unsigned long long)slots << 32) | (unsigned)pairs);
             if (items) item0 = atomicAdd(&p.out.cnt[2], items);
-            if (edges) {
-                atomicAdd(&p.out.cnt[3], edges);
-                atomicAdd((unsigned long long *)(p.out.cnt + 4), checks);
-            }
         }
         ps0 = __shfl_sync(kFull, ps0, 0);
         item0 = __shfl_sync(kFull, item0, 0);
         int off = (int)(uint32_t)ps0, slot = (int)(ps0 >> 32);
+        int rounds = 0, groups = 0;
+#pragma unroll
+        for (int h = 0; h < NN; ++h) {
+            const unsigned m = __ballot_sync(kFull, dm[h] != 0ull);
+            groups += __popc((m | (m >> 1)) & 0x55555555u);
+            rounds = max(rounds, (K[h] + 31) >> 5);
+        }
+        const bool few = NN * rounds < groups;
+        if (few) {
+            // a lane per pair, the loads of all nodes in flight
+            int first[NN];  // pairs in the mask words of the lanes before
+#pragma unroll
+            for (int h = 0; h < NN; ++h) {
+                const int c = __popcll(dm[h]);
+                first[h] = c;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const int x = __shfl_up_sync(kFull, first[h], o);
+                    if (lane >= o) first[h] += x;
+                }
+                first[h] -= c;
+            }
+            for (int r = lane; r < 32 * rounds; r += 32) {
+                uint64_t x[NN];
+                int w[NN];
+#pragma unroll
+                for (int h = 0; h < NN; ++h) {
+                    w[h] = -1;
+                    x[h] = 0ull;
+                    if (r - lane >= K[h]) continue;
+                    int q = 0;  // the last lane with first <= r: it has pairs, or r is past the last one
+#pragma unroll
+                    for (int s = 16; s >= 1; s >>= 1)
+                        if (__shfl_sync(kFull, first[h], (q + s) & 31) <= r) q += s;
+                    const uint64_t d = __shfl_sync(kFull, dm[h], q);
+                    const int f = __shfl_sync(kFull, first[h], q);
+                    if (r < K[h]) {
+                        w[h] = 64 * q + nth_set_bit(d, r - f);
+                        x[h] = (uint64_t)__ldcg((const unsigned long long *)p.nxt + (size_t)v[h] * B + w[h]);
+                    }
+                }
+                int at = off + r;
+#pragma unroll
+                for (int h = 0; h < NN; ++h) {
+                    if (w[h] >= 0) {
+                        p.nxt[(size_t)v[h] * B + w[h]] = 0ull;
+                        p.out.pw[at] = (uint16_t)w[h];
+                        p.out.pb[at] = x[h];
+                        pc += __popcll(x[h]);
+                    }
+                    at += K[h];
+                }
+            }
+        }
 #pragma unroll
         for (int h = 0; h < NN; ++h) {
             if (K[h] == 0) continue;
@@ -793,6 +847,10 @@ __global__ void __launch_bounds__(kBlock) k_collect_wide(Params p_) {
             for (int c = lane; c < nch; c += 32) p.out.work[item0 + c] = make_int2(slot, c * ne);
             item0 += nch;
             ++slot;
+            if (few) {
+                off += K[h];
+                continue;
+            }
             uint64_t *row = p.nxt + (size_t)v[h] * B;
             for (int q = 0; q < nq; q += 2) {  // 128 words: two mask words, four 32-word groups
                 const uint64_t d0 = __shfl_sync(kFull, dm[h], q);
@@ -820,6 +878,23 @@ __global__ void __launch_bounds__(kBlock) k_collect_wide(Params p_) {
         }
     }
     add_level_count(p, pc);
+    // out-edges and checks of the slots: one addition a block (every warp's met at one address otherwise)
+    __shared__ unsigned long long s_checks[kWarps];
+    __shared__ int s_edges[kWarps];
+    if (lane == 0) {
+        s_checks[threadIdx.x >> 5] = checks;
+        s_edges[threadIdx.x >> 5] = edges;
+    }
+    __syncthreads();
+    if (threadIdx.x != 0) return;
+    for (int i = 1; i < kWarps; ++i) {
+        checks += s_checks[i];
+        edges += s_edges[i];
+    }
+    if (edges) {
+        atomicAdd(&p.out.cnt[3], edges);
+        atomicAdd((unsigned long long *)(p.out.cnt + 4), checks);
+    }
 }
 
 // ---------------------------------------------------------------- LT counting form

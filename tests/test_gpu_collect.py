@@ -42,3 +42,20 @@ def test_full_counters(n, words):
     T = 64 * words - 1
     a = P.cnd_ic_simulate_ex(G, np.zeros(1, np.int32), T, 3, edge_checks=True)
     assert (a.spread == n).all() and (a.node_count == T).all() and a.edge_checks == T * (n - 1)
+
+
+@pytest.mark.parametrize("model", ["ic", "lt"])
+@pytest.mark.parametrize("words", [257, 700, 2047])
+def test_wide_passes_with_few_words_per_node(model, words):
+    """Many one-word items: a listed node holds anything from one to some hundred words, scattered over the pass."""
+    g = I.erdos_renyi_m(1500, 6000, graph_seed=words)
+    p, w = I.ic_weighted_cascade(g), I.lt_weighted_cascade(g)
+    G = P.cnd_graph_create(g.n, g.row_ptr, g.col, p, w)
+    off, seeds, _, keys = I.batch_items(g.n, words, 1, 12, (1,), graph_seed=words)
+    seeds[off[:-1]] = 7  # and one node that is in every item
+    trials = np.full(words, 37, dtype=np.int32)
+    f = P.cnd_ic_simulate_batch if model == "ic" else P.cnd_lt_simulate_batch
+    a, b = (f(G, off, seeds, trials, keys, node_count=True, edge_checks=True, level_counts_len=30, direction="push",
+              word_bits=64 * wb) for wb in (words, 100))
+    assert np.array_equal(a.spread, b.spread) and np.array_equal(a.node_count, b.node_count)
+    assert a.edge_checks == b.edge_checks and np.array_equal(a.level_counts, b.level_counts)
