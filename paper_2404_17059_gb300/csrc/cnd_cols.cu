@@ -509,18 +509,23 @@ void choose_shape(int model, const cnd_graph_dev &G, int64_t trials, ColShape &c
 // where a pass spreads them over all; a pass takes some 48 us a step, and how many steps there are
 // follows from how fast a cascade grows, G.ic_branching.
 // IC up to a branching of 1.3, where cascades are long or touch little: always (kColMaxEdges; above 0.8 up to
-// 1,000 edges a node).  Elsewhere by both estimated times, in us, the columns' with 0.4 of it on top: fits to
+// 1,000 edges a node).  Always too up to 90,000 edges, and up to kWideTrials * 4 trials without hub rows up to
+// 200,000 edges or with a branching of up to 4.2 up to 260,000: of these, 1 % took over 1.05 times the passes' time,
+// 1.1 at most.  Elsewhere by both estimated times, in us, the columns' with 0.3 of it on top: fits to
 // 1,595 calls of 1 to 20,000 trials (G(n, p), Watts-Strogatz, BA and R-MAT, 12,000 to 3 M edges, U[0, 1], WC and
-// uniform p) that leave 30 % (root mean square).  With the rule before, 443 of them took over 1.08 times the
-// passes' time, up to 8 times: G(5000, p) of 1 M edges, p = 0.05, 64 trials 1.3 against 0.4 ms, R-MAT 14 of 776,000
+// uniform p) that leave 30 % (root mean square).  7 of 1,785 calls are left above 1.08 times the passes' time, at 1.28 at
+// most; with no term for edges it were 443, up to 8 times: G(5000, p) of 1 M edges, p = 0.05, 64 trials 1.3 against 0.4 ms, R-MAT 14 of 776,000
 // edges, p = 0.1, 1,000 trials 2.2 against 0.9 ms, G(20000, p) of 20 M edges, p = 0.1, one trial 13.2 against 0.4 ms.
 // LT: the passes' pull steps count dense rows faster than atomics on shared memory; 1,000 nodes, 20,000 trials,
 // 200 / 400 / 1,000 edges a node: 15.9 against 16.0 / 29.2 against 16.9 / 85 against 31 ms.
+constexpr int64_t kWideTrials = 4096;
+
 bool columns_pay(int model, const cnd_graph_dev &G, int64_t trials, int64_t words) {
     if (model == 1) return G.m <= 200ll * G.n;
     if (G.m > kColMaxEdges) return false;
     const double r = G.ic_branching;
-    if (r <= 0.8 || (r <= 1.3 && G.m <= 1000ll * G.n)) return true;
+    if (r <= 0.8 || (r <= 1.3 && G.m <= 1000ll * G.n) || G.m <= 90000) return true;
+    if (trials <= 4 * kWideTrials && (G.m <= 200000 ? G.max_out_degree < kHub || r <= 4.2 : G.m <= 260000 && r <= 4.2)) return true;
     ColShape c;
     int32_t bits = 0;
     choose_shape(model, G, trials, c, bits);
@@ -533,7 +538,7 @@ bool columns_pay(int model, const cnd_graph_dev &G, int64_t trials, int64_t word
     const double per_edge = (0.35 + 0.8 * (double)std::min<int64_t>(bits, std::max<int64_t>(2, trials)) * onward) * hubs * 1e-3;
     const double t_columns = 90.0 + waves * c.per_sm * (double)G.m * per_edge;
     const double t_passes = 160.0 + 48.0 * steps + 3.8e-4 * (double)G.m * (double)words * onward;
-    return 1.4 * t_columns < t_passes;
+    return 1.3 * t_columns < t_passes;
 }
 
 }  // namespace
@@ -552,8 +557,6 @@ bool columns_pay(int model, const cnd_graph_dev &G, int64_t trials, int64_t word
 //   no hub rows:   G(20000, 200000) p = 0.1 10,000 trials 8.6 -> 2.5 ms; U[0, 1] 10,000 / 30,000 / 65,536 trials
 //                  3.54 -> 3.55 / 8.4 -> 9.5 / 18.7 -> 19.0 ms
 //   LT, any:       BA 5k 1,000 trials 2,395 -> 370 us, 65,536 trials 20.1 -> 8.1 ms
-constexpr int64_t kWideTrials = 4096;
-
 bool columns_fit(int model, const cnd_graph_dev &G, const cnd_sim_opts &o, int64_t trials, int64_t words) {
     if (model == 1 && (!G.lt_cnt_edge || o.lt_accumulate)) return false;
     if (o.word_bits || o.chunk_edges || o.direction != CND_DIR_AUTO || o.pull_permille || o.defer_bits || o.stats)
@@ -562,6 +565,13 @@ bool columns_fit(int model, const cnd_graph_dev &G, const cnd_sim_opts &o, int64
     if (!column_shape(model, G, 1, c) || !columns_pay(model, G, trials, words)) return false;
     if (model == 1 || trials <= kWideTrials || column_shape(model, G, 4, c)) return true;
     return G.max_out_degree < kHub && (trials <= 4 * kWideTrials || column_shape(model, G, 2, c));
+}
+
+int32_t column_bits(int model, const cnd_graph_dev &G, int64_t trials) {
+    ColShape c;
+    int32_t bits = 0;
+    choose_shape(model, G, trials, c, bits);
+    return bits;
 }
 
 cnd_status plan_columns(int model, const cnd_graph_dev &G, const std::vector<ItemDesc> &items, ColPlan &plan) {

@@ -34,6 +34,9 @@ struct ColPlan {
 // True if a call of `trials` trials in all, in `words` words of 64 of the same item, runs in the column engine.
 bool columns_fit(int model, const cnd_graph_dev &G, const cnd_sim_opts &o, int64_t trials, int64_t words);
 
+// The trials of a column of such a call.
+int32_t column_bits(int model, const cnd_graph_dev &G, int64_t trials);
+
 cnd_status plan_columns(int model, const cnd_graph_dev &G, const std::vector<ItemDesc> &items, ColPlan &plan);
 
 // Runs the items' trials.  items: plan.items on the device; scratch: plan.scratch bytes, 16-byte aligned.

@@ -3245,19 +3245,12 @@ cnd_status cnd_sim_plan(const cnd_graph *g, int32_t model, int32_t n_items, int6
         return CND_EINVAL;
     }
     const cnd_graph_dev &G = g->d;
-    std::vector<ItemDesc> items((size_t)n_items);
-    int64_t words = 0;
-    for (int32_t i = 0; i < n_items; ++i) {
-        items[i].trials = n_trials / n_items + (i < n_trials % n_items ? 1 : 0);
-        words += (items[i].trials + 63) / 64;
-    }
+    const int64_t each = n_trials / n_items, more = n_trials % n_items;  // `more` items have one trial more
+    const int64_t words = more * ((each + 64) / 64) + (n_items - more) * ((each + 63) / 64);
     int32_t engine = CND_ENGINE_PASSES, bits = 0;
     if (words > 0 && columns_fit(model, G, o, n_trials, words)) {
-        ColPlan plan;
-        const cnd_status st = plan_columns(model, G, items, plan);
-        if (st != CND_OK) return st;
         engine = CND_ENGINE_COLUMNS;
-        bits = plan.bits;
+        bits = column_bits(model, G, n_trials);
     } else if (words > 0) {
         size_t free_b = (size_t)free_bytes, total_b = 0;
         if (free_bytes == 0) {

@@ -186,6 +186,7 @@ def test_engine_of_a_call(model):
             for kw in ({"graph": 1}, {"max_levels": 3}, {"first_trial": 64}, {"n_items": 7}):
                 assert P.cnd_sim_plan(G, model, 100, **kw)[0] == "columns"
             assert P.cnd_sim_plan(G, model, 0) == ("passes", 0)
+            assert P.cnd_sim_plan(G, model, 2**31 - 1, n_items=2**31 - 1)[1] > 0  # no list of the items is made
             with pytest.raises(P.CndError):
                 P.cnd_sim_plan(G, model, 100, word_bits=65)
     assert all(engine[n] == "columns" for n in (1, 33, 6000)) and engine[30_000] == "passes"
