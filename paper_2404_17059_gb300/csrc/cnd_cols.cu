@@ -514,8 +514,9 @@ void choose_shape(int model, const cnd_graph_dev &G, int64_t trials, ColShape &c
 // 1.1 at most.  Elsewhere by both estimated times, in us, the columns' with 0.3 of it on top: fits to
 // 1,595 calls of 1 to 20,000 trials (G(n, p), Watts-Strogatz, BA and R-MAT, 12,000 to 3 M edges, U[0, 1], WC and
 // uniform p) that leave 30 % (root mean square).  7 of 1,785 calls are left above 1.08 times the passes' time, at 1.28 at
-// most; with no term for edges 443 are, up to 8 times: G(5000, p) of 1 M edges, p = 0.05, 64 trials 1.3 against 0.4 ms, R-MAT 14 of 776,000
-// edges, p = 0.1, 1,000 trials 2.2 against 0.9 ms, G(20000, p) of 20 M edges, p = 0.1, one trial 13.2 against 0.4 ms.
+// most; with no term for edges 443 are, up to 8 times: G(5000, p) of 1 M edges, p = 0.05, 64 trials 1.3 against 0.4
+// ms, R-MAT 14 of 776,000 edges, p = 0.1, 1,000 trials 2.2 against 0.9 ms, G(20000, p) of 20 M edges, p = 0.1, one
+// trial 13.2 against 0.4 ms.
 // LT: the passes' pull steps count dense rows faster than atomics on shared memory; 1,000 nodes, 20,000 trials,
 // 200 / 400 / 1,000 edges a node: 15.9 against 16.0 / 29.2 against 16.9 / 85 against 31 ms.
 constexpr int64_t kWideTrials = 4096;
@@ -525,7 +526,8 @@ bool columns_pay(int model, const cnd_graph_dev &G, int64_t trials, int64_t word
     if (G.m > kColMaxEdges) return false;
     const double r = G.ic_branching;
     if (r <= 0.8 || (r <= 1.3 && G.m <= 1000ll * G.n) || G.m <= 90000) return true;
-    if (trials <= 4 * kWideTrials && (G.m <= 200000 ? G.max_out_degree < kHub || r <= 4.2 : G.m <= 260000 && r <= 4.2)) return true;
+    if (trials <= 4 * kWideTrials && ((G.m <= 200000 && G.max_out_degree < kHub) || (G.m <= 260000 && r <= 4.2)))
+        return true;
     ColShape c;
     int32_t bits = 0;
     choose_shape(model, G, trials, c, bits);

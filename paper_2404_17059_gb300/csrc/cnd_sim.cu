@@ -1921,10 +1921,12 @@ __global__ void k_ctl(Params p, Loops loops, int32_t at, int32_t max_levels, int
     if (go && may_pull && next == loops.n - 1) c->pull_bodies += 1ull;
     // conditions keep their values: only what changes is set (1 us each)
     if (at < 0) {
-        for (int i = 0; i < loops.n; ++i) cudaGraphSetConditional(loops.h[i], go && i == next ? 1u : 0u);
+        cudaGraphSetConditional(loops.h[0], go && next == 0 ? 1u : 0u);
+        if (loops.n == 2) cudaGraphSetConditional(loops.h[1], go && next == 1 ? 1u : 0u);
     } else if (!go || next != at) {
-        cudaGraphSetConditional(loops.h[at], 0u);
-        if (go) cudaGraphSetConditional(loops.h[next], 1u);
+        if (at == 0) cudaGraphSetConditional(loops.h[0], 0u);
+        else cudaGraphSetConditional(loops.h[1], 0u);
+        if (go) cudaGraphSetConditional(loops.h[1], 1u);  // from the first loop into the second
     }
 }
 
