@@ -10,7 +10,7 @@ pytestmark = pytest.mark.gpu
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
 
-@pytest.mark.parametrize("workload,engine", [("er1k", "columns"), ("rmat24 --scale 14", "passes")])
+@pytest.mark.parametrize("workload,engine", [("er1k", "columns"), ("rmat24 --scale 15", "passes")])
 def test_timed_steps_run_in_the_engine_of_the_default_call(workload, engine):
     out = subprocess.run([sys.executable, "bench.py", "--workload", *workload.split(), "--steps", "3", "--warmup", "3",
                           "--no-cpu-baseline"], cwd=ROOT, capture_output=True, text=True, timeout=600)
